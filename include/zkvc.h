@@ -81,9 +81,9 @@ int zkvc_profile_span(int stage, double* start_ms, double* end_ms);
  * 2: sixteen independent mad.hi.u32 chains; 3: eight independent mad.wide.u32 chains
  * (64-bit accumulators); 4: two carry chains of eight mad.lo; 5 to 8: two independent
  * chains of whole Fp Montgomery products per thread (264 IMADs each): 5 CIOS with
- * carry-chain rows, 6 CIOS with 64-bit accumulators, 7 product scanning with 96-bit
- * column accumulators in mad.lo.cc / madc.hi.cc (the product the kernels use), 8 the same
- * with mul.wide and additions; 9 and 10: latency, one warp running one dependent chain
+ * carry-chain rows, 6 CIOS with 64-bit accumulators, 7 operand scanning with even and odd
+ * accumulators (the product the kernels use), 8 product scanning with mul.wide and
+ * additions; 9 and 10: latency, one warp running one dependent chain
  * of products per thread (9: the kernels' product, 10: the 64-bit-accumulator CIOS); each
  * checked against the CIOS product on every thread (ZKVC_ECUDA if any result differs).  A full-occupancy grid over every SM runs `iters` iterations (16 IMADs per
  * thread for forms 0 .. 4), once untimed (iters / 8) and once timed with CUDA events on

@@ -355,9 +355,10 @@ template size_t msm_api_ws<Fp>(size_t);
 //   2  sixteen independent mad.hi.u32 chains
 //   3  eight independent mad.wide.u32 chains (64-bit accumulators; two IMADs each)
 //   4  two carry chains of eight mad.lo.cc / madc.lo.cc
-//   5  whole Fp Montgomery products, the inlined carry-chain CIOS (f_mul): two independent
-//      product chains per thread, 264 IMADs per product
-//   6  the same with the out-of-line 64-bit-accumulator CIOS of the point formulas (f_mulc)
+//   5  whole Fp Montgomery products, the inlined carry-chain CIOS: two independent product
+//      chains per thread, 264 IMADs per product
+//   6  the same with the out-of-line 64-bit-accumulator CIOS
+//   7  the same with the kernels' product (f_mul, even and odd accumulators)
 // A full-occupancy grid of 256-thread blocks covers all SMs.  The result xor goes to
 // `sink` so that nothing is dead code.
 template <int FORM>
@@ -435,24 +436,15 @@ __global__ void __launch_bounds__(256) k_imad_rate(uint32_t iters, uint32_t seed
 
 // Product-scanning Montgomery multiplication (finely integrated: every column sums its
 // a_j b_(i-j) and m_j p_(i-j) terms into a 96-bit accumulator, and the low word of column
-// i < 8 yields m_i), written out for the throughput comparison of zkvc_imad_rate: WIDE = 0
-// accumulates with mad.lo.cc / madc.hi.cc / addc (the field code's f_mul), WIDE = 1 (form
-// 8) with one 64-bit product (mul.wide) and three additions.
-template <int WIDE>
+// i < 8 yields m_i), written out for the throughput comparison of zkvc_imad_rate (form 8):
+// one 64-bit product (mul.wide) and three additions per term.
 __device__ __forceinline__ void col_acc(uint32_t& t0, uint32_t& t1, uint32_t& t2, uint32_t x, uint32_t y) {
-  if constexpr (WIDE) {
-    const uint64_t p = (uint64_t)x * y;
-    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
-        : "+r"(t0), "+r"(t1), "+r"(t2)
-        : "r"((uint32_t)p), "r"((uint32_t)(p >> 32)));
-  } else {
-    asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\tmadc.hi.cc.u32 %1, %3, %4, %1;\n\taddc.u32 %2, %2, 0;"
-        : "+r"(t0), "+r"(t1), "+r"(t2)
-        : "r"(x), "r"(y));
-  }
+  const uint64_t p = (uint64_t)x * y;
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+      : "+r"(t0), "+r"(t1), "+r"(t2)
+      : "r"((uint32_t)p), "r"((uint32_t)(p >> 32)));
 }
 
-template <int WIDE>
 __device__ __forceinline__ Fp f_mul_fips(const Fp& a, const Fp& b) {
   uint32_t m[8], r[8];
   uint32_t t0 = 0, t1 = 0, t2 = 0;
@@ -460,12 +452,12 @@ __device__ __forceinline__ Fp f_mul_fips(const Fp& a, const Fp& b) {
   for (int i = 0; i < 8; i++) {
 #pragma unroll
     for (int j = 0; j < i; j++) {
-      col_acc<WIDE>(t0, t1, t2, a.v[j], b.v[i - j]);
-      col_acc<WIDE>(t0, t1, t2, m[j], mod_limb<FpCfg>(i - j));
+      col_acc(t0, t1, t2, a.v[j], b.v[i - j]);
+      col_acc(t0, t1, t2, m[j], mod_limb<FpCfg>(i - j));
     }
-    col_acc<WIDE>(t0, t1, t2, a.v[i], b.v[0]);
+    col_acc(t0, t1, t2, a.v[i], b.v[0]);
     m[i] = t0 * FpCfg::INV;
-    col_acc<WIDE>(t0, t1, t2, m[i], mod_limb<FpCfg>(0));
+    col_acc(t0, t1, t2, m[i], mod_limb<FpCfg>(0));
     t0 = t1;
     t1 = t2;
     t2 = 0;
@@ -474,8 +466,8 @@ __device__ __forceinline__ Fp f_mul_fips(const Fp& a, const Fp& b) {
   for (int i = 8; i < 15; i++) {
 #pragma unroll
     for (int j = i - 7; j < 8; j++) {
-      col_acc<WIDE>(t0, t1, t2, a.v[j], b.v[i - j]);
-      col_acc<WIDE>(t0, t1, t2, m[j], mod_limb<FpCfg>(i - j));
+      col_acc(t0, t1, t2, a.v[j], b.v[i - j]);
+      col_acc(t0, t1, t2, m[j], mod_limb<FpCfg>(i - j));
     }
     r[i - 8] = t0;
     t0 = t1;
@@ -509,8 +501,8 @@ __global__ void __launch_bounds__(256) k_mont_rate(uint32_t iters, uint32_t seed
       a = f_mul(a, m);
       b = f_mul(b, m);
     } else if constexpr (FORM == 8) {
-      a = f_mul_fips<1>(a, m);
-      b = f_mul_fips<1>(b, m);
+      a = f_mul_fips(a, m);
+      b = f_mul_fips(b, m);
     } else if constexpr (FORM == 9) {  // latency: one dependent chain
       a = f_mul(a, m);
     } else {
@@ -522,7 +514,7 @@ __global__ void __launch_bounds__(256) k_mont_rate(uint32_t iters, uint32_t seed
   if constexpr (FORM == 5) got = f_mul_cios(a, b);
   else if constexpr (FORM == 6 || FORM == 10) got = f_mulc_cios(a, b);
   else if constexpr (FORM == 7 || FORM == 9) got = f_mul(a, b);
-  else got = f_mul_fips<1>(a, b);
+  else got = f_mul_fips(a, b);
   if (got != f_mul_cios(a, b)) atomicAdd(sink + 1, 1u);
   uint32_t acc = 0;
 #pragma unroll

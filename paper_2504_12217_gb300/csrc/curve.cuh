@@ -35,15 +35,25 @@ using G2A = Affine<Fp2>;
 using G1J = XYZZ<Fp>;
 using G2J = XYZZ<Fp2>;
 
-// Products used by the point formulas: the compact (rolled, out-of-line) Montgomery
-// product.  Smaller code avoids instruction-fetch stalls, which dominate these large
-// formulas on GB300: the bucket-accumulation loop runs at 3.7 G mixed additions/s with
-// compact products against 2.9 G/s fully unrolled, and the chained XYZZ addition takes
-// 10.5 us instead of 12.9 us.
+// Products used by the point formulas: the out-of-line Montgomery products.  Smaller code
+// avoids instruction-fetch stalls, which dominate these large formulas on GB300 when every
+// product is inlined.  f_mul2x(a, b, c, d) = a b + c d shares one reduction; a subtracted
+// product takes f_comp(a) = N - a (in [1, N], which the products accept) as a factor.
 __device__ __forceinline__ Fp f_mulx(const Fp& a, const Fp& b) { return f_mulc(a, b); }
-__device__ __forceinline__ Fp f_sqrx(const Fp& a) { return f_mulc(a, a); }
+__device__ __forceinline__ Fp f_sqrx(const Fp& a) { return f_sqrc(a); }
+__device__ __forceinline__ Fp f_mul2x(const Fp& a, const Fp& b, const Fp& c, const Fp& d) { return f_mul2c(a, b, c, d); }
 __device__ __forceinline__ Fp2 f_mulx(const Fp2& a, const Fp2& b) { return f_mul(a, b); }
 __device__ __forceinline__ Fp2 f_sqrx(const Fp2& a) { return f_sqr(a); }
+__device__ __forceinline__ Fp2 f_mul2x(const Fp2& a, const Fp2& b, const Fp2& c, const Fp2& d) {
+  return f_mul2(a, b, c, d);
+}
+__device__ __forceinline__ Fp f_comp(const Fp& a) {
+  Fp r;
+  const Fp m = Fp::modulus();
+  sub8(r.v, m.v, a.v);
+  return r;
+}
+__device__ __forceinline__ Fp2 f_comp(const Fp2& a) { return {f_comp(a.c0), f_comp(a.c1)}; }
 
 template <class F>
 __device__ __forceinline__ Affine<F> p_neg(const Affine<F>& a) {
@@ -68,7 +78,7 @@ __device__ __forceinline__ XYZZ<F> p_dbl_body(const XYZZ<F>& p) {
   F X2 = f_sqrx(p.X);
   F M = f_add(f_dbl(X2), X2);
   F X3 = f_sub(f_sqrx(M), f_dbl(S));
-  F Y3 = f_sub(f_mulx(M, f_sub(S, X3)), f_mulx(W, p.Y));
+  F Y3 = f_mul2x(M, f_sub(S, X3), f_comp(W), p.Y);
   return {X3, Y3, f_mulx(V, p.ZZ), f_mulx(W, p.ZZZ)};
 }
 
@@ -77,13 +87,13 @@ template <class F>
 __device__ __forceinline__ XYZZ<F> p_dbl_affine(const Affine<F>& a) {
   if (a.is_inf() || a.y.is_zero()) return XYZZ<F>::inf();
   F U = f_dbl(a.y);
-  F V = f_sqr(U);
-  F W = f_mul(U, V);
-  F S = f_mul(a.x, V);
-  F X2 = f_sqr(a.x);
+  F V = f_sqrx(U);
+  F W = f_mulx(U, V);
+  F S = f_mulx(a.x, V);
+  F X2 = f_sqrx(a.x);
   F M = f_add(f_dbl(X2), X2);
-  F X3 = f_sub(f_sqr(M), f_dbl(S));
-  F Y3 = f_sub(f_mul(M, f_sub(S, X3)), f_mul(W, a.y));
+  F X3 = f_sub(f_sqrx(M), f_dbl(S));
+  F Y3 = f_mul2x(M, f_sub(S, X3), f_comp(W), a.y);
   return {X3, Y3, V, W};
 }
 
@@ -104,7 +114,7 @@ __device__ __forceinline__ XYZZ<F> p_add_affine_body(const XYZZ<F>& p, const Aff
   F PPP = f_mulx(P, PP);
   F Q = f_mulx(p.X, PP);
   F X3 = f_sub(f_sub(f_sqrx(R), PPP), f_dbl(Q));
-  F Y3 = f_sub(f_mulx(R, f_sub(Q, X3)), f_mulx(p.Y, PPP));
+  F Y3 = f_mul2x(R, f_sub(Q, X3), f_comp(p.Y), PPP);
   return {X3, Y3, f_mulx(p.ZZ, PP), f_mulx(p.ZZZ, PPP)};
 }
 
@@ -127,7 +137,7 @@ __device__ __forceinline__ XYZZ<F> p_add_body(const XYZZ<F>& p, const XYZZ<F>& q
   F PPP = f_mulx(P, PP);
   F Q = f_mulx(U1, PP);
   F X3 = f_sub(f_sub(f_sqrx(R), PPP), f_dbl(Q));
-  F Y3 = f_sub(f_mulx(R, f_sub(Q, X3)), f_mulx(S1, PPP));
+  F Y3 = f_mul2x(R, f_sub(Q, X3), f_comp(S1), PPP);
   return {X3, Y3, f_mulx(f_mulx(p.ZZ, q.ZZ), PP), f_mulx(f_mulx(p.ZZZ, q.ZZZ), PPP)};
 }
 

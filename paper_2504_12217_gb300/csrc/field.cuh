@@ -4,12 +4,10 @@
 // field Fr (witness, QAP polynomials, NTT) and the base field Fp (curve coordinates).
 // Both moduli are below 2^254, which the bounds below rely on.
 //
-// Multiplication is CIOS Montgomery (coarsely integrated operand scanning): for each
-// limb b_i of the multiplier the row t += a * b_i is two carry chains of mad.lo / mad.hi
-// (PTX mad.lo.cc / madc.hi.cc, one IMAD each), then m = t_0 * (-N^-1 mod 2^32) and
-// t = (t + m N) / 2^32 the same way.  With a, b < N < 2^254 every intermediate stays
-// below 2^288, so a 9-word accumulator never carries out and the result is < 2N before
-// the single conditional subtraction.  Cost: 4 * 8 * 8 + 8 = 264 IMADs per product.
+// Multiplication is Montgomery's by operand scanning: for each limb b_i of the multiplier
+// t += a b_i, then m = t_0 (-N^-1 mod 2^32) and t = (t + m N) / 2^32, with the terms split
+// by parity over two accumulators (below).  Cost: 2 * 8 * 8 wide multiply-adds and 8 low
+// products, counted as 4 * 8 * 8 + 8 = 264 IMADs per product.
 #pragma once
 #include <cstdint>
 
@@ -233,7 +231,7 @@ template <class C>
 __device__ __forceinline__ Field<C> f_dbl(const Field<C>& a) { return f_add(a, a); }
 
 // Montgomery product a b R^-1 mod N, CIOS with carry-chain rows (reference form; the
-// product-scanning f_mul below is the one the kernels use).
+// even/odd f_mul below is the one the kernels use).
 template <class C>
 __device__ __forceinline__ Field<C> f_mul_cios(const Field<C>& a, const Field<C>& b) {
   uint32_t t[9];
@@ -258,68 +256,395 @@ __device__ __forceinline__ Field<C> f_mul_cios(const Field<C>& a, const Field<C>
   return br ? r : d;
 }
 
-// One term x y of a product-scanning column: (t2, t1, t0) += x y as mad.lo.cc /
-// madc.hi.cc / addc.
-__device__ __forceinline__ void col_mac(uint32_t& t0, uint32_t& t1, uint32_t& t2, uint32_t x, uint32_t y) {
-  asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\tmadc.hi.cc.u32 %1, %3, %4, %1;\n\taddc.u32 %2, %2, 0;"
-      : "+r"(t0), "+r"(t1), "+r"(t2)
-      : "r"(x), "r"(y));
+// ------------------------------------------------------------------ even/odd products
+// The kernels' products keep a number as two accumulators: e holds the limbs of the terms
+// x_i y_j with i + j even and o those with i + j odd (o[k] weighs 2^(32 (k + 1))).  The
+// terms x_s y, x_(s+2) y, x_(s+4) y, x_(s+6) y of one row then land on neighbouring aligned
+// limb pairs of one accumulator, so a row is two carry chains of four 32 x 32 + 64 -> 64-bit
+// multiply-adds each (mad.lo.cc / madc.hi.cc on a register pair) with the carry handed on
+// inside the chain: one multiply-add instruction per term, against one multiply-add and one
+// carry addition in product scanning.  The row-by-row form follows Koc, Acar and Kaliski's
+// operand scanning (1996); the split by parity keeps its carries off the critical pairs.
+//
+// What bounds it: the multiplier's 32 wide multiply-adds per SM and clock; a product has
+// 128 of them and 8 low products, 132 clocks per warp and SM.  Measured on GB300 (2,070
+// MHz, 32 warps per SM): 147 clocks = 68.4 G products/s (product scanning before: 159,
+// 63.2 G); one warp alone 900 cycles per product (1,141); f_sqr 125 clocks, 80.6 G;
+// f_mul2 217 clocks, 46.4 G (two products and an addition before: 323); Fp2 product 387
+// clocks, 26.0 G (546); Fp2 square 301 (358).
+#define ZKVC_CHAIN_3                                                          \
+  "mad.lo.cc.u32  %0, %8,  %12, %0;\n\tmadc.hi.cc.u32 %1, %8,  %12, %1;\n\t"   \
+  "madc.lo.cc.u32 %2, %9,  %12, %2;\n\tmadc.hi.cc.u32 %3, %9,  %12, %3;\n\t"   \
+  "madc.lo.cc.u32 %4, %10, %12, %4;\n\tmadc.hi.cc.u32 %5, %10, %12, %5;\n\t"
+#define ZKVC_CHAIN_4C                                                         \
+  "mad.lo.cc.u32  %0, %9,  %13, %0;\n\tmadc.hi.cc.u32 %1, %9,  %13, %1;\n\t"   \
+  "madc.lo.cc.u32 %2, %10, %13, %2;\n\tmadc.hi.cc.u32 %3, %10, %13, %3;\n\t"   \
+  "madc.lo.cc.u32 %4, %11, %13, %4;\n\tmadc.hi.cc.u32 %5, %11, %13, %5;\n\t"   \
+  "madc.lo.cc.u32 %6, %12, %13, %6;\n\tmadc.hi.cc.u32 %7, %12, %13, %7;\n\t"
+#define ZKVC_CHAIN_X(x, s, y) "r"(x[s]), "r"(x[s + 2]), "r"(x[s + 4]), "r"(x[s + 6]), "r"(y)
+
+namespace eo {
+// t[0..7] += (x_s, x_(s+2), x_(s+4), x_(s+6)) y; the caller's bound leaves no carry out
+__device__ __forceinline__ void chain(uint32_t* t, const uint32_t* x, int s, uint32_t y) {
+  asm(ZKVC_CHAIN_3 "madc.lo.cc.u32 %6, %11, %12, %6;\n\tmadc.hi.u32 %7, %11, %12, %7;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7])
+      : ZKVC_CHAIN_X(x, s, y));
+}
+// the same with t[7] fresh (zero before)
+__device__ __forceinline__ void chain_f1(uint32_t* t, const uint32_t* x, int s, uint32_t y) {
+  asm(ZKVC_CHAIN_3 "madc.lo.cc.u32 %6, %11, %12, %6;\n\tmadc.hi.u32 %7, %11, %12, 0;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "=r"(t[7])
+      : ZKVC_CHAIN_X(x, s, y));
+}
+// t[6] and t[7] fresh
+__device__ __forceinline__ void chain_f2(uint32_t* t, const uint32_t* x, int s, uint32_t y) {
+  asm(ZKVC_CHAIN_3 "madc.lo.cc.u32 %6, %11, %12, 0;\n\tmadc.hi.u32 %7, %11, %12, 0;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "=r"(t[6]), "=r"(t[7])
+      : ZKVC_CHAIN_X(x, s, y));
+}
+// the carry out is added to top
+__device__ __forceinline__ void chain_c(uint32_t* t, uint32_t& top, const uint32_t* x, int s, uint32_t y) {
+  asm(ZKVC_CHAIN_4C "addc.u32 %8, %8, 0;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(top)
+      : ZKVC_CHAIN_X(x, s, y));
+}
+// the carry out becomes top
+__device__ __forceinline__ void chain_cf(uint32_t* t, uint32_t& top, const uint32_t* x, int s, uint32_t y) {
+  asm(ZKVC_CHAIN_4C "addc.u32 %8, 0, 0;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "=r"(top)
+      : ZKVC_CHAIN_X(x, s, y));
+}
+// w += pend with its carry into t, then chain_f2
+__device__ __forceinline__ void chain_p2(uint32_t& w, uint32_t pend, uint32_t* t, const uint32_t* x, int s,
+                                         uint32_t y) {
+  asm("add.cc.u32 %8, %8, %14;\n\t"
+      "madc.lo.cc.u32 %0, %9,  %13, %0;\n\tmadc.hi.cc.u32 %1, %9,  %13, %1;\n\t"
+      "madc.lo.cc.u32 %2, %10, %13, %2;\n\tmadc.hi.cc.u32 %3, %10, %13, %3;\n\t"
+      "madc.lo.cc.u32 %4, %11, %13, %4;\n\tmadc.hi.cc.u32 %5, %11, %13, %5;\n\t"
+      "madc.lo.cc.u32 %6, %12, %13, 0;\n\tmadc.hi.u32 %7, %12, %13, 0;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "=r"(t[6]), "=r"(t[7]), "+r"(w)
+      : ZKVC_CHAIN_X(x, s, y), "r"(pend));
+}
+// t[0..7] = (x_s, x_(s+2), x_(s+4), x_(s+6)) y
+__device__ __forceinline__ void mul4(uint32_t* t, const uint32_t* x, int s, uint32_t y) {
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    const uint64_t p = (uint64_t)x[s + 2 * j] * y;
+    t[2 * j] = (uint32_t)p;
+    t[2 * j + 1] = (uint32_t)(p >> 32);
+  }
+}
+// Short chains of a square's rows: N products x0 y, x1 y, .. into t[0 .. 2N - 1].  MODE 0:
+// the carry out becomes t[2N]; 1: t[2N - 1] is fresh; 2: the last two limbs are fresh.
+template <int N, int MODE>
+__device__ __forceinline__ void chain_s(uint32_t* t, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t y) {
+  if constexpr (N == 3 && MODE == 0)
+    asm("mad.lo.cc.u32  %0, %7, %10, %0;\n\tmadc.hi.cc.u32 %1, %7, %10, %1;\n\t"
+        "madc.lo.cc.u32 %2, %8, %10, %2;\n\tmadc.hi.cc.u32 %3, %8, %10, %3;\n\t"
+        "madc.lo.cc.u32 %4, %9, %10, %4;\n\tmadc.hi.cc.u32 %5, %9, %10, %5;\n\taddc.u32 %6, 0, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "=r"(t[6])
+        : "r"(x0), "r"(x1), "r"(x2), "r"(y));
+  else if constexpr (N == 3 && MODE == 1)
+    asm("mad.lo.cc.u32  %0, %6, %9, %0;\n\tmadc.hi.cc.u32 %1, %6, %9, %1;\n\t"
+        "madc.lo.cc.u32 %2, %7, %9, %2;\n\tmadc.hi.cc.u32 %3, %7, %9, %3;\n\t"
+        "madc.lo.cc.u32 %4, %8, %9, %4;\n\tmadc.hi.u32 %5, %8, %9, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "=r"(t[5])
+        : "r"(x0), "r"(x1), "r"(x2), "r"(y));
+  else if constexpr (N == 3)
+    asm("mad.lo.cc.u32  %0, %6, %9, %0;\n\tmadc.hi.cc.u32 %1, %6, %9, %1;\n\t"
+        "madc.lo.cc.u32 %2, %7, %9, %2;\n\tmadc.hi.cc.u32 %3, %7, %9, %3;\n\t"
+        "madc.lo.cc.u32 %4, %8, %9, 0;\n\tmadc.hi.u32 %5, %8, %9, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "=r"(t[4]), "=r"(t[5])
+        : "r"(x0), "r"(x1), "r"(x2), "r"(y));
+  else if constexpr (N == 2 && MODE == 0)
+    asm("mad.lo.cc.u32  %0, %5, %7, %0;\n\tmadc.hi.cc.u32 %1, %5, %7, %1;\n\t"
+        "madc.lo.cc.u32 %2, %6, %7, %2;\n\tmadc.hi.cc.u32 %3, %6, %7, %3;\n\taddc.u32 %4, 0, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "=r"(t[4])
+        : "r"(x0), "r"(x1), "r"(y));
+  else if constexpr (N == 2)
+    asm("mad.lo.cc.u32  %0, %4, %6, %0;\n\tmadc.hi.cc.u32 %1, %4, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %6, %2;\n\tmadc.hi.u32 %3, %5, %6, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "=r"(t[3])
+        : "r"(x0), "r"(x1), "r"(y));
+  else if constexpr (MODE == 0)
+    asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\tmadc.hi.cc.u32 %1, %3, %4, %1;\n\taddc.u32 %2, 0, 0;"
+        : "+r"(t[0]), "+r"(t[1]), "=r"(t[2])
+        : "r"(x0), "r"(y));
+  else
+    asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, 0;" : "+r"(t[0]), "=r"(t[1]) : "r"(x0), "r"(y));
 }
 
-// Montgomery product a b R^-1 mod N by finely integrated product scanning (Koc, Acar and
-// Kaliski, "Analyzing and comparing Montgomery multiplication algorithms", 1996): column
-// i of the 16-word result sums every a_j b_(i-j) and m_j N_(i-j) into a 96-bit
-// accumulator; for i < 8 its low word then fixes m_i = t_0 (-N^-1) mod 2^32 and m_i N_0
-// clears it; the columns 8 .. 15 are the result.  A column holds at most 16 products
-// below 2^64 plus the carry of the previous one, so 96 bits never overflow; with a, b < N
-// the result is below 2N and one conditional subtraction makes it canonical.  Same IMAD
-// count as CIOS (264); on GB300 it runs at 18.1 T IMAD-equivalents/s in a throughput
-// loop against 12.3-12.6 T/s for the CIOS forms (zkvc_imad_rate forms 5-7): its
-// independent low/high word pairs and short carries issue better than CIOS's long
-// carry chains.
+// One reduction row: q = e_0 (-N^-1) mod 2^32 and (e, o) += q N, which clears e_0.
 template <class C>
-__device__ __forceinline__ Field<C> f_mul(const Field<C>& a, const Field<C>& b) {
-  uint32_t m[8];
-  Field<C> r, d;
-  uint32_t t0 = 0, t1 = 0, t2 = 0;
+__device__ __forceinline__ void red_row(uint32_t* e, uint32_t* o) {
+  uint32_t n[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) n[i] = mod_limb<C>(i);
+  const uint32_t q = e[0] * C::INV;
+  chain(o, n, 1, q);
+  chain_c(e, o[7], n, 0, q);
+}
+
+// The division by 2^32 after a row: o becomes the even accumulator, e_2.. the odd one, and
+// e_1 stays pending (added to the new e_0 by the next chain_p2 or by merge).
+__device__ __forceinline__ void shift(uint32_t* e, uint32_t* o, uint32_t* pend) {
+  *pend = e[1];
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const uint32_t up = j < 6 ? e[j + 2] : 0u;
+    e[j] = o[j];
+    o[j] = up;
+  }
+}
+
+// r = e + 2^32 o + pend over eight limbs, for the state after a shift (o_6 = o_7 = 0)
+__device__ __forceinline__ void merge(uint32_t (&r)[8], const uint32_t* e, const uint32_t* o, uint32_t pend) {
+  asm("add.cc.u32  %0, %8,  %16;\n\taddc.cc.u32 %1, %9,  %17;\n\taddc.cc.u32 %2, %10, %18;\n\t"
+      "addc.cc.u32 %3, %11, %19;\n\taddc.cc.u32 %4, %12, %20;\n\taddc.cc.u32 %5, %13, %21;\n\t"
+      "addc.cc.u32 %6, %14, %22;\n\taddc.u32 %7, %15, 0;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(pend), "r"(o[0]),
+        "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]));
+}
+
+// the whole product a b: e[0..15], o[0..14]
+__device__ __forceinline__ void mul_wide(uint32_t* e, uint32_t* o, const uint32_t* a, const uint32_t* b) {
+  mul4(e, a, 0, b[0]);
+  mul4(o, a, 1, b[0]);
+#pragma unroll
+  for (int i = 1; i < 8; i += 2) {
+    if (i == 1)
+      chain_f2(e + 2, a, 1, b[1]);
+    else
+      chain_f1(e + i + 1, a, 1, b[i]);
+    chain_cf(o + i - 1, o[i + 7], a, 0, b[i]);
+    if (i < 7) {
+      chain_cf(e + i + 1, e[i + 9], a, 0, b[i + 1]);
+      chain_f1(o + i + 1, a, 1, b[i + 1]);
+    }
+  }
+}
+
+// the whole square a^2 (a < 2^255): 28 products a_i a_j (i < j) against limbs of 2a, whose
+// row i starts at limb i + 1 without the bit that comes up from a_i, then the 8 diagonals
+__device__ __forceinline__ void sqr_wide(uint32_t* e, uint32_t* o, const uint32_t* a) {
+  uint32_t d[8], s[8];
+#pragma unroll
+  for (int j = 1; j < 8; j++) {
+    d[j] = __funnelshift_l(a[j - 1], a[j], 1);
+    s[j] = a[j] << 1;
+  }
+  const uint32_t x[8] = {s[1], d[2], d[3], d[4], d[5], d[6], d[7], 0};
+  mul4(o, x, 0, a[0]);
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    const uint64_t p = (uint64_t)d[2 + 2 * j] * a[0];
+    e[2 + 2 * j] = (uint32_t)p;
+    e[3 + 2 * j] = (uint32_t)(p >> 32);
+  }
+  chain_s<3, 0>(o + 2, s[2], d[4], d[6], a[1]);
+  chain_s<3, 2>(e + 4, d[3], d[5], d[7], a[1]);
+  chain_s<3, 1>(o + 4, s[3], d[5], d[7], a[2]);
+  chain_s<2, 0>(e + 6, d[4], d[6], 0, a[2]);
+  chain_s<2, 0>(o + 6, s[4], d[6], 0, a[3]);
+  chain_s<2, 1>(e + 8, d[5], d[7], 0, a[3]);
+  chain_s<2, 1>(o + 8, s[5], d[7], 0, a[4]);
+  chain_s<1, 0>(e + 10, d[6], 0, 0, a[4]);
+  chain_s<1, 0>(o + 10, s[6], 0, 0, a[5]);
+  chain_s<1, 1>(e + 12, d[7], 0, 0, a[5]);
+  chain_s<1, 1>(o + 12, s[7], 0, 0, a[6]);
+  o[14] = 0;
+  asm("mul.lo.u32     %0,  %16, %16;\n\tmul.hi.u32     %1,  %16, %16;\n\t"
+      "mad.lo.cc.u32  %2,  %17, %17, %2;\n\tmadc.hi.cc.u32 %3,  %17, %17, %3;\n\t"
+      "madc.lo.cc.u32 %4,  %18, %18, %4;\n\tmadc.hi.cc.u32 %5,  %18, %18, %5;\n\t"
+      "madc.lo.cc.u32 %6,  %19, %19, %6;\n\tmadc.hi.cc.u32 %7,  %19, %19, %7;\n\t"
+      "madc.lo.cc.u32 %8,  %20, %20, %8;\n\tmadc.hi.cc.u32 %9,  %20, %20, %9;\n\t"
+      "madc.lo.cc.u32 %10, %21, %21, %10;\n\tmadc.hi.cc.u32 %11, %21, %21, %11;\n\t"
+      "madc.lo.cc.u32 %12, %22, %22, %12;\n\tmadc.hi.cc.u32 %13, %22, %22, %13;\n\t"
+      "madc.lo.cc.u32 %14, %23, %23, 0;\n\tmadc.hi.u32 %15, %23, %23, 0;"
+      : "=&r"(e[0]), "=&r"(e[1]), "+&r"(e[2]), "+&r"(e[3]), "+&r"(e[4]), "+&r"(e[5]), "+&r"(e[6]), "+&r"(e[7]),
+        "+&r"(e[8]), "+&r"(e[9]), "+&r"(e[10]), "+&r"(e[11]), "+&r"(e[12]), "+&r"(e[13]), "=&r"(e[14]), "=&r"(e[15])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]));
+}
+
+// t = e + 2^32 o, 16 limbs
+__device__ __forceinline__ void merge_wide(uint32_t* t, const uint32_t* e, const uint32_t* o) {
+  uint32_t c;
+  t[0] = e[0];
+  asm("add.cc.u32  %0, %8,  %15;\n\taddc.cc.u32 %1, %9,  %16;\n\taddc.cc.u32 %2, %10, %17;\n\t"
+      "addc.cc.u32 %3, %11, %18;\n\taddc.cc.u32 %4, %12, %19;\n\taddc.cc.u32 %5, %13, %20;\n\t"
+      "addc.cc.u32 %6, %14, %21;\n\taddc.u32 %7, 0, 0;"
+      : "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7]), "=r"(c)
+      : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+        "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]));
+  asm("add.cc.u32  %8, %8,  0xffffffff;\n\taddc.cc.u32 %0, %9,  %17;\n\taddc.cc.u32 %1, %10, %18;\n\t"
+      "addc.cc.u32 %2, %11, %19;\n\taddc.cc.u32 %3, %12, %20;\n\taddc.cc.u32 %4, %13, %21;\n\t"
+      "addc.cc.u32 %5, %14, %22;\n\taddc.cc.u32 %6, %15, %23;\n\taddc.u32 %7, %16, %24;"
+      : "=&r"(t[8]), "=&r"(t[9]), "=&r"(t[10]), "=&r"(t[11]), "=&r"(t[12]), "=&r"(t[13]), "=&r"(t[14]), "=&r"(t[15]),
+        "+&r"(c)
+      : "r"(e[8]), "r"(e[9]), "r"(e[10]), "r"(e[11]), "r"(e[12]), "r"(e[13]), "r"(e[14]), "r"(e[15]), "r"(o[7]),
+        "r"(o[8]), "r"(o[9]), "r"(o[10]), "r"(o[11]), "r"(o[12]), "r"(o[13]), "r"(o[14]));
+}
+
+// x += y and x -= y over 16 limbs modulo 2^512; w_sub returns 1 if it borrowed
+__device__ __forceinline__ void w_add(uint32_t* x, const uint32_t* y) {
+  uint32_t lo[8], hi[8], a[8], b[8];
 #pragma unroll
   for (int i = 0; i < 8; i++) {
-#pragma unroll
-    for (int j = 0; j < i; j++) {
-      col_mac(t0, t1, t2, a.v[j], b.v[i - j]);
-      col_mac(t0, t1, t2, m[j], mod_limb<C>(i - j));
-    }
-    col_mac(t0, t1, t2, a.v[i], b.v[0]);
-    m[i] = t0 * C::INV;
-    col_mac(t0, t1, t2, m[i], mod_limb<C>(0));  // t0 becomes 0
-    t0 = t1;
-    t1 = t2;
-    t2 = 0;
+    a[i] = x[i];
+    b[i] = y[i];
   }
+  uint32_t c = add8(lo, a, b);
+  asm("add.cc.u32  %8, %8,  0xffffffff;\n\taddc.cc.u32 %0, %9,  %17;\n\taddc.cc.u32 %1, %10, %18;\n\t"
+      "addc.cc.u32 %2, %11, %19;\n\taddc.cc.u32 %3, %12, %20;\n\taddc.cc.u32 %4, %13, %21;\n\t"
+      "addc.cc.u32 %5, %14, %22;\n\taddc.cc.u32 %6, %15, %23;\n\taddc.u32 %7, %16, %24;"
+      : "=&r"(hi[0]), "=&r"(hi[1]), "=&r"(hi[2]), "=&r"(hi[3]), "=&r"(hi[4]), "=&r"(hi[5]), "=&r"(hi[6]),
+        "=&r"(hi[7]), "+&r"(c)
+      : "r"(x[8]), "r"(x[9]), "r"(x[10]), "r"(x[11]), "r"(x[12]), "r"(x[13]), "r"(x[14]), "r"(x[15]), "r"(y[8]),
+        "r"(y[9]), "r"(y[10]), "r"(y[11]), "r"(y[12]), "r"(y[13]), "r"(y[14]), "r"(y[15]));
 #pragma unroll
-  for (int i = 8; i < 15; i++) {
-#pragma unroll
-    for (int j = i - 7; j < 8; j++) {
-      col_mac(t0, t1, t2, a.v[j], b.v[i - j]);
-      col_mac(t0, t1, t2, m[j], mod_limb<C>(i - j));
-    }
-    r.v[i - 8] = t0;
-    t0 = t1;
-    t1 = t2;
-    t2 = 0;
+  for (int i = 0; i < 8; i++) {
+    x[i] = lo[i];
+    x[8 + i] = hi[i];
   }
-  r.v[7] = t0;  // r < 2N < 2^255: no further word
-  const Field<C> mm = Field<C>::modulus();
-  const uint32_t br = sub8(d.v, r.v, mm.v);
+}
+__device__ __forceinline__ uint32_t w_sub(uint32_t* x, const uint32_t* y) {
+  uint32_t lo[8], hi[8], a[8], b[8], c;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    a[i] = x[i];
+    b[i] = y[i];
+  }
+  const uint32_t br = sub8(lo, a, b);
+  asm("sub.cc.u32  %8, 0,   %25;\n\tsubc.cc.u32 %0, %9,  %17;\n\tsubc.cc.u32 %1, %10, %18;\n\t"
+      "subc.cc.u32 %2, %11, %19;\n\tsubc.cc.u32 %3, %12, %20;\n\tsubc.cc.u32 %4, %13, %21;\n\t"
+      "subc.cc.u32 %5, %14, %22;\n\tsubc.cc.u32 %6, %15, %23;\n\tsubc.cc.u32 %7, %16, %24;\n\tsubc.u32 %8, 0, 0;"
+      : "=&r"(hi[0]), "=&r"(hi[1]), "=&r"(hi[2]), "=&r"(hi[3]), "=&r"(hi[4]), "=&r"(hi[5]), "=&r"(hi[6]),
+        "=&r"(hi[7]), "=&r"(c)
+      : "r"(x[8]), "r"(x[9]), "r"(x[10]), "r"(x[11]), "r"(x[12]), "r"(x[13]), "r"(x[14]), "r"(x[15]), "r"(y[8]),
+        "r"(y[9]), "r"(y[10]), "r"(y[11]), "r"(y[12]), "r"(y[13]), "r"(y[14]), "r"(y[15]), "r"(br));
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    x[i] = lo[i];
+    x[8 + i] = hi[i];
+  }
+  return c & 1u;
+}
+}  // namespace eo
+
+// r < 2N brought below N
+template <class C>
+__device__ __forceinline__ Field<C> f_once(const Field<C>& r) {
+  Field<C> d;
+  const Field<C> m = Field<C>::modulus();
+  const uint32_t br = sub8(d.v, r.v, m.v);
   return br ? r : d;
 }
 
+// Montgomery product a b R^-1 mod N for a < 2N and any b < 2^256: after each row the state
+// is below a + N < 2^256 and before the division below 2^288, so nothing leaves limb 8; the
+// result is below a b / R + N < 2N for b < 2N, and for any b where a < N.  (Values that may
+// exceed N come second: f_to_mont reduces an arbitrary 256-bit value.)
 template <class C>
-__device__ __forceinline__ Field<C> f_sqr(const Field<C>& a) { return f_mul(a, a); }
+__device__ __forceinline__ Field<C> f_mul(const Field<C>& a, const Field<C>& b) {
+  uint32_t e[8], o[8], pend;
+  eo::mul4(e, a.v, 0, b.v[0]);
+  eo::mul4(o, a.v, 1, b.v[0]);
+  eo::red_row<C>(e, o);
+  eo::shift(e, o, &pend);
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    eo::chain_p2(e[0], pend, o, a.v, 1, b.v[i]);
+    eo::chain_c(e, o[7], a.v, 0, b.v[i]);
+    eo::red_row<C>(e, o);
+    eo::shift(e, o, &pend);
+  }
+  Field<C> r;
+  eo::merge(r.v, e, o, pend);
+  return f_once(r);
+}
+
+// (a b + c d) R^-1 mod N with one reduction, for operands up to N: the state stays below
+// a + c + N <= 3N < 2^256, the result below 2N^2 / R + N < 2N.
+template <class C>
+__device__ __forceinline__ Field<C> f_mul2(const Field<C>& a, const Field<C>& b, const Field<C>& c,
+                                           const Field<C>& d) {
+  uint32_t e[8], o[8], pend;
+  eo::mul4(e, a.v, 0, b.v[0]);
+  eo::mul4(o, a.v, 1, b.v[0]);
+  eo::chain(o, c.v, 1, d.v[0]);
+  eo::chain_c(e, o[7], c.v, 0, d.v[0]);
+  eo::red_row<C>(e, o);
+  eo::shift(e, o, &pend);
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    eo::chain_p2(e[0], pend, o, a.v, 1, b.v[i]);
+    eo::chain_c(e, o[7], a.v, 0, b.v[i]);
+    eo::chain(o, c.v, 1, d.v[i]);
+    eo::chain_c(e, o[7], c.v, 0, d.v[i]);
+    eo::red_row<C>(e, o);
+    eo::shift(e, o, &pend);
+  }
+  Field<C> r;
+  eo::merge(r.v, e, o, pend);
+  return f_once(r);
+}
+
+// t R^-1 mod N for a 16-limb t < N R given as low limbs e[0..7] + 2^32 o[0..7] (o[7] = 0)
+// and its top half: the low half reduces to at most N + 1, the sum to less than 2N.
+template <class C>
+__device__ __forceinline__ Field<C> f_redc(uint32_t* e, uint32_t* o, const uint32_t (&top)[8]) {
+  uint32_t n[8], pend;
+#pragma unroll
+  for (int i = 0; i < 8; i++) n[i] = mod_limb<C>(i);
+  eo::red_row<C>(e, o);
+  eo::shift(e, o, &pend);
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    const uint32_t q = (e[0] + pend) * C::INV;
+    eo::chain_p2(e[0], pend, o, n, 1, q);
+    eo::chain_c(e, o[7], n, 0, q);
+    eo::shift(e, o, &pend);
+  }
+  Field<C> r;
+  uint32_t lo[8];
+  eo::merge(lo, e, o, pend);
+  add8(r.v, lo, top);
+  return f_once(r);
+}
+
+// the same for t[0..15]
+template <class C>
+__device__ __forceinline__ Field<C> f_redc_wide(const uint32_t* t) {
+  uint32_t e[8], o[8], top[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    e[i] = t[i];
+    o[i] = 0;
+    top[i] = t[8 + i];
+  }
+  return f_redc<C>(e, o, top);
+}
+
+// a^2 R^-1 mod N for a <= N: 36 products and a reduction instead of 64
+template <class C>
+__device__ __forceinline__ Field<C> f_sqr(const Field<C>& a) {
+  uint32_t E[16], O[15], e[8], o[8], x[8], y[8], top[8];
+  eo::sqr_wide(E, O, a.v);
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    e[i] = E[i];
+    o[i] = i < 7 ? O[i] : 0u;
+    x[i] = E[8 + i];
+    y[i] = O[7 + i];
+  }
+  add8(top, x, y);
+  return f_redc<C>(e, o, top);
+}
 
 // Out-of-line Montgomery product with 64-bit accumulation: CIOS rows written with
 // 32 x 32 + 64-bit multiply-adds in plain C (reference form: 12.6 T IMAD-equivalents/s in
-// zkvc_imad_rate form 6, against 18.1 T/s for f_mulc below).
+// zkvc_imad_rate form 6, against 18.1 T/s for product scanning and 19 T/s for f_mulc below).
 template <class C>
 __device__ __noinline__ Field<C> f_mulc_cios(Field<C> a, Field<C> b) {
   uint32_t t[10];
@@ -361,20 +686,28 @@ __device__ __noinline__ Field<C> f_mulc_cios(Field<C> a, Field<C> b) {
   return br ? r : d;
 }
 
-// Out-of-line product-scanning Montgomery product for the point formulas: called, not
-// inlined, so that the large formulas keep one copy of the product's ~400 instructions
-// (fully inlined point formulas stall on instruction fetch).
+// Out-of-line products for the point formulas: called, not inlined, so that the large
+// formulas keep one copy of each (fully inlined point formulas stall on instruction fetch).
 template <class C>
 __device__ __noinline__ Field<C> f_mulc(Field<C> a, Field<C> b) {
   return f_mul(a, b);
 }
+template <class C>
+__device__ __noinline__ Field<C> f_sqrc(Field<C> a) {
+  return f_sqr(a);
+}
+template <class C>
+__device__ __noinline__ Field<C> f_mul2c(Field<C> a, Field<C> b, Field<C> c, Field<C> d) {
+  return f_mul2(a, b, c, d);
+}
 
+// a R mod N for any a < 2^256 (the second operand of f_mul may exceed N)
 template <class C>
 __device__ __forceinline__ Field<C> f_to_mont(const Field<C>& a) {
   Field<C> r2;
 #pragma unroll
   for (int i = 0; i < 8; i++) r2.v[i] = r2_limb<C>(i);
-  return f_mul(a, r2);
+  return f_mul(r2, a);
 }
 
 template <class C>
@@ -699,19 +1032,70 @@ __device__ __forceinline__ Fp2 f_sub(const Fp2& a, const Fp2& b) { return {f_sub
 __device__ __forceinline__ Fp2 f_neg(const Fp2& a) { return {f_neg(a.c0), f_neg(a.c1)}; }
 __device__ __forceinline__ Fp2 f_dbl(const Fp2& a) { return {f_dbl(a.c0), f_dbl(a.c1)}; }
 
-// Karatsuba: (a0 + a1 i)(b0 + b1 i) = (a0 b0 - a1 b1) + ((a0 + a1)(b0 + b1) - a0 b0 - a1 b1) i
-// (out of line, on the compact Fp product: G2 formulas call it ~14 times each)
+// Products of Fp2 with lazy reduction: (a0 + a1 i)(b0 + b1 i) takes the three whole products
+// a0 b0, a1 b1 and (a0 + a1)(b0 + b1) (Karatsuba; the sums stay unreduced, below 2^255),
+// adds and subtracts them at full width and reduces the two coefficients once each: 3 x 64
+// + 2 x 72 multiply-adds instead of 3 x 136 (Aranha, Karabina, Longa, Gebotys and Lopez,
+// "Faster explicit formulas for computing pairings over ordinary curves", 2011).  Operands
+// up to N.  Out of line: G2 formulas call them about ten times each.
+namespace eo {
+// re = Re(a b), im = Im(a b) at full width: im < 2 N^2; re modulo 2^512, returning 1 if
+// negative
+__device__ __forceinline__ uint32_t mul2_wide(uint32_t* re, uint32_t* im, const Fp2& a, const Fp2& b) {
+  uint32_t t1[16], e[16], o[15], sa[8], sb[8];
+  mul_wide(e, o, a.c0.v, b.c0.v);
+  merge_wide(re, e, o);
+  mul_wide(e, o, a.c1.v, b.c1.v);
+  merge_wide(t1, e, o);
+  add8(sa, a.c0.v, a.c1.v);
+  add8(sb, b.c0.v, b.c1.v);
+  mul_wide(e, o, sa, sb);
+  merge_wide(im, e, o);
+  w_sub(im, re);
+  w_sub(im, t1);
+  return w_sub(re, t1);
+}
+// t += N R if neg
+__device__ __forceinline__ void fix_neg(uint32_t* t, uint32_t neg) {
+  uint32_t h[8], m[8], x[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    m[i] = mod_limb<FpCfg>(i) & (0u - neg);
+    x[i] = t[8 + i];
+  }
+  add8(h, x, m);
+#pragma unroll
+  for (int i = 0; i < 8; i++) t[8 + i] = h[i];
+}
+}  // namespace eo
+
 static __device__ __noinline__ Fp2 f_mul(Fp2 a, Fp2 b) {
-  Fp t0 = f_mulc(a.c0, b.c0);
-  Fp t1 = f_mulc(a.c1, b.c1);
-  Fp t2 = f_mulc(f_add(a.c0, a.c1), f_add(b.c0, b.c1));
-  return {f_sub(t0, t1), f_sub(f_sub(t2, t0), t1)};
+  uint32_t re[16], im[16];
+  const uint32_t neg = eo::mul2_wide(re, im, a, b);
+  eo::fix_neg(re, neg);
+  return {f_redc_wide<FpCfg>(re), f_redc_wide<FpCfg>(im)};
 }
 
-// (a0 + a1 i)^2 = (a0 + a1)(a0 - a1) + 2 a0 a1 i
+// a b + c d: |Re| < 2 N^2 < N R and Im < 4 N^2 < N R, so one reduction each still holds
+static __device__ __noinline__ Fp2 f_mul2(Fp2 a, Fp2 b, Fp2 c, Fp2 d) {
+  uint32_t re[16], im[16], r2[16], i2[16];
+  eo::mul2_wide(re, im, a, b);
+  eo::mul2_wide(r2, i2, c, d);
+  eo::w_add(im, i2);
+  eo::w_add(re, r2);
+  eo::fix_neg(re, re[15] >> 31);
+  return {f_redc_wide<FpCfg>(re), f_redc_wide<FpCfg>(im)};
+}
+
+// (a0 + a1 i)^2 = (a0 + a1)(a0 - a1) + 2 a0 a1 i, the factors unreduced (below 2N)
 static __device__ __noinline__ Fp2 f_sqr(Fp2 a) {
-  Fp t = f_mulc(a.c0, a.c1);
-  return {f_mulc(f_add(a.c0, a.c1), f_sub(a.c0, a.c1)), f_dbl(t)};
+  Fp s, d, t, u;
+  const Fp m = Fp::modulus();
+  add8(s.v, a.c0.v, a.c1.v);
+  sub8(u.v, m.v, a.c1.v);
+  add8(d.v, a.c0.v, u.v);
+  add8(t.v, a.c0.v, a.c0.v);
+  return {f_mulc(s, d), f_mulc(t, a.c1)};
 }
 
 __device__ __forceinline__ Fp2 f_inv(const Fp2& a) {
