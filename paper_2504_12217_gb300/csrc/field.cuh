@@ -67,7 +67,6 @@ struct FpCfg {
                                  0x8181585du, 0xb85045b6u, 0xe131a029u, 0x30644e72u}};
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
-  static constexpr U256c R3 = cx_pow2_mod(768, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
 };
 
@@ -76,7 +75,6 @@ struct FrCfg {
                                  0x8181585du, 0xb85045b6u, 0xe131a029u, 0x30644e72u}};
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
-  static constexpr U256c R3 = cx_pow2_mod(768, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
 };
 
@@ -98,8 +96,6 @@ template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t r1_limb(int i) { ZKVC_LIMB_SWITCH(C::R1, i) }
 template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t r2_limb(int i) { ZKVC_LIMB_SWITCH(C::R2, i) }
-template <class C>
-__host__ __device__ __forceinline__ constexpr uint32_t r3_limb(int i) { ZKVC_LIMB_SWITCH(C::R3, i) }
 
 // ------------------------------------------------------------------ carry-chain rows
 // t[0..8] += a[0..7] * b : low halves into t[0..7] (carry into t[8]), then high halves
@@ -740,278 +736,214 @@ __device__ __forceinline__ Field<C> f_pow(const Field<C>& a, const uint32_t (&e)
   return r;
 }
 
-// Inverse of a Montgomery-form element (a R -> a^-1 R); 0 maps to 0.  The integer
-// inverse y^-1 mod N of y = a R comes from the binary GCD, and a product with R^3 brings
-// y^-1 = a^-1 R^-1 back to Montgomery form.  Not constant-time.
+// Inverse of a Montgomery-form element (a R -> a^-1 R); 0 maps to 0.  Not constant-time.
 //
-// Binary GCD with Bezout coefficients: (a, b) = (y, N), (u, v) = (1, 0), invariants
-// a = u y and b = v y (mod N); an odd a larger than b becomes a - b (u - v), a smaller one
-// is swapped first; an even a is halved (u halved mod N).  a reaches 0 and b = gcd = 1
-// within 2 len(N) - 1 steps, and then v = y^-1.
+// Divsteps (Bernstein and Yang, "Fast constant-time gcd computation and modular inversion",
+// 2019) on (f, g) = (N, a R): f odd, a step halves g, or g + f, or swaps the two first.  30
+// steps at a time run on the low 32 bits alone, since their decisions need no magnitudes,
+// and are recorded as a matrix of 31-bit integers with
+//   2^30 (f, g)' = [[u, v], [q, r]] (f, g);
+// the same matrix then updates (f, g) exactly and (d, e) modulo N, where d = f / (a R) and
+// e = g / (a R) up to the factor R^2 that e starts with, so that d ends as +-a^-1 R with
+// f = +-1 and no closing product.  The steps inside a batch run as many at once as the
+// trailing zeros and the step counter allow (up to six), so a batch is about eight rounds of
+// short dependent integer operations.  Numbers are signed 30-bit limbs: a division by 2^30
+// drops a limb, and no magnitude comparison or carry chain is left.  At most
+// (49 * 254 + 57) / 17 = 735 steps reach g = 0 for values below 2^254: 25 batches (18 on
+// average).
 //
-// Fast path (Pornin, "Optimized Binary GCD for Modular Inversion", 2020): 30 steps at a
-// time on 62-bit stand-ins for a and b (their low 30 bits and top 32 bits at the common
-// length n = max(len a, len b, 62)), whose parity and order decisions are recorded as an
-// integer matrix [[f0, g0], [f1, g1]] with entries at most 2^30 in magnitude; then the
-// exact update (a, b) <- ((f0 a + g0 b) / 2^30, (f1 a + g1 b) / 2^30), made non-negative
-// by flipping a row's sign, and (u, v) <- the same rows applied to (u, v) and divided by
-// 2^30 mod N (one Montgomery step), which keeps the invariants without a final
-// power-of-two correction.  ceil((2 * 254 - 1) / 30) = 17 rounds reach a = 0, b = 1 for
-// 254-bit moduli; a round after that leaves (a, b, v) unchanged.  Should the check at the
-// end ever fail, the one-step-at-a-time loop below recomputes the inverse.  (One thread:
-// about 50 k cycles against 78 k for the one-step loop.)
-__device__ __forceinline__ void shr1_8(uint32_t (&x)[8], uint32_t top) {
-#pragma unroll
-  for (int i = 0; i < 7; i++) x[i] = (x[i] >> 1) | (x[i + 1] << 31);
-  x[7] = (x[7] >> 1) | (top << 31);
+// What bounds it: the latency of one thread, half in the rounds and half in the updates'
+// wide products.  Measured: one thread 31 k cycles, a warp of 32 inversions 40 k, against
+// 53 k for the binary GCD with magnitude stand-ins before.  (The rounds with selects in
+// place of the branches take 39 k and 54 k.)
+struct S30 {
+  int32_t v[9];
+};
+
+namespace inv30 {
+constexpr uint32_t M30 = 0x3fffffffu;
+
+// limb i of x in base 2^30
+__host__ __device__ constexpr int32_t limb30(const U256c& x, int i) {
+  const int bit = 30 * i, w = bit / 32, sh = bit % 32;
+  const uint64_t lo = x.w[w], hi = w + 1 < 8 ? x.w[w + 1] : 0u;
+  return (int32_t)(((lo | (hi << 32)) >> sh) & M30);
 }
-
-__device__ __forceinline__ bool is_one8(const uint32_t (&x)[8]) {
-  uint32_t acc = x[0] ^ 1u;
-#pragma unroll
-  for (int i = 1; i < 8; i++) acc |= x[i];
-  return acc == 0;
-}
-
-
-namespace bgcd {
-// bit length of x | y
-__device__ __forceinline__ int len2(const uint32_t (&x)[8], const uint32_t (&y)[8]) {
-  int n = 0;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    const uint32_t w = x[i] | y[i];
-    n = w ? 32 * i + 32 - __clz(w) : n;
-  }
-  return n;
-}
-
-// (x mod 2^30) + 2^30 floor(x / 2^(n - 32)) for len(x) <= n, 62 <= n <= 256
-__device__ __forceinline__ uint64_t approx(const uint32_t (&x)[8], int n) {
-  const int s = n - 32, q = s >> 5, r = s & 31;
-  uint32_t lo = 0, hi = 0;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    lo = i == q ? x[i] : lo;
-    hi = i == q + 1 ? x[i] : hi;
-  }
-  const uint64_t top = ((((uint64_t)hi << 32) | lo) >> r) & 0xffffffffull;
-  return (uint64_t)(x[0] & 0x3fffffffu) | (top << 30);
-}
-
-// t = x f + y g as a 9-limb two's complement number (x, y < 2^254, |f|, |g| <= 2^30):
-// x f is x |f| with every limb complemented and 1 added when f < 0
-__device__ __forceinline__ void lin9(uint32_t (&t)[9], const uint32_t (&x)[8], int32_t f, const uint32_t (&y)[8],
-                                     int32_t g) {
-  const uint32_t mf = (uint32_t)(f < 0 ? -f : f), mg = (uint32_t)(g < 0 ? -g : g);
-  const uint32_t sf = (uint32_t)(f >> 31), sg = (uint32_t)(g >> 31);
-  uint64_t cf = 0, cg = 0, c = (sf & 1u) + (sg & 1u);
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    if (i < 8) {
-      cf += (uint64_t)x[i] * mf;
-      cg += (uint64_t)y[i] * mg;
-    }
-    c += (uint64_t)((uint32_t)cf ^ sf) + ((uint32_t)cg ^ sg);
-    t[i] = (uint32_t)c;
-    c >>= 32;
-    cf >>= 32;
-    cg >>= 32;
-  }
-}
-
-// t >>= 30, arithmetic
-__device__ __forceinline__ void sar30(uint32_t (&t)[9]) {
-#pragma unroll
-  for (int i = 0; i < 8; i++) t[i] = (t[i] >> 30) | (t[i + 1] << 2);
-  t[8] = (uint32_t)((int32_t)t[8] >> 30);
-}
-
-// t = -t when s = ~0 (s = 0: unchanged)
-__device__ __forceinline__ void cneg9(uint32_t (&t)[9], uint32_t s) {
-  uint64_t c = s & 1u;
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    c += (uint32_t)(t[i] ^ s);
-    t[i] = (uint32_t)c;
-    c >>= 32;
-  }
-}
-
-// t += m, or t -= m, over 9 limbs
-__device__ __forceinline__ void addm9(uint32_t (&t)[9], const uint32_t (&m)[8], bool sub) {
-  const uint32_t x = sub ? 0xffffffffu : 0u;
-  uint64_t c = sub ? 1u : 0u;
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    c += (uint64_t)t[i] + ((i < 8 ? m[i] : 0u) ^ x);
-    t[i] = (uint32_t)c;
-    c >>= 32;
-  }
-}
-
-// (x f + y g) / 2^30 mod m in [0, m), for x, y in [0, m): q = t (-m^-1) mod 2^30 makes
-// t + q m divisible by 2^30, and -2m < (t + q m) / 2^30 < 3m
-__device__ __forceinline__ void upd_mod(uint32_t (&out)[8], const uint32_t (&x)[8], int32_t f, const uint32_t (&y)[8],
-                                        int32_t g, const uint32_t (&m)[8], uint32_t minv) {
-  uint32_t t[9];
-  lin9(t, x, f, y, g);
-  const uint32_t q = (t[0] * minv) & 0x3fffffffu;
-  uint64_t c = 0;
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    if (i < 8) c += (uint64_t)m[i] * q;
-    c += t[i];
-    t[i] = (uint32_t)c;
-    c >>= 32;
-  }
-  sar30(t);
-  for (int k = 0; k < 2 && (int32_t)t[8] < 0; k++) addm9(t, m, false);
-  for (int k = 0; k < 2; k++) {
-    uint32_t d9[9];
-#pragma unroll
-    for (int i = 0; i < 9; i++) d9[i] = t[i];
-    addm9(d9, m, true);
-    if ((int32_t)d9[8] < 0) break;
-#pragma unroll
-    for (int i = 0; i < 9; i++) t[i] = d9[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 8; i++) out[i] = t[i];
-}
-}  // namespace bgcd
-
-// y^-1 mod N for 0 < y < N (integers, 8 limbs); false if the rounds did not finish
 template <class C>
-__device__ __noinline__ bool inv_bgcd(const uint32_t (&y)[8], uint32_t (&out)[8]) {
-  uint32_t a[8], b[8], u[8], v[8], m[8];
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    m[i] = mod_limb<C>(i);
-    a[i] = y[i];
-    b[i] = m[i];
-    u[i] = i == 0;
-    v[i] = 0;
+__host__ __device__ constexpr int32_t mod30(int i) {
+  switch (i) {
+    case 0: return limb30(C::MOD, 0);
+    case 1: return limb30(C::MOD, 1);
+    case 2: return limb30(C::MOD, 2);
+    case 3: return limb30(C::MOD, 3);
+    case 4: return limb30(C::MOD, 4);
+    case 5: return limb30(C::MOD, 5);
+    case 6: return limb30(C::MOD, 6);
+    case 7: return limb30(C::MOD, 7);
+    default: return limb30(C::MOD, 8);
   }
-  const uint32_t minv = C::INV;  // -N^-1 mod 2^32, hence also mod 2^30
-  for (int round = 0; round < 17; round++) {
-    const int n = max(bgcd::len2(a, b), 62);
-    uint64_t ab = bgcd::approx(a, n), bb = bgcd::approx(b, n);
-    int32_t f0 = 1, g0 = 0, f1 = 0, g1 = 1;
-    // 30 binary-GCD steps on the stand-ins, without branches
-#pragma unroll 10
-    for (int j = 0; j < 30; j++) {
-      const bool odd = ab & 1u;
-      const bool sw = odd && ab < bb;
-      const uint64_t na = sw ? bb : ab, nb = sw ? ab : bb;
-      const int32_t nf0 = sw ? f1 : f0, ng0 = sw ? g1 : g0, nf1 = sw ? f0 : f1, ng1 = sw ? g0 : g1;
-      ab = (odd ? na - nb : na) >> 1;
-      bb = nb;
-      f0 = odd ? nf0 - nf1 : nf0;
-      g0 = odd ? ng0 - ng1 : ng0;
-      f1 = nf1 * 2;
-      g1 = ng1 * 2;
+}
+template <class C>
+__host__ __device__ constexpr int32_t rr30(int i) {
+  switch (i) {
+    case 0: return limb30(C::R2, 0);
+    case 1: return limb30(C::R2, 1);
+    case 2: return limb30(C::R2, 2);
+    case 3: return limb30(C::R2, 3);
+    case 4: return limb30(C::R2, 4);
+    case 5: return limb30(C::R2, 5);
+    case 6: return limb30(C::R2, 6);
+    case 7: return limb30(C::R2, 7);
+    default: return limb30(C::R2, 8);
+  }
+}
+
+struct Mat {
+  int32_t u, v, q, r;
+};
+
+// 30 divsteps from the low 32 bits of f (odd) and g; eta = -delta
+__device__ __forceinline__ int divsteps30(int eta, uint32_t f, uint32_t g, Mat* t) {
+  uint32_t u = 1, v = 0, q = 0, r = 1;
+  int i = 30;
+  for (;;) {
+    const int z = __clz((int)__brev(g | (0xffffffffu << i)));  // even steps: halvings
+    g >>= z;
+    u <<= z;
+    v <<= z;
+    eta -= z;
+    i -= z;
+    if (i == 0) break;
+    if (eta < 0) {  // g odd and delta > 0: (f, g) <- (g, -f)
+      eta = -eta;
+      uint32_t x = f;
+      f = g;
+      g = 0u - x;
+      x = u;
+      u = q;
+      q = 0u - x;
+      x = v;
+      v = r;
+      r = 0u - x;
     }
-    uint32_t ta[9], tb[9];
-    bgcd::lin9(ta, a, f0, b, g0);
-    bgcd::lin9(tb, a, f1, b, g1);
-    bgcd::sar30(ta);
-    bgcd::sar30(tb);
-    const uint32_t sa = (uint32_t)((int32_t)ta[8] >> 31), sb = (uint32_t)((int32_t)tb[8] >> 31);
-    bgcd::cneg9(ta, sa);
-    bgcd::cneg9(tb, sb);
-    f0 = sa ? -f0 : f0;
-    g0 = sa ? -g0 : g0;
-    f1 = sb ? -f1 : f1;
-    g1 = sb ? -g1 : g1;
-    uint32_t nu[8], nv[8];
-    bgcd::upd_mod(nu, u, f0, v, g0, m, minv);
-    bgcd::upd_mod(nv, u, f1, v, g1, m, minv);
+    // the next min(eta + 1, i) steps keep f: add the multiple of f that clears as many of
+    // g's low bits (at most six: f (f^2 - 2) = -1 / f mod 2^6)
+    const uint32_t w = (f * g * (f * f - 2u)) & ~(0xffffffffu << min(min(eta + 1, i), 6));
+    g += f * w;
+    q += u * w;
+    r += v * w;
+  }
+  t->u = (int32_t)u;
+  t->v = (int32_t)v;
+  t->q = (int32_t)q;
+  t->r = (int32_t)r;
+  return eta;
+}
+
+// (f, g) <- t (f, g) / 2^30, exact
+__device__ __forceinline__ void update_fg(S30& f, S30& g, const Mat& t) {
+  int64_t cf = (int64_t)t.u * f.v[0] + (int64_t)t.v * g.v[0];
+  int64_t cg = (int64_t)t.q * f.v[0] + (int64_t)t.r * g.v[0];
+  cf >>= 30;
+  cg >>= 30;
+#pragma unroll
+  for (int i = 1; i < 9; i++) {
+    const int32_t fi = f.v[i], gi = g.v[i];
+    cf += (int64_t)t.u * fi + (int64_t)t.v * gi;
+    cg += (int64_t)t.q * fi + (int64_t)t.r * gi;
+    f.v[i - 1] = (int32_t)((uint32_t)cf & M30);
+    g.v[i - 1] = (int32_t)((uint32_t)cg & M30);
+    cf >>= 30;
+    cg >>= 30;
+  }
+  f.v[8] = (int32_t)cf;
+  g.v[8] = (int32_t)cg;
+}
+
+// (d, e) <- t (d, e) / 2^30 mod N; d and e stay in (-2N, N)
+template <class C>
+__device__ __forceinline__ void update_de(S30& d, S30& e, const Mat& t) {
+  constexpr uint32_t ninv = (0u - C::INV) & M30;  // N^-1 mod 2^30
+  const int32_t sd = d.v[8] >> 31, se = e.v[8] >> 31;
+  // multiples of N: one for each negative operand, then what makes the sum divisible
+  int32_t md = (t.u & sd) + (t.v & se), me = (t.q & sd) + (t.r & se);
+  int64_t cd = (int64_t)t.u * d.v[0] + (int64_t)t.v * e.v[0];
+  int64_t ce = (int64_t)t.q * d.v[0] + (int64_t)t.r * e.v[0];
+  md -= (int32_t)((ninv * (uint32_t)cd + (uint32_t)md) & M30);
+  me -= (int32_t)((ninv * (uint32_t)ce + (uint32_t)me) & M30);
+  cd += (int64_t)mod30<C>(0) * md;
+  ce += (int64_t)mod30<C>(0) * me;
+  cd >>= 30;
+  ce >>= 30;
+#pragma unroll
+  for (int i = 1; i < 9; i++) {
+    const int32_t di = d.v[i], ei = e.v[i];
+    cd += (int64_t)t.u * di + (int64_t)t.v * ei + (int64_t)mod30<C>(i) * md;
+    ce += (int64_t)t.q * di + (int64_t)t.r * ei + (int64_t)mod30<C>(i) * me;
+    d.v[i - 1] = (int32_t)((uint32_t)cd & M30);
+    e.v[i - 1] = (int32_t)((uint32_t)ce & M30);
+    cd >>= 30;
+    ce >>= 30;
+  }
+  d.v[8] = (int32_t)cd;
+  e.v[8] = (int32_t)ce;
+}
+
+// x in (-2N, N), negated if neg, brought to [0, N): limbs carry signed values until the end
+template <class C>
+__device__ __forceinline__ void normalize(S30& x, bool neg) {
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    const int32_t add = x.v[8] >> 31;  // negative: add N (to (-N, N), then to [0, N))
+#pragma unroll
+    for (int i = 0; i < 9; i++) x.v[i] += mod30<C>(i) & add;
+    if (k == 0 && neg) {
+#pragma unroll
+      for (int i = 0; i < 9; i++) x.v[i] = -x.v[i];
+    }
 #pragma unroll
     for (int i = 0; i < 8; i++) {
-      a[i] = ta[i];
-      b[i] = tb[i];
-      u[i] = nu[i];
-      v[i] = nv[i];
+      x.v[i + 1] += x.v[i] >> 30;
+      x.v[i] &= (int32_t)M30;
     }
   }
-  uint32_t z = b[0] ^ 1u;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    z |= a[i] | (i ? b[i] : 0u);
-    out[i] = v[i];
-  }
-  return z == 0;
 }
+}  // namespace inv30
 
 template <class C>
 __device__ __noinline__ Field<C> f_inv(const Field<C>& a) {
   if (a.is_zero()) return Field<C>::zero();
-  {
-    uint32_t r[8];
-    if (inv_bgcd<C>(a.v, r)) {
-      Field<C> x, r3;
+  S30 d, e, f, g;
 #pragma unroll
-      for (int i = 0; i < 8; i++) {
-        x.v[i] = r[i];
-        r3.v[i] = r3_limb<C>(i);
-      }
-      return f_mul(x, r3);
-    }
+  for (int i = 0; i < 9; i++) {
+    const int bit = 30 * i, w = bit / 32, sh = bit % 32;
+    const uint32_t lo = a.v[w], hi = w + 1 < 8 ? a.v[w + 1] : 0u;
+    g.v[i] = (int32_t)(__funnelshift_r(lo, hi, sh) & inv30::M30);
+    f.v[i] = inv30::mod30<C>(i);
+    d.v[i] = 0;
+    e.v[i] = inv30::rr30<C>(i);
   }
-  uint32_t p[8], u[8], v[8], x1[8], x2[8];
+  int eta = -1;
+  for (int batch = 0; batch < 25; batch++) {
+    inv30::Mat t;
+    // the low 32 bits: 30 of limb 0 and two of limb 1
+    eta = inv30::divsteps30(eta, (uint32_t)f.v[0] | ((uint32_t)f.v[1] << 30),
+                            (uint32_t)g.v[0] | ((uint32_t)g.v[1] << 30), &t);
+    inv30::update_de<C>(d, e, t);
+    inv30::update_fg(f, g, t);
+    int32_t z = 0;
+#pragma unroll
+    for (int i = 0; i < 9; i++) z |= g.v[i];
+    if (z == 0) break;
+  }
+  inv30::normalize<C>(d, f.v[8] < 0);
+  Field<C> r;
 #pragma unroll
   for (int i = 0; i < 8; i++) {
-    p[i] = mod_limb<C>(i);
-    u[i] = a.v[i];
-    v[i] = p[i];
-    x1[i] = 0;
-    x2[i] = 0;
+    const int bit = 32 * i, l = bit / 30, sh = bit % 30;  // bits [32 i, 32 i + 32) span limbs l, l + 1
+    r.v[i] = ((uint32_t)d.v[l] >> sh) | ((uint32_t)d.v[l + 1] << (30 - sh));
   }
-  x1[0] = 1;
-  while (!is_one8(u) && !is_one8(v)) {
-    while ((u[0] & 1u) == 0) {
-      shr1_8(u, 0);
-      if (x1[0] & 1u) {
-        uint32_t c = add8(x1, x1, p);
-        shr1_8(x1, c);
-      } else {
-        shr1_8(x1, 0);
-      }
-    }
-    while ((v[0] & 1u) == 0) {
-      shr1_8(v, 0);
-      if (x2[0] & 1u) {
-        uint32_t c = add8(x2, x2, p);
-        shr1_8(x2, c);
-      } else {
-        shr1_8(x2, 0);
-      }
-    }
-    uint32_t d[8];
-    if (!sub8(d, u, v)) {  // u >= v
-#pragma unroll
-      for (int i = 0; i < 8; i++) u[i] = d[i];
-      if (sub8(d, x1, x2)) add8(d, d, p);
-#pragma unroll
-      for (int i = 0; i < 8; i++) x1[i] = d[i];
-    } else {
-      sub8(d, v, u);
-#pragma unroll
-      for (int i = 0; i < 8; i++) v[i] = d[i];
-      if (sub8(d, x2, x1)) add8(d, d, p);
-#pragma unroll
-      for (int i = 0; i < 8; i++) x2[i] = d[i];
-    }
-  }
-  Field<C> r, r3;
-  const bool uone = is_one8(u);
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    r.v[i] = uone ? x1[i] : x2[i];
-    r3.v[i] = r3_limb<C>(i);
-  }
-  return f_mul(r, r3);
+  return r;
 }
 
 using Fp = Field<FpCfg>;
