@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "coop.cuh"
@@ -186,9 +187,29 @@ size_t scan_u32_temp_bytes(size_t n) {
 }
 
 // ------------------------------------------------------------------ planning
+constexpr uint64_t TREE_MIN_TERMS = 1ull << 22;
+constexpr uint32_t TREE_MAX_ROUNDS = 5;
+constexpr uint32_t TREE_NONE = 0xffffffffu;        // a padding term of a bucket
+constexpr uint64_t TREE_NONE_BASE = 0x7fffffffull;  // base indices stay below: no term equals TREE_NONE
 // Threads of the G1 accumulation kernel resident on the whole GPU at `at` threads per
 // block (one per chunk), from the occupancy of its register use; cached per block size.
 static uint64_t accum_resident_threads(uint32_t at);
+
+// Pairwise affine rounds before level 0 (k_tree below), by the run's bucket terms and their
+// average per bucket.  r rounds pad every bucket to a multiple of 2^r terms, 2^(r-1) pads
+// on average, so r keeps them to about a sixteenth; what r rounds leave to the XYZZ
+// additions is 2^-r of the terms.  Measured (G1 MSM, eight windows of 16 bits): 2^18 points
+// = 4.2 M terms 1.54 ms with rounds, 1.59 without, 2^20 3.52 and 4.28, 3,000,001 8.53 and
+// 10.83; below 2^22 terms the rounds' launches and inversions cost what they save (2^17
+// points 1.26 and 1.25, 2^16 points 0.87 and 0.81).  G2 of 2^18 points 4.01 and 4.27.  At
+// 64 terms per bucket a fourth round loses (3.72 against 3.57 ms at 2^20 points).
+static uint32_t tree_rounds(uint64_t slots, uint32_t keys, uint64_t base_end) {
+  if (slots < TREE_MIN_TERMS || base_end >= TREE_NONE_BASE) return 0;
+  const uint64_t avg = slots / std::max<uint32_t>(keys, 1u);
+  uint32_t r = 0;
+  while (r < TREE_MAX_ROUNDS && (avg >> (r + 1)) >= 8) r++;
+  return r;
+}
 
 int msm_plan_finalize(MsmPlan& p) {
   uint32_t key = 0;
@@ -202,7 +223,7 @@ int msm_plan_finalize(MsmPlan& p) {
     key += o.nkeys;
   }
   p.keys = key;
-  uint64_t slot = 0;
+  uint64_t slot = 0, base_end = 0;
   uint32_t pts = 0;
   p.max_nd = 0;
   for (auto& s : p.segs) {
@@ -226,6 +247,7 @@ int msm_plan_finalize(MsmPlan& p) {
       ZK_CHECK(s.nwin >= nd, ZKVC_EINVAL, "msm: %u digits but %u stored windows", nd, s.nwin);
     }
     ZK_CHECK(s.base_off + uint64_t(s.count) * s.nwin <= 0x80000000ull, ZKVC_EINVAL, "msm: base index overflow");
+    base_end = std::max<uint64_t>(base_end, s.base_off + uint64_t(s.count) * s.nwin);
     s.nd = nd;
     s.slot_off = slot;
     s.point_off = pts;
@@ -236,22 +258,29 @@ int msm_plan_finalize(MsmPlan& p) {
   // term indices, bucket offsets and chunk bounds are 32-bit: 2^31 slots leave every sum
   // of an index and a chunk length below 2^32
   ZK_CHECK(slot <= (1ull << 31), ZKVC_EINVAL, "msm: %llu digit slots (at most 2^31)", (unsigned long long)slot);
+  p.rounds = tree_rounds(slot, key, base_end);
+  p.pad_slots = p.rounds ? key * ((1u << p.rounds) - 1u) : 0u;
   // default chunk: about two chunks per bucket, but at least ~40 k chunks so that the
-  // accumulation fills the GPU, and 16 at the least; and at least the chunk that puts
-  // every term into one wave of resident accumulation threads (the chunks are balanced,
-  // so a second, partial wave would only add a tail)
+  // accumulation fills the GPU, and 16 at the least (8 after affine rounds, where level 0
+  // is a small part); and at least the chunk that puts every point into one wave of
+  // resident accumulation threads (the chunks are balanced, so a second, partial wave
+  // would only add a tail).  Counted in the points that the affine rounds leave.
+  const uint64_t pts0 = (slot + p.pad_slots) >> p.rounds;
   if (p.tune.chunk) {
+    ZK_CHECK(p.tune.chunk <= 1024, ZKVC_EINVAL, "msm: chunk of %u terms", p.tune.chunk);
     p.chunk = p.tune.chunk;
+    p.chunk_pts = std::max<uint32_t>(1u, p.chunk >> p.rounds);
   } else {
-    const uint64_t per_bucket = slot / (2ull * std::max<uint32_t>(key, 1u));
-    const uint64_t fill = slot / 40960ull;
+    const uint64_t per_bucket = pts0 / (2ull * std::max<uint32_t>(key, 1u));
+    const uint64_t fill = pts0 / 40960ull;
     // (7/8 of the resident threads: the prover's other streams hold some SM slots)
     const uint64_t resident = accum_resident_threads(p.tune.accum_threads) * 7 / 8;
-    const uint64_t one_wave = resident ? (slot + resident - 1) / resident : 0;
-    p.chunk = (uint32_t)std::min<uint64_t>(
-        std::max<uint64_t>(std::max<uint64_t>(16, std::min(per_bucket, fill)), one_wave), 1024);
+    const uint64_t one_wave = resident ? (pts0 + resident - 1) / resident : 0;
+    const uint64_t least = p.rounds ? 8 : 16;
+    p.chunk_pts = (uint32_t)std::min<uint64_t>(
+        std::max<uint64_t>(std::max<uint64_t>(least, std::min(per_bucket, fill)), one_wave), 1024u >> p.rounds);
+    p.chunk = p.chunk_pts << p.rounds;
   }
-  ZK_CHECK(p.chunk >= 1 && p.chunk <= 1024, ZKVC_EINVAL, "msm: chunk of %u terms", p.chunk);
   ZK_CHECK(p.tune.accum_threads >= 32 && p.tune.accum_threads <= 256 && p.tune.accum_threads % 32 == 0,
            ZKVC_EINVAL, "msm: %u accumulation threads", p.tune.accum_threads);
   ZK_CHECK(p.tune.lanes == 0 || p.tune.lanes == 1 || p.tune.lanes == 4, ZKVC_EINVAL, "msm: %u lanes per chunk",
@@ -260,7 +289,7 @@ int msm_plan_finalize(MsmPlan& p) {
   p.points = pts;
   // lanes per chunk: quads where the run has too few chunks to fill the GPU (their point
   // operations have a third of a thread's latency), one thread where it is throughput-bound
-  p.lanes = p.tune.lanes ? p.tune.lanes : (slot / p.chunk < 40960 ? 4u : 1u);
+  p.lanes = p.tune.lanes ? p.tune.lanes : (pts0 / p.chunk_pts < 40960 ? 4u : 1u);
   // outputs with their own base arrays: every output must name one, and all must have
   // the same power-of-two key count, so that a key's output is key >> key_shift
   p.key_shift = -1;
@@ -548,6 +577,331 @@ __device__ __forceinline__ XYZZ<F> madd_lanes(const XYZZ<F>& p, const Affine<F>&
   else return p_add_affine_quad(p, q);
 }
 
+// ------------------------------------------------------------------ affine rounds
+// Large runs first add their sorted terms pairwise in affine coordinates, r rounds of
+// (P_2i, P_2i+1) -> P_i, before the XYZZ accumulation takes the 2^-r of them that remain.
+// An affine addition costs 5M + 1S with its inversion shared (Montgomery's trick: the
+// prefix products of the denominators, one inversion, and two products per denominator on
+// the way back; Montgomery, "Speeding the Pollard and elliptic curve methods of
+// factorization", 1987), against 8M + 2S for the mixed XYZZ addition.  Every bucket is padded to a
+// multiple of 2^r terms (TREE_NONE, read as infinity), so that no pair straddles two
+// buckets and every round is a plain halving of the array.
+
+// pcounts[k] = counts[k] rounded up to 2^r; counts[K] += the block's terms
+__global__ void __launch_bounds__(256) k_tree_pad(uint32_t* counts, uint32_t K, uint32_t r, uint32_t* pcounts) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x, m = (1u << r) - 1u;
+  const uint32_t c = k < K ? counts[k] : 0u;
+  if (k < K) pcounts[k] = (c + m) & ~m;
+  const uint32_t w = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0 && w) atomicAdd(counts + K, w);
+}
+
+// the padding terms, and the bucket offsets in points after r rounds
+__global__ void __launch_bounds__(256) k_tree_fill(const uint32_t* __restrict__ counts,
+                                                   const uint32_t* __restrict__ offs, uint32_t K, uint32_t r,
+                                                   uint32_t* sorted, uint32_t* offs_pts) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k > K) return;
+  offs_pts[k] = offs[k] >> r;
+  if (k == K) return;
+  for (uint32_t i = offs[k] + counts[k]; i < offs[k + 1]; i++) sorted[i] = TREE_NONE;
+}
+
+// A round over the pairs of a slab takes three launches, so that no block waits for an
+// inversion: k_tree_up multiplies the denominators (each thread those of its TREE_PER or
+// fewer pairs, one after another, then the block's 128 products down to TREE_W), k_tree_inv
+// inverts the blocks' products, k_tree_down walks back: the inverse of a block's product
+// gives the threads' and, pair by pair, each denominator's, and the pair's sum replaces its
+// prefix product (kept in the sum's own place).
+//
+// What bounds it: k_tree_down by its products (G1: 27 clocks per pair and SM, 20 if the
+// multiplier never idled), k_tree_up of the first round by the gather of single 64-byte
+// points (4.2 TB/s of them).  A block that kept its pairs through all rounds, inverting once
+// per round itself, took 49 clocks per pair: warps idle at the barrier around the inversion.
+// Measured for 15.4 M additions of a 2^20-point MSM: 1.9 ms against 2.6 for XYZZ.
+constexpr int TREE_BT = 128, TREE_W = 4, TREE_LEVELS = 2 * TREE_BT - TREE_W;
+constexpr uint32_t TREE_PER = 32;                 // pairs per thread at most
+constexpr uint64_t TREE_SLAB = 1ull << 25;        // terms per slab: 1.6 GB of points in G1
+// resident blocks per SM that the registers are cut to (k_tree_down: 96 in G1)
+template <class F>
+struct TreeMinB {
+  static constexpr int value = sizeof(F) > 32 ? 2 : 5;
+};
+
+// what a round works on: the slab's terms [start, start + len) of the sorted array, halved
+// `step` times already
+template <class F>
+struct TreeRound {
+  const uint32_t* sorted;
+  const uint32_t* offs;
+  uint32_t K, nout;
+  const Affine<F>* bases;
+  const Affine<F>* const* obases;
+  int key_shift;
+  uint32_t step, per;
+  uint64_t start, len;
+  const Affine<F>* src;  // points of the round before (step > 0)
+  Affine<F>* dst;
+  F* levels;             // TREE_LEVELS products per block
+};
+
+template <class F>
+__device__ __forceinline__ uint32_t tree_pairs(const TreeRound<F>& a) {
+  const uint64_t S = a.offs[a.K];
+  if (a.start >= S) return 0;
+  return (uint32_t)((S - a.start < a.len ? S - a.start : a.len) >> (a.step + 1));
+}
+
+// Operands of a thread's pairs: pointers (null: infinity) and whether y is negated.  The
+// term words are loaded a pair ahead of their use (word), the points a pair ahead of theirs.
+template <class F>
+struct TreeOperands {
+  const Affine<F>*p, *q;
+  bool np, nq;
+  uint32_t lo = 1, hi = 0;  // terms of the output whose base array is at hand
+  const Affine<F>* base = nullptr;
+
+  static __device__ __forceinline__ uint2 word(const TreeRound<F>& a, uint32_t i) {
+    return a.step ? make_uint2(0, 0) : *reinterpret_cast<const uint2*>(a.sorted + a.start + 2 * size_t(i));
+  }
+  __device__ __forceinline__ void at(const TreeRound<F>& a, uint32_t i, uint2 v) {
+    if (a.step == 0) {
+      const uint32_t t = (uint32_t)a.start + 2 * i;
+      if (a.key_shift < 0) {
+        base = a.bases;
+      } else if (t < lo || t >= hi) {  // the output whose buckets hold this term
+        uint32_t l = 0, h = a.nout - 1;
+        while (l < h) {
+          const uint32_t m = (l + h + 1) >> 1;
+          if (a.offs[size_t(m) << a.key_shift] <= t) l = m; else h = m - 1;
+        }
+        lo = a.offs[size_t(l) << a.key_shift];
+        hi = a.offs[size_t(l + 1) << a.key_shift];
+        base = a.obases[l];
+      }
+      p = v.x == TREE_NONE ? nullptr : base + (v.x & 0x7fffffffu);
+      q = v.y == TREE_NONE ? nullptr : base + (v.y & 0x7fffffffu);
+      np = (v.x >> 31) != 0;
+      nq = (v.y >> 31) != 0;
+    } else {
+      p = a.src + 2 * size_t(i);
+      q = p + 1;
+      np = nq = false;
+    }
+  }
+};
+
+// The denominator of p + q for the operands' x: x_q - x_p; 2 y for a doubling; one where
+// none is needed (an operand at infinity, or q = -p).
+template <class F>
+__device__ __forceinline__ F tree_denominator(const TreeOperands<F>& o, const F& xp, const F& xq) {
+  bool ip = o.p == nullptr, iq = o.q == nullptr;
+  if (!ip && xp.is_zero()) ip = ld_field(&o.p->y).is_zero();
+  if (!iq && xq.is_zero()) iq = ld_field(&o.q->y).is_zero();
+  F d = f_sub(xq, xp);
+  if (ip || iq) return F::one();
+  if (d.is_zero()) {
+    F yp = ld_field(&o.p->y), yq = ld_field(&o.q->y);
+    if (o.np) yp = f_neg(yp);
+    if (o.nq) yq = f_neg(yq);
+    d = (yp == yq && !yp.is_zero()) ? f_dbl(yp) : F::one();
+  }
+  return d;
+}
+
+template <class F>
+__global__ void __launch_bounds__(TREE_BT, TreeMinB<F>::value) k_tree_up(TreeRound<F> a) {
+  __shared__ F sh[TREE_LEVELS];
+  const uint32_t t = threadIdx.x, n = tree_pairs(a);
+  const uint32_t i0 = blockIdx.x * TREE_BT * a.per;
+  if (i0 >= n) return;
+  F run = F::one();
+  if (i0 + t < n) {
+    const uint32_t m = min(a.per, (n - 1 - i0 - t) / TREE_BT + 1);
+    TreeOperands<F> o;
+    F xp = F::zero(), xq = F::zero();
+    o.at(a, i0 + t, TreeOperands<F>::word(a, i0 + t));
+    if (o.p) xp = ld_field(&o.p->x);
+    if (o.q) xq = ld_field(&o.q->x);
+    uint2 v = make_uint2(0, 0);
+    if (m > 1) v = TreeOperands<F>::word(a, i0 + TREE_BT + t);
+    for (uint32_t j = 0; j < m; j++) {
+      const uint32_t i = i0 + j * TREE_BT + t;
+      const F d = tree_denominator(o, xp, xq);
+      if (j + 1 < m) {  // the next pair's x, while this pair's product runs
+        o.at(a, i + TREE_BT, v);
+        if (j + 2 < m) v = TreeOperands<F>::word(a, i + 2 * TREE_BT);
+        xp = F::zero();
+        xq = F::zero();
+        if (o.p) xp = ld_field(&o.p->x);
+        if (o.q) xq = ld_field(&o.q->x);
+      }
+      if (j == 0) {
+        run = d;
+      } else {
+        st_field(&a.dst[i].x, run);
+        run = f_mul(run, d);
+      }
+    }
+  }
+  st_field(sh + t, run);
+  uint32_t at = 0;
+  for (uint32_t w = TREE_BT / 2; w >= (uint32_t)TREE_W; w >>= 1) {  // node t of a level: t and t + w below
+    __syncthreads();
+    if (t < w) st_field(sh + at + 2 * w + t, f_mulx(ld_field(sh + at + t), ld_field(sh + at + w + t)));
+    at += 2 * w;
+  }
+  __syncthreads();
+  F* const lev = a.levels + size_t(blockIdx.x) * TREE_LEVELS;
+  for (uint32_t i = t; i < (uint32_t)TREE_LEVELS; i += TREE_BT) st_field(lev + i, ld_field(sh + i));
+}
+
+template <class F>
+__global__ void __launch_bounds__(64) k_tree_inv(TreeRound<F> a) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, blk = i / TREE_W;
+  if (blk * TREE_BT * a.per >= tree_pairs(a)) return;
+  F* const v = a.levels + size_t(blk) * TREE_LEVELS + (TREE_LEVELS - TREE_W) + i % TREE_W;
+  st_field(v, f_inv(ld_field(v)));
+}
+
+// 16-byte asynchronous copies into this thread's column of the staging array (chunk c of
+// thread t at c TREE_BT + t: conflict-free); a null source stores zeros (the copy then reads
+// no byte of `valid`)
+template <int CHUNKS>
+__device__ __forceinline__ void tree_stage(uint4* dst, const void* src, const void* valid) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst), bytes = src ? 16u : 0u;
+  const uint8_t* s = static_cast<const uint8_t*>(src ? src : valid);
+#pragma unroll
+  for (int c = 0; c < CHUNKS; c++)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + c * TREE_BT * 16), "l"(s + 16 * c), "r"(bytes)
+                 : "memory");
+}
+template <class T>
+__device__ __forceinline__ T tree_unstage(const uint4* src) {
+  T r;
+  uint32_t* w = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+  for (int c = 0; c < (int)(sizeof(T) / 16); c++) {
+    const uint4 q = src[c * TREE_BT];
+    w[4 * c] = q.x;
+    w[4 * c + 1] = q.y;
+    w[4 * c + 2] = q.z;
+    w[4 * c + 3] = q.w;
+  }
+  return r;
+}
+
+template <class F>
+__global__ void __launch_bounds__(TREE_BT, TreeMinB<F>::value) k_tree_down(TreeRound<F> a) {
+  // two stages in turn: a stage is refilled an iteration after its words were used
+  constexpr int CP = sizeof(Affine<F>) / 16, CF = sizeof(F) / 16, STAGE = (2 * CP + CF) * TREE_BT;
+  extern __shared__ uint4 tree_stages[];
+  const uint32_t t = threadIdx.x, n = tree_pairs(a);
+  const uint32_t i0 = blockIdx.x * TREE_BT * a.per;
+  if (i0 + t >= n) return;
+  uint32_t j = (n - 1 - i0 - t) / TREE_BT;
+  if (j >= a.per) j = a.per - 1;
+  TreeOperands<F> o;
+  auto fetch = [&](uint32_t jj, uint2 v) {
+    const uint32_t i = i0 + jj * TREE_BT + t;
+    uint4* const stage = tree_stages + (jj & 1) * STAGE + t;
+    o.at(a, i, v);
+    tree_stage<CP>(stage, o.p, a.levels);
+    tree_stage<CP>(stage + CP * TREE_BT, o.q, a.levels);
+    if (jj) tree_stage<CF>(stage + 2 * CP * TREE_BT, &a.dst[i].x, a.levels);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(j, TreeOperands<F>::word(a, i0 + j * TREE_BT + t));
+  uint2 v = make_uint2(0, 0);
+  if (j) v = TreeOperands<F>::word(a, i0 + (j - 1) * TREE_BT + t);
+  const F* lev = a.levels + size_t(blockIdx.x) * TREE_LEVELS;
+  // the inverse of this thread's product: from its node of the last level, times the
+  // sibling of each level on the way to the leaves
+  F inv = ld_field(lev + (TREE_LEVELS - TREE_W) + (t & (TREE_W - 1)));
+  uint32_t at = TREE_LEVELS - TREE_W;
+  for (uint32_t w = TREE_W; w < (uint32_t)TREE_BT; w <<= 1) {
+    at -= 2 * w;
+    inv = f_mulx(inv, ld_field(lev + at + ((t & (2 * w - 1)) ^ w)));
+  }
+  for (;; j--) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const uint4* const stage = tree_stages + (j & 1) * STAGE + t;
+    Affine<F> p = tree_unstage<Affine<F>>(stage), q = tree_unstage<Affine<F>>(stage + CP * TREE_BT);
+    F iv = inv;
+    if (j) iv = tree_unstage<F>(stage + 2 * CP * TREE_BT);
+    if (o.np) p.y = f_neg(p.y);
+    if (o.nq) q.y = f_neg(q.y);
+    if (j) {  // the next pair's points, while this pair's products run
+      fetch(j - 1, v);
+      if (j > 1) v = TreeOperands<F>::word(a, i0 + (j - 2) * TREE_BT + t);
+    }
+    const bool ip = p.is_inf(), iq = q.is_inf();
+    F d = f_sub(q.x, p.x), num = f_sub(q.y, p.y);
+    bool none = false;
+    if (ip || iq) {
+      d = F::one();
+    } else if (d.is_zero()) {
+      if (num.is_zero() && !p.y.is_zero()) {
+        d = f_dbl(p.y);
+        const F xx = f_sqrx(p.x);
+        num = f_add(f_dbl(xx), xx);
+      } else {
+        d = F::one();
+        none = true;
+      }
+    }
+    if (j) {
+      iv = f_mul(inv, iv);
+      inv = f_mul(inv, d);
+    }
+    const F l = f_mul(num, iv);
+    Affine<F> s;
+    s.x = f_sub(f_sub(f_sqr(l), p.x), q.x);
+    s.y = f_sub(f_mul(l, f_sub(p.x, s.x)), p.y);
+    if (ip) s = q;
+    else if (iq) s = p;
+    else if (none) s = Affine<F>::inf();
+    st_field(a.dst + (i0 + j * TREE_BT + t), s);
+    if (j == 0) break;
+  }
+}
+
+// pairs per thread of a round of at most `pairs`: as many as leave four waves of resident
+// blocks, 1 to TREE_PER
+template <class F>
+static uint32_t tree_per(uint64_t pairs) {
+  const uint64_t wave = uint64_t(TREE_BT) * TreeMinB<F>::value * (uint64_t)device_sm_count();
+  return (uint32_t)std::min<uint64_t>(TREE_PER, std::max<uint64_t>(1, pairs / (4 * wave)));
+}
+
+// blocks whose products a slab of `len` terms needs room for: the first round's count bounds
+// the later rounds' as long as each thread takes at least one pair
+template <class F>
+static uint64_t tree_level_blocks(uint64_t len, uint32_t rounds) {
+  uint64_t most = 0;
+  for (uint32_t r = 0; r < rounds; r++) {
+    const uint64_t pairs = len >> (r + 1), per = tree_per<F>(pairs);
+    most = std::max<uint64_t>(most, (pairs + TREE_BT * per - 1) / (TREE_BT * per));
+  }
+  return most;
+}
+
+// shared memory of k_tree_down: two stages of two points and a prefix product per thread
+template <class F>
+static size_t tree_down_smem() {
+  static std::once_flag once;
+  constexpr size_t bytes = 2 * (2 * sizeof(Affine<F>) + sizeof(F)) * TREE_BT;
+  std::call_once(once, [] { cudaFuncSetAttribute(k_tree_down<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
+  return bytes;
+}
+
+// slabs of equal length (a multiple of 2^rounds) for `terms` terms
+static uint64_t tree_slab(uint64_t terms, uint32_t rounds) {
+  const uint64_t n = (terms + TREE_SLAB - 1) / TREE_SLAB;
+  const uint64_t len = n ? (terms + n - 1) / n : 0, m = (1ull << rounds) - 1;
+  return (len + m) & ~m;
+}
+
 #ifndef ZKVC_ACCUM_MINB
 #define ZKVC_ACCUM_MINB 1
 #endif
@@ -558,7 +912,8 @@ struct AccumMinB {
 
 // level 0: chunk q sums the sorted terms [q T0, (q + 1) T0) with mixed additions, storing
 // its running sum at slot q + k whenever bucket k ends inside the chunk and at its end
-template <class F, int QL>
+// (DIRECT: the terms are the points left by the affine rounds, in order, unsigned)
+template <class F, int QL, bool DIRECT>
 __global__ void __launch_bounds__(256, AccumMinB<F>::value) k_accum0(const uint32_t* __restrict__ sorted,
                                                                     const uint32_t* __restrict__ offs, uint32_t K,
                                                                     uint32_t T0, const Affine<F>* __restrict__ bases,
@@ -573,7 +928,7 @@ __global__ void __launch_bounds__(256, AccumMinB<F>::value) k_accum0(const uint3
   const uint32_t end = end64 < S ? (uint32_t)end64 : S;
   uint32_t k = find_key(offs, K, start);  // the bucket holding term `start`
   uint32_t next = offs[k + 1];
-  if (key_shift >= 0) bases = obases[k >> key_shift];
+  if (!DIRECT && key_shift >= 0) bases = obases[k >> key_shift];
   const bool lead = QL == 1 || quad_lane() == 0;
   XYZZ<F> acc = XYZZ<F>::inf();
   // one loop of exactly end - start additions for every lane (no divergence between
@@ -588,11 +943,16 @@ __global__ void __launch_bounds__(256, AccumMinB<F>::value) k_accum0(const uint3
         k++;
         next = offs[k + 1];
       } while (p >= next);
-      if (key_shift >= 0) bases = obases[k >> key_shift];
+      if (!DIRECT && key_shift >= 0) bases = obases[k >> key_shift];
     }
-    uint32_t v = sorted[p];
-    Affine<F> P = ld_field(bases + (v & 0x7fffffffu));
-    if (v >> 31) P.y = f_neg(P.y);
+    Affine<F> P;
+    if constexpr (DIRECT) {
+      P = ld_field(bases + p);
+    } else {
+      const uint32_t v = sorted[p];
+      P = ld_field(bases + (v & 0x7fffffffu));
+      if (v >> 31) P.y = f_neg(P.y);
+    }
     acc = madd_lanes<QL>(acc, P);
   }
   if (lead) st_field(part + q + k, acc);
@@ -637,7 +997,7 @@ static uint64_t accum_resident_threads(uint32_t at) {
   if (at < 32 || at > 256 || at % 32) return 0;
   int nb = per_sm[at / 32].load(std::memory_order_relaxed);
   if (nb <= 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_accum0<Fp, 1>, (int)at, 0) != cudaSuccess || nb <= 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_accum0<Fp, 1, false>, (int)at, 0) != cudaSuccess || nb <= 0) {
       cudaGetLastError();
       return 0;
     }
@@ -992,6 +1352,11 @@ __global__ void __launch_bounds__(SliceBT<F>::value) k_bits_chain(
 struct Layout {
   uint32_t *keys, *vals, *sorted, *counts, *offs, *cursor, *nch, *choff, *chunk_key, *arrive, *flist;
   void *part, *S, *D;
+  uint32_t* offs_pts;  // bucket offsets in the points left by the affine rounds
+  void* tree_out;      // those points
+  void *tree_a, *tree_b;  // a slab's points after its first and second round (then in turn)
+  void* tree_levels;
+  uint64_t tree_slab;
   MsmSeg* segs;
   MsmOut* outs;
   const void** obases;
@@ -1089,16 +1454,23 @@ static void tables(const MsmPlan& p, uint32_t bt, uint32_t wave, HostTables& h, 
 template <class F>
 static void layout(const MsmPlan& p, Arena& a, Layout& L, HostTables& h) {
   const size_t S = p.slots, K = p.keys;
-  const uint32_t T0 = p.chunk ? p.chunk : 32;
+  const uint32_t T0 = p.chunk_pts ? p.chunk_pts : 32;
+  const size_t SP = S + p.pad_slots;  // terms with the affine rounds' padding
   L.keys = a.take<uint32_t>(S);
   L.vals = a.take<uint32_t>(S);
-  L.sorted = a.take<uint32_t>(S);
-  L.counts = a.take<uint32_t>(K);
+  L.sorted = a.take<uint32_t>(SP);
+  L.counts = a.take<uint32_t>(K + 1);
   L.offs = a.take<uint32_t>(K + 1);
   L.cursor = a.take<uint32_t>(K);
   L.nch = a.take<uint32_t>(K);
   L.choff = a.take<uint32_t>(K + 1);
-  L.qmax = (uint32_t)(S / T0 + K + 1);
+  L.offs_pts = a.take<uint32_t>(p.rounds ? K + 1 : 0);
+  L.tree_out = a.take<Affine<F>>(p.rounds ? (SP >> p.rounds) : 0);
+  L.tree_slab = p.rounds ? tree_slab(SP, p.rounds) : 0;
+  L.tree_a = a.take<Affine<F>>(p.rounds > 1 ? L.tree_slab / 2 : 0);
+  L.tree_b = a.take<Affine<F>>(p.rounds > 2 ? L.tree_slab / 4 : 0);
+  L.tree_levels = a.take<F>(tree_level_blocks<F>(L.tree_slab, p.rounds) * TREE_LEVELS);
+  L.qmax = (uint32_t)((SP >> p.rounds) / T0 + K + 1);
   L.chunk_key = a.take<uint32_t>(L.qmax);
   L.arrive = a.take<uint32_t>(L.qmax);
   L.flist = a.take<uint32_t>(L.qmax);
@@ -1209,7 +1581,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   Arena a = ex->st->after_layout;
   const uint32_t K = p.keys;
   const uint64_t S = p.slots;
-  const uint32_t T0 = p.chunk;
+  const uint32_t T0 = p.chunk_pts;
   ZK_CHECK(T0 >= 1, ZKVC_EINVAL, "msm: plan not finalized");
   ZK_CHECK(p.key_shift >= 0 || bases, ZKVC_EINVAL, "msm: no base array");
 
@@ -1218,7 +1590,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   // then rarely repeat a key within a tile), else by k_hist
   bool spread = true;
   for (const auto& o : p.outs) spread = spread && o.c >= 12;
-  ZK_CUDA(cudaMemsetAsync(L.counts, 0, size_t(K) * sizeof(uint32_t), st));
+  ZK_CUDA(cudaMemsetAsync(L.counts, 0, (size_t(K) + 1) * sizeof(uint32_t), st));
   if (p.points > 0) {
     k_digits<<<(p.points + 255) / 256, 256, 0, st>>>(L.segs, (int)p.segs.size(), L.outs, p.points, L.keys, L.vals,
                                                      spread ? L.counts : nullptr);
@@ -1230,13 +1602,21 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
     k_hist<<<sb, HB_THREADS, 0, st>>>(L.keys, S, L.counts); ZK_COUNT_LAUNCH();
     ZK_CUDA(cudaGetLastError());
   }
-  ZK_TRY(scan_u32(L.counts, L.offs, K, a, st, L.cursor));
+  const uint32_t R = p.rounds;
+  if (R) {  // bucket sizes padded for the affine rounds (nch is free until k_chunk_layout)
+    k_tree_pad<<<(K + 255) / 256, 256, 0, st>>>(L.counts, K, R, L.nch); ZK_COUNT_LAUNCH();
+  }
+  ZK_TRY(scan_u32(R ? L.nch : L.counts, L.offs, K, a, st, L.cursor));
+  if (R) {
+    k_tree_fill<<<(K + 1 + 255) / 256, 256, 0, st>>>(L.counts, L.offs, K, R, L.sorted, L.offs_pts); ZK_COUNT_LAUNCH();
+  }
+  const uint32_t* offs = R ? L.offs_pts : L.offs;
   if (S > 0) {
     k_scatter<<<sb, HB_THREADS, 0, st>>>(L.keys, L.vals, S, L.cursor, L.sorted); ZK_COUNT_LAUNCH();
     ZK_CUDA(cudaGetLastError());
   }
   // chunks of T0 sorted terms and the buckets' partial-sum slots
-  k_chunk_layout<<<(K + 1 + 255) / 256, 256, 0, st>>>(L.counts, L.offs, K, T0, L.nch, L.choff, L.chunk_key,
+  k_chunk_layout<<<(K + 1 + 255) / 256, 256, 0, st>>>(L.counts, offs, K, T0, L.nch, L.choff, L.chunk_key,
                                                        L.flist);
   ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
@@ -1253,29 +1633,50 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   unsigned fb = (unsigned)((uint64_t(L.qmax) * flanes + 127) / 128);
   if (accum_stage >= 0) prof_mark(accum_stage, true, st);
   const auto* ob = reinterpret_cast<const Affine<F>* const*>(L.obases);
-  if (lanes == 4)
-    k_accum0<F, 4><<<qb, at, 0, st>>>(L.sorted, L.offs, K, T0, bases, ob, p.key_shift, part);
-  else
-    k_accum0<F, 1><<<qb, at, 0, st>>>(L.sorted, L.offs, K, T0, bases, ob, p.key_shift, part);
+  if (R) {
+    Affine<F>* const pts = reinterpret_cast<Affine<F>*>(L.tree_out);
+    TreeRound<F> a{L.sorted, L.offs, K, (uint32_t)p.outs.size(), bases, ob, p.key_shift, 0, 0, 0, L.tree_slab,
+                   nullptr, nullptr, reinterpret_cast<F*>(L.tree_levels)};
+    for (a.start = 0; a.start < S + p.pad_slots; a.start += a.len) {
+      for (a.step = 0; a.step < R; a.step++) {
+        a.src = a.dst;
+        a.dst = a.step + 1 == R ? pts + (a.start >> R) : reinterpret_cast<Affine<F>*>(a.step & 1 ? L.tree_b : L.tree_a);
+        const uint64_t pairs = a.len >> (a.step + 1);
+        a.per = tree_per<F>(pairs);
+        const unsigned blocks = (unsigned)((pairs + TREE_BT * a.per - 1) / (TREE_BT * a.per));
+        k_tree_up<F><<<blocks, TREE_BT, 0, st>>>(a); ZK_COUNT_LAUNCH();
+        k_tree_inv<F><<<(blocks * TREE_W + 63) / 64, 64, 0, st>>>(a); ZK_COUNT_LAUNCH();
+        k_tree_down<F><<<blocks, TREE_BT, tree_down_smem<F>(), st>>>(a); ZK_COUNT_LAUNCH();
+      }
+    }
+    if (lanes == 4)
+      k_accum0<F, 4, true><<<qb, at, 0, st>>>(nullptr, offs, K, T0, pts, nullptr, -1, part);
+    else
+      k_accum0<F, 1, true><<<qb, at, 0, st>>>(nullptr, offs, K, T0, pts, nullptr, -1, part);
+  } else if (lanes == 4) {
+    k_accum0<F, 4, false><<<qb, at, 0, st>>>(L.sorted, offs, K, T0, bases, ob, p.key_shift, part);
+  } else {
+    k_accum0<F, 1, false><<<qb, at, 0, st>>>(L.sorted, offs, K, T0, bases, ob, p.key_shift, part);
+  }
   ZK_COUNT_LAUNCH();
   if (accum_stage >= 0) {
     prof_mark(accum_stage, false, st);
-    if (uint32_t* hu = prof_units(accum_stage)) ZK_CUDA(cudaMemcpyAsync(hu, L.offs + K, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    if (uint32_t* hu = prof_units(accum_stage)) ZK_CUDA(cudaMemcpyAsync(hu, R ? L.counts + K : L.offs + K, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   }
   ZK_CUDA(cudaGetLastError());
   if (after_accum) ZK_CUDA(cudaEventRecord(after_accum, st));
   // chunk boundaries 1 .. chunks - 1 index the fold list (chunks <= slots / T0 + 1)
-  const uint64_t nlist = p.slots / T0 + 2;
+  const uint64_t nlist = ((p.slots + p.pad_slots) >> R) / T0 + 2;
   const bool by_boundary = nlist < K;
   const uint32_t* fl = by_boundary ? L.flist : nullptr;
   const uint64_t n_serial = by_boundary ? nlist : uint64_t(K);
   const unsigned sfb = (unsigned)((n_serial * flanes + 127) / 128);
   const unsigned fab = std::max(sfb, fb);
   if (flanes == 4)
-    k_fold<F, 4><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, L.offs, T0,
+    k_fold<F, 4><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0,
                                       (uint32_t)n_serial);
   else
-    k_fold<F, 1><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, L.offs, T0,
+    k_fold<F, 1><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0,
                                       (uint32_t)n_serial);
   ZK_COUNT_LAUNCH();
   // sum_v v B_v per (output, window) by bit decomposition
@@ -1298,7 +1699,8 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
 
 const uint32_t* msm_term_count(const MsmExec* ex) {
   if (!ex || !ex->st) return nullptr;
-  return ex->st->L.offs + ex->plan.keys;
+  // (with affine rounds the offsets hold padding; k_tree_pad counts the terms)
+  return (ex->plan.rounds ? ex->st->L.counts : ex->st->L.offs) + ex->plan.keys;
 }
 
 template <class F>

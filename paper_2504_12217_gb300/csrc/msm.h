@@ -57,7 +57,10 @@ struct MsmPlan {
   uint32_t keys = 0;
   uint32_t points = 0;
   uint32_t max_nd = 0;
-  uint32_t chunk = 0;          // planner: the level-0 chunk in use
+  uint32_t chunk = 0;          // planner: the level-0 chunk in use, in bucket terms
+  uint32_t rounds = 0;         // planner: pairwise affine rounds before level 0
+  uint32_t pad_slots = 0;      // planner: bound on the terms that padding adds for them
+  uint32_t chunk_pts = 0;      // planner: level-0 chunk in points left by the rounds
   uint32_t lanes = 1;          // planner: lanes per chunk in use
   int32_t key_shift = -1;      // planner: log2 of the keys per output when outputs carry
                                // their own bases (all outputs then have equal 2^k keys)
