@@ -13,7 +13,7 @@
 
 namespace zkvc {
 int setup_impl(int a, int n, int b, const uint8_t* toxic, cudaStream_t st, zkvc_pk** pk, zkvc_vk** vk);
-size_t prove_workspace_bytes(const zkvc_pk* pk, int mode);
+size_t prove_workspace_bytes(const zkvc_pk* pk, int mode, bool lean = false);
 int prove_autotune(zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, const uint8_t* rs, cudaStream_t st,
                    uint32_t* chosen);
 int prove_impl(const zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, const uint8_t* rs, int32_t* dY,

@@ -192,8 +192,10 @@ static uint32_t window_bits(size_t n) {
 template <class F>
 constexpr bool msm_api_glv() { return true; }
 
-static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* out) {
+static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* out, bool affine = true) {
   MsmPlan& p = *out;
+  p = MsmPlan();
+  p.affine = affine;
   const size_t pts = glv ? 2 * n : n;
   const uint32_t bits = glv ? 128 : 255;
   // the window rule's c, then the smallest c with the same window count, so that the top
@@ -217,11 +219,11 @@ static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* 
 }
 
 template <class F>
-size_t msm_api_ws(size_t n) {
+size_t msm_api_ws(size_t n, bool affine) {
   constexpr bool glv = msm_api_glv<F>();
   const size_t pts = glv ? 2 * n : n;
   MsmPlan p;
-  if (n > ZKVC_MSM_MAX_POINTS || variable_base_plan(n, nullptr, glv, &p) != ZKVC_OK) return 0;
+  if (n > ZKVC_MSM_MAX_POINTS || variable_base_plan(n, nullptr, glv, &p, affine) != ZKVC_OK) return 0;
   return msm_workspace_bytes<F>(p) + round256(pts * sizeof(Affine<F>)) + (glv ? round256(pts * sizeof(uint4)) : 0) +
          2 * 256 + sizeof(XYZZ<F>) + sizeof(Affine<F>);
 }
@@ -310,6 +312,10 @@ int msm_api(const uint8_t* d_points, const uint8_t* d_scalars, size_t n, void* d
   MsmPlan p;
   ZK_TRY(variable_base_plan(n, nullptr, glv, &p));
   size_t need = msm_api_ws<F>(n);
+  if (ws_bytes < need && p.rounds) {  // short scratch: without the affine rounds
+    ZK_TRY(variable_base_plan(n, nullptr, glv, &p, false));
+    need = msm_api_ws<F>(n, false);
+  }
   ZK_CHECK(ws_bytes >= need, ZKVC_EINVAL, "msm: workspace %zu < %zu bytes", ws_bytes, need);
   Arena a;
   a.base = reinterpret_cast<uint8_t*>(d_ws);
@@ -343,7 +349,7 @@ int msm_api(const uint8_t* d_points, const uint8_t* d_scalars, size_t n, void* d
 }
 
 template int msm_api<Fp>(const uint8_t*, const uint8_t*, size_t, void*, size_t, uint8_t*, cudaStream_t);
-template size_t msm_api_ws<Fp>(size_t);
+template size_t msm_api_ws<Fp>(size_t, bool);
 
 // ------------------------------------------------------------------ integer-pipe rate
 // Throughput microbenchmark of the 32-bit multiply-adds that Montgomery products are made

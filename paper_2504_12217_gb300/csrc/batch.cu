@@ -185,6 +185,7 @@ struct zkvc_batch {
   uint8_t* dproofs = nullptr;
   std::vector<NttGroup> groups;
   MsmPlan p_small, p_main, p_g2;
+  bool lean = false;  // MSM runs without affine rounds, for memory too small for them
   MsmExec x_small, x_main, x_g2;
   void *ws_small = nullptr, *ws_main = nullptr, *ws_g2 = nullptr;
   size_t ws_small_bytes = 0, ws_main_bytes = 0, ws_g2_bytes = 0;
@@ -252,6 +253,7 @@ static void batch_plans(zkvc_batch* B) {
   B->p_small = MsmPlan();
   B->p_main = MsmPlan();
   B->p_g2 = MsmPlan();
+  B->p_small.affine = B->p_main.affine = B->p_g2.affine = !B->lean;
   for (int i = 0; i < B->count; i++) {
     const zkvc_pk* pk = B->pks[i];
     const Shape& sh = pk->shape;
@@ -640,6 +642,12 @@ static int batch_create(const zkvc_pk* const* pks, int count, int flags, zkvc_ba
   int rc = [&]() -> int {
     B->mem_bytes = carve(B, true);
     cudaError_t e = cudaMalloc(&B->mem, B->mem_bytes);
+    if (e != cudaSuccess) {  // once more with the smaller MSM workspaces
+      cudaGetLastError();
+      B->lean = true;
+      B->mem_bytes = carve(B, true);
+      e = cudaMalloc(&B->mem, B->mem_bytes);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       B->mem = nullptr;
@@ -732,9 +740,10 @@ int batch_serve_open(int cap, zkvc_batch** out) {
   return ZKVC_OK;
 }
 
-// Device bytes of a batch of these keys (host computation only).
-size_t batch_serve_bytes(const zkvc_pk* const* pks, int count) {
+// Device bytes of a batch of these keys (host computation only); lean: the least it runs in.
+size_t batch_serve_bytes(const zkvc_pk* const* pks, int count, bool lean) {
   zkvc_batch B;
+  B.lean = lean;
   B.owns_mem = false;
   cudaGetDevice(&B.device);
   B.pks.assign(pks, pks + count);
@@ -758,7 +767,12 @@ int batch_serve_run(zkvc_batch* B, const zkvc_pk* const* pks, int count, uint8_t
   B->pks.assign(pks, pks + count);
   B->count = count;
   B->mem = nullptr;
-  const size_t need = carve(B, true);
+  B->lean = false;
+  size_t need = carve(B, true);
+  if (need > mem_bytes) {
+    B->lean = true;
+    need = carve(B, true);
+  }
   ZK_CHECK(need <= mem_bytes, ZKVC_ENOMEM, "server batch: %zu bytes needed, %zu given", need, mem_bytes);
   B->mem = mem;
   B->mem_bytes = mem_bytes;

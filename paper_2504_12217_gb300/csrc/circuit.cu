@@ -970,7 +970,8 @@ static MsmSeg gseg(const GRegion& r, uint64_t count, uint32_t out, int kind, con
   return s;
 }
 
-static void gen_plans(const GenericKey& G, const void* src[G_COUNT], const Fr* h, const Fr* rs, GenPlans* P) {
+static void gen_plans(const GenericKey& G, const void* src[G_COUNT], const Fr* h, const Fr* rs, GenPlans* P,
+                      bool lean) {
   const GShape& sh = G.sh;
   P->pre.outs = {{C1, 1, 0, 0}, {C1, 1, 0, 0}, {C1, 1, 0, 0}};
   auto& s = P->pre.segs;
@@ -993,6 +994,7 @@ static void gen_plans(const GenericKey& G, const void* src[G_COUNT], const Fr* h
     if (G.B2[g].count) P->g2.segs.push_back(gseg(G.B2[g], sh.count[g], 0, sh.kind[g], src[g]));
   P->g2.segs.push_back(gseg(G.BETA2, 1, 0, SK_ONE, nullptr));
   P->g2.segs.push_back(gseg(G.DELTA2, 1, 0, SK_FR_CANON, rs + 1));
+  P->pre.affine = P->h.affine = P->g2.affine = !lean;
   msm_plan_finalize(P->pre);
   msm_plan_finalize(P->h);
   msm_plan_finalize(P->g2);
@@ -1003,7 +1005,8 @@ static size_t aux_bytes(const GShape& sh) {
   return std::max<size_t>(1, sh.n_aux) * e;
 }
 
-static size_t gen_carve(const zkvc_pk* pk, void* base, size_t cap, GenBufs* B, bool measuring) {
+// lean: MSM runs without affine rounds, for a workspace too small for them
+static size_t gen_carve(const zkvc_pk* pk, void* base, size_t cap, GenBufs* B, bool measuring, bool lean) {
   const GenericKey& G = *pk->gen;
   const GShape& sh = G.sh;
   Arena a;
@@ -1027,7 +1030,7 @@ static size_t gen_carve(const zkvc_pk* pk, void* base, size_t cap, GenBufs* B, b
   B->proof = a.take<uint8_t>(256);
   GenPlans P;
   const void* src[G_COUNT] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  gen_plans(G, src, nullptr, nullptr, &P);
+  gen_plans(G, src, nullptr, nullptr, &P, lean);
   B->ws_pre_bytes = msm_workspace_bytes<Fp>(P.pre);
   B->ws_h_bytes = msm_workspace_bytes<Fp>(P.h);
   B->ws_g2_bytes = msm_workspace_bytes<Fp2>(P.g2);
@@ -1037,9 +1040,9 @@ static size_t gen_carve(const zkvc_pk* pk, void* base, size_t cap, GenBufs* B, b
   return a.off;
 }
 
-size_t prove_generic_workspace_bytes(const zkvc_pk* pk) {
+size_t prove_generic_workspace_bytes(const zkvc_pk* pk, bool lean) {
   GenBufs B;
-  return gen_carve(pk, nullptr, 0, &B, true);
+  return gen_carve(pk, nullptr, 0, &B, true, lean);
 }
 
 struct GenStreams {
@@ -1055,9 +1058,11 @@ int prove_generic(const zkvc_pk* pk, const int8_t* dX, const int8_t* dW, const u
   const GenericKey& G = *pk->gen;
   const GShape& sh = G.sh;
   size_t need = prove_generic_workspace_bytes(pk);
+  const bool lean = ws_bytes < need;
+  if (lean) need = prove_generic_workspace_bytes(pk, true);
   ZK_CHECK(ws_bytes >= need, ZKVC_EINVAL, "prove: workspace %zu < %zu bytes", ws_bytes, need);
   GenBufs B;
-  gen_carve(pk, ws, ws_bytes, &B, false);
+  gen_carve(pk, ws, ws_bytes, &B, false, lean);
   const size_t N = sh.N;
   Fr* Aev = B.ev;
   Fr* Bev = B.ev + N;
@@ -1120,7 +1125,7 @@ int prove_generic(const zkvc_pk* pk, const int8_t* dX, const int8_t* dW, const u
   k_gen_wfull<<<(unsigned)((sh.n_vars + 255) / 256), 256, 0, st>>>(src, sh.n_vars, B.w); ZK_COUNT_LAUNCH();
   const void* msrc[G_COUNT] = {nullptr, dX, dY, dW, B.aux};
   GenPlans P;
-  gen_plans(G, msrc, Hev, B.rs, &P);
+  gen_plans(G, msrc, Hev, B.rs, &P, lean);
   // G2 MSM on the side stream (needs W and s)
   ZK_CUDA(cudaEventRecord(t_gen.fork, st));
   ZK_CUDA(cudaStreamWaitEvent(t_gen.side, t_gen.fork, 0));

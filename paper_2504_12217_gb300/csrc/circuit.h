@@ -59,7 +59,7 @@ struct GenericKey {
 
 int setup_generic(int a, int n, int b, int circuit, int pub, const uint8_t* toxic, cudaStream_t st, zkvc_pk** pk,
                   zkvc_vk** vk);
-size_t prove_generic_workspace_bytes(const zkvc_pk* pk);
+size_t prove_generic_workspace_bytes(const zkvc_pk* pk, bool lean = false);
 // y_given: dY holds a claimed Y to prove instead of receiving X W (ZKVC_EUNSAT if the
 // circuit's rows then fail).
 int prove_generic(const zkvc_pk* pk, const int8_t* dX, const int8_t* dW, const uint8_t* rs_host, int32_t* dY, void* ws,

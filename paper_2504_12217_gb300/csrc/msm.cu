@@ -258,7 +258,7 @@ int msm_plan_finalize(MsmPlan& p) {
   // term indices, bucket offsets and chunk bounds are 32-bit: 2^31 slots leave every sum
   // of an index and a chunk length below 2^32
   ZK_CHECK(slot <= (1ull << 31), ZKVC_EINVAL, "msm: %llu digit slots (at most 2^31)", (unsigned long long)slot);
-  p.rounds = tree_rounds(slot, key, base_end);
+  p.rounds = p.affine ? tree_rounds(slot, key, base_end) : 0;
   p.pad_slots = p.rounds ? key * ((1u << p.rounds) - 1u) : 0u;
   // default chunk: about two chunks per bucket, but at least ~40 k chunks so that the
   // accumulation fills the GPU, and 16 at the least (8 after affine rounds, where level 0
@@ -1459,7 +1459,7 @@ static void layout(const MsmPlan& p, Arena& a, Layout& L, HostTables& h) {
   L.keys = a.take<uint32_t>(S);
   L.vals = a.take<uint32_t>(S);
   L.sorted = a.take<uint32_t>(SP);
-  L.counts = a.take<uint32_t>(K + 1);
+  L.counts = a.take<uint32_t>(K + (p.rounds ? 1 : 0));  // with rounds also the term count
   L.offs = a.take<uint32_t>(K + 1);
   L.cursor = a.take<uint32_t>(K);
   L.nch = a.take<uint32_t>(K);
@@ -1590,7 +1590,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   // then rarely repeat a key within a tile), else by k_hist
   bool spread = true;
   for (const auto& o : p.outs) spread = spread && o.c >= 12;
-  ZK_CUDA(cudaMemsetAsync(L.counts, 0, (size_t(K) + 1) * sizeof(uint32_t), st));
+  ZK_CUDA(cudaMemsetAsync(L.counts, 0, (size_t(K) + (p.rounds ? 1 : 0)) * sizeof(uint32_t), st));
   if (p.points > 0) {
     k_digits<<<(p.points + 255) / 256, 256, 0, st>>>(L.segs, (int)p.segs.size(), L.outs, p.points, L.keys, L.vals,
                                                      spread ? L.counts : nullptr);

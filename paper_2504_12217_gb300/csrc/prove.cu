@@ -250,7 +250,8 @@ struct Plans {
 };
 
 static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* dY, const Fr* ak, const Fr* bk,
-                  const Fr* S, const Fr* h, const Fr* rs, const Fr* sw, const Fr* sa, const Fr* rb, Plans* P) {
+                  const Fr* S, const Fr* h, const Fr* rs, const Fr* sw, const Fr* sa, const Fr* rb, Plans* P,
+                  bool lean) {
   const Shape& sh = pk->shape;
   const Region* g = pk->lay.g1;
   const uint32_t an = sh.a * sh.n, ab = sh.a * sh.b, n = sh.n;
@@ -293,6 +294,7 @@ static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* 
       seg_of(g2[R2_BETA], 0, 1, 0, SK_ONE, nullptr),
       seg_of(g2[R2_DELTA], 0, 1, 0, SK_FR_CANON, rs + 1),
   };
+  P->small.affine = P->rest.affine = P->h.affine = P->g2.affine = !lean;
   P->small.tune.chunk = pk->prove_tune[0];
   P->rest.tune.chunk = pk->prove_tune[1];
   P->h.tune.chunk = pk->prove_tune[2];
@@ -307,7 +309,8 @@ static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* 
   msm_plan_finalize(P->g2);
 }
 
-static size_t carve(const zkvc_pk* pk, int mode, void* base, size_t cap, ProveBufs* B, bool measuring) {
+// lean: MSM runs without affine rounds, for a workspace too small for them
+static size_t carve(const zkvc_pk* pk, int mode, void* base, size_t cap, ProveBufs* B, bool measuring, bool lean) {
   const Shape& sh = pk->shape;
   const bool chain = mode == ZKVC_PROVE_CHAIN;
   Arena a;
@@ -333,7 +336,8 @@ static size_t carve(const zkvc_pk* pk, int mode, void* base, size_t cap, ProveBu
   B->res2 = a.take<G2J>(1);
   B->proof = a.take<uint8_t>(256);
   Plans P;
-  plans(pk, mode, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, &P);
+  plans(pk, mode, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, &P,
+        lean);
   B->ws_small_bytes = msm_workspace_bytes<Fp>(P.small);
   B->ws_rest_bytes = chain ? 0 : msm_workspace_bytes<Fp>(P.rest);
   B->ws_h_bytes = msm_workspace_bytes<Fp>(P.h);
@@ -381,9 +385,9 @@ static int side_streams(SideStreams** out) {
   return ZKVC_OK;
 }
 
-size_t prove_workspace_bytes(const zkvc_pk* pk, int mode) {
+size_t prove_workspace_bytes(const zkvc_pk* pk, int mode, bool lean) {
   ProveBufs B;
-  return carve(pk, mode, nullptr, 0, &B, true);
+  return carve(pk, mode, nullptr, 0, &B, true, lean);
 }
 
 static int fork_to(SideStreams* side, int i, cudaStream_t st) {
@@ -405,12 +409,14 @@ static int prove_enqueue_impl(const zkvc_pk* pk, int mode, const int8_t* dX, con
                               int* flags_out, cudaStream_t st, bool y_given = false) {
   ZK_CHECK(pk && dX && dW && rs_host && dY && ws && proof_out && flags_out, ZKVC_EINVAL, "prove: null argument");
   ZK_CHECK(mode == ZKVC_PROVE_FOLD || mode == ZKVC_PROVE_CHAIN, ZKVC_EINVAL, "prove: mode %d", mode);
-  size_t need = prove_workspace_bytes(pk, mode);
+  size_t need = prove_workspace_bytes(pk, mode, false);
+  const bool lean = ws_bytes < need;
+  if (lean) need = prove_workspace_bytes(pk, mode, true);
   ZK_CHECK(ws_bytes >= need, ZKVC_EINVAL, "prove: workspace %zu < %zu bytes", ws_bytes, need);
   const bool chain = mode == ZKVC_PROVE_CHAIN;
   const Shape& sh = pk->shape;
   ProveBufs B;
-  carve(pk, mode, ws, ws_bytes, &B, false);
+  carve(pk, mode, ws, ws_bytes, &B, false, lean);
   const size_t N = sh.N;
   Fr* Aev = B.ev;
   Fr* Bev = B.ev + N;
@@ -434,7 +440,7 @@ static int prove_enqueue_impl(const zkvc_pk* pk, int mode, const int8_t* dX, con
   SideStreams* side = nullptr;
   ZK_TRY(side_streams(&side));
   Plans P;
-  plans(pk, mode, dX, dY, B.ak, B.bk, B.S, Hev, B.rs, B.sw, B.sa, B.rb, &P);
+  plans(pk, mode, dX, dY, B.ak, B.bk, B.S, Hev, B.rs, B.sw, B.sa, B.rb, &P, lean);
   // The witness runs on two streams: the CRPC sums a_k, b_k (X, W only) and the domain
   // evaluations past row n (X, Y) on side stream 3, which then carries the critical
   // NTT -> H chain; Y = X W, Y(z) and the PSQ chain on the main stream.  The side streams
@@ -770,7 +776,7 @@ int prove_autotune(zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, co
   uint32_t saved[ZKVC_PK_TUNING_LEN];
   for (int i = 0; i < ZKVC_PK_TUNING_LEN; i++) saved[i] = pk->prove_tune[i];
   for (int i = 0; i < 4; i++) pk->prove_tune[i] = 2;  // the largest workspace of all candidates
-  size_t need = std::max(prove_workspace_bytes(pk, ZKVC_PROVE_FOLD), prove_workspace_bytes(pk, ZKVC_PROVE_CHAIN));
+  size_t need = std::max(prove_workspace_bytes(pk, ZKVC_PROVE_FOLD, false), prove_workspace_bytes(pk, ZKVC_PROVE_CHAIN, false));
   for (int i = 0; i < 4; i++) pk->prove_tune[i] = saved[i];
   void* ws = nullptr;
   int32_t* dY = nullptr;

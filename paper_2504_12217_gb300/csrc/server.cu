@@ -34,12 +34,12 @@
 #include "groth16.h"
 
 namespace zkvc {
-size_t prove_workspace_bytes(const zkvc_pk* pk, int mode);
+size_t prove_workspace_bytes(const zkvc_pk* pk, int mode, bool lean);
 int prove_enqueue(const zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, const uint8_t* rs_host,
                   int32_t* dY, void* ws, size_t ws_bytes, uint8_t* proof_out, int* flags_out, cudaStream_t st);
 int prove_status(int flags);
 int batch_serve_open(int cap, zkvc_batch** out);
-size_t batch_serve_bytes(const zkvc_pk* const* pks, int count);
+size_t batch_serve_bytes(const zkvc_pk* const* pks, int count, bool lean);
 int batch_serve_run(zkvc_batch* B, const zkvc_pk* const* pks, int count, uint8_t* mem, size_t mem_bytes,
                     const int8_t* const* hX, const int8_t* const* hW, const uint8_t* rs, int32_t* const* hY,
                     uint8_t* proofs, int* status);
@@ -139,15 +139,18 @@ struct zkvc_server {
   bool stop = false;
   std::vector<std::thread> workers;
   std::string fatal;  // set if a worker could not start
-  std::vector<size_t> fp_fold, fp_chain;  // request footprint per key and mode
+  std::vector<size_t> fp_fold, fp_chain;  // least request footprint per key and mode
+  std::vector<size_t> fp_fold_full, fp_chain_full;
   ~zkvc_server();
 };
 
 namespace zkvc {
 
-static size_t footprint(const zkvc_pk* pk, int mode) {
+// Device bytes of one request: the least it runs in (lean: admission counts on this), or
+// with room for the affine rounds of large MSM runs, taken when it is free.
+static size_t footprint(const zkvc_pk* pk, int mode, bool lean) {
   const Shape& sh = pk->shape;
-  return prove_workspace_bytes(pk, mode) + round256(size_t(sh.a) * sh.n) + round256(size_t(sh.n) * sh.b) +
+  return prove_workspace_bytes(pk, mode, lean) + round256(size_t(sh.a) * sh.n) + round256(size_t(sh.n) * sh.b) +
          round256(size_t(sh.a) * sh.b * 4);
 }
 
@@ -268,13 +271,16 @@ static void worker_main(zkvc_server* S) {
             est += f;
             kp.push_back(S->pks[h->key]);
           }
-          while (kp.size() >= 2) {
-            const size_t exact = batch_serve_bytes(kp.data(), (int)kp.size());
-            if (S->alloc.alloc(exact, &off)) {
-              fp = exact;
-              break;
+          fp = 0;
+          while (kp.size() >= 2 && fp == 0) {
+            for (const bool lean : {false, true}) {
+              const size_t exact = batch_serve_bytes(kp.data(), (int)kp.size(), lean);
+              if (S->alloc.alloc(exact, &off)) {
+                fp = exact;
+                break;
+              }
             }
-            kp.pop_back();
+            if (fp == 0) kp.pop_back();
           }
           if (kp.size() >= 2) {
             for (size_t i = 0; i < kp.size(); i++) {
@@ -308,7 +314,11 @@ static void worker_main(zkvc_server* S) {
             S->cv_done.notify_all();
             continue;
           }
-          if (S->alloc.alloc(fp, &off)) {
+          const size_t full = mode == ZKVC_PROVE_CHAIN ? S->fp_chain_full[h->key] : S->fp_fold_full[h->key];
+          bool placed = S->alloc.alloc(full, &off);
+          if (placed) fp = full;
+          else placed = S->alloc.alloc(fp, &off);
+          if (placed) {
             S->queue.pop_front();
             q = h;
             S->in_flight++;
@@ -430,9 +440,11 @@ int zkvc_server_create(const zkvc_pk* const* pks, int npk, int slots, size_t mem
   }
   S->alloc.reset(mem_budget);
   for (const zkvc_pk* pk : S->pks) {
-    S->fp_fold.push_back(footprint(pk, ZKVC_PROVE_FOLD));
-    S->fp_chain.push_back(footprint(pk, ZKVC_PROVE_CHAIN));
-    if (policy == ZKVC_SERVER_MERGE) S->fp_batch.push_back(batch_serve_bytes(&pk, 1));
+    S->fp_fold.push_back(footprint(pk, ZKVC_PROVE_FOLD, true));
+    S->fp_chain.push_back(footprint(pk, ZKVC_PROVE_CHAIN, true));
+    S->fp_fold_full.push_back(footprint(pk, ZKVC_PROVE_FOLD, false));
+    S->fp_chain_full.push_back(footprint(pk, ZKVC_PROVE_CHAIN, false));
+    if (policy == ZKVC_SERVER_MERGE) S->fp_batch.push_back(batch_serve_bytes(&pk, 1, true));
   }
   for (int i = 0; i < slots; i++) S->workers.emplace_back(worker_main, S.get());
   *out = S.release();
@@ -524,7 +536,7 @@ int zkvc_server_merge_stats(zkvc_server* s, uint64_t* merged_requests, uint64_t*
 
 size_t zkvc_server_request_bytes(const zkvc_pk* pk, int mode) {
   if (!pk || (mode != ZKVC_PROVE_FOLD && mode != ZKVC_PROVE_CHAIN)) return 0;
-  return footprint(pk, mode);
+  return footprint(pk, mode, true);
 }
 
 }  // extern "C"

@@ -1,6 +1,7 @@
 """Large MSMs go through the pairwise affine rounds (from 2^22 bucket terms): every case of
 an affine addition -- distinct points, doublings, cancellations, infinity on either side --
 over whole buckets, against the oracle's [sum s_i k_i]G for points of known discrete logs."""
+import ctypes
 import math
 import random
 
@@ -66,3 +67,24 @@ def _count(n, a, la, b, lb):
         if i % lb == b:
             return (n - 1 - i) // period + 1 if i < n else 0
     return 0
+
+
+@pytest.mark.parametrize("group", [1, 2])
+def test_short_workspace(group):
+    """A workspace that holds the run only without the affine rounds gives the same sum; one
+    that does not hold that either is refused."""
+    from paper_2504_12217_gb300 import native as nv
+    rng = random.Random(32)
+    logs, scalars = _case("random", rng)
+    P, _, _, _ = _points(group, logs)
+    s = torch.tensor(list(b"".join(v.to_bytes(32, "little") for v in scalars)), dtype=torch.uint8).view(-1, 32).cuda()
+    i = torch.arange(N, device="cuda")
+    points, sc = P[i % len(logs)].contiguous(), s[i % len(scalars)].contiguous()
+    full = nv.zkvc_msm_workspace_bytes(N, group)
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    call = nv.lib().zkvc_msm_g1 if group == 1 else nv.lib().zkvc_msm_g2
+    out = [(ctypes.c_uint8 * (64 * group))() for _ in range(3)]
+    rc = [call(nv._dev_ptr(points), nv._dev_ptr(sc), N, nv._dev_ptr(ws), size, o, nv._stream())
+          for size, o in zip((full, full // 2, full // 16), out)]
+    assert rc == [nv.ZKVC_OK, nv.ZKVC_OK, nv.ZKVC_EINVAL]
+    assert bytes(out[0]) == bytes(out[1]) and any(out[0])
