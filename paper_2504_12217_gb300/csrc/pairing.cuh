@@ -1,17 +1,30 @@
 // Optimal ate pairing over BN254 on the GPU, for Groth16 verification (zkVC Sec. II:
-// Verify checks e(A, B) = e(alpha, beta) e(IC(x), gamma) e(C, delta)).
+// Verify checks e(A, B) = e(alpha, beta) e(IC(x), gamma) e(C, delta)), by one block per
+// pairing or proof.
 //
 // Tower: Fp6 = Fp2[v]/(v^3 - xi), Fp12 = Fp6[w]/(w^2 - v), xi = 9 + i, so w^6 = xi and an
 // element is sum_m c_m w^m (c_m in Fp2, m = 2j + k for the coefficient j of v in part k).
-// G2 lives on the D-type twist y^2 = x^3 + 3/xi; psi(x, y) = (x w^2, y w^3) maps it into
-// E(Fp12).
+// G2 lives on the D-type twist y^2 = x^3 + b', b' = 3/xi; psi(x, y) = (x w^2, y w^3) maps it
+// into E(Fp12).
 //
-// Miller loop: f_(6u+2, Q)(P) with T on the twist in Jacobian coordinates (no inversions).
-// The tangent / chord through T (and Q) evaluated at P is l = yP - lambda xP w +
-// (lambda xR - yR) w^3 for a point R on the line; each line is used scaled by a factor in
-// Fp2 (2 Y Z^3 for doublings, Z3 for additions), which the final exponentiation removes.
-// Two closing additions with pi(Q) and -pi^2(Q) (Frobenius on the twist) complete the
-// optimal ate loop; 6u + 2 > 0 for this curve, so no final conjugation.
+// What bounds it: latency.  A pairing is about 450 products of Fp12 one after another, and
+// a verifier's queue is a few dozen proofs, so a thread per pairing leaves the GPU idle.
+// Here the 36 Fp2 products of an Fp12 product run side by side: three warps, 12 results
+// (6 coefficients x 2 parts) of six lanes, each lane one coefficient product's real or
+// imaginary part as a sum of two Fp products with one reduction (f_mul2).  A fourth warp
+// runs the point arithmetic of the Miller loop a step ahead, one lane per part of a
+// product.  Measured for 32 proofs (128 Miller loops, 32 final exponentiations): Miller
+// loops 16.5 -> 0.32 ms, final exponentiations 18.6 -> 0.33, the subgroup test (a 254-bit
+// multiplication per proof before) 6.2 -> 0.
+//
+// Miller loop f_(6u+2, Q)(P) over the signed digits of 6u + 2 (66 digits, 22 nonzero), T in
+// homogeneous projective coordinates (Aranha, Karabina, Longa, Gebotys and Lopez, "Faster
+// explicit formulas for computing pairings over ordinary curves", 2011).  The tangent / chord
+// through T (and Q) evaluated at P is l = yP - lambda xP w + (lambda xR - yR) w^3 for a point
+// R on the line; each line is used scaled by a factor in Fp2 (2 Y Z for doublings, X - xQ Z
+// for additions), which the final exponentiation removes, as it does the vertical lines that
+// negative digits leave out.  Two closing additions with pi(Q) and -pi^2(Q) (Frobenius on
+// the twist) complete the optimal ate loop; 6u + 2 > 0 for this curve, so no final conjugation.
 //
 // Final exponentiation f^((p^12 - 1)/r): the easy part f^((p^6 - 1)(p^2 + 1)) with one
 // inversion and a Frobenius, then the hard part (p^4 - p^2 + 1)/r = p^3 + l2 p^2 + l1 p + l0
@@ -24,217 +37,416 @@
 
 namespace zkvc {
 
-struct Fp6 {
-  Fp2 c0, c1, c2;
-};
-struct Fp12 {
-  Fp6 c0, c1;
-};
-
-// ------------------------------------------------------------------ Fp2 helpers
-__device__ __forceinline__ Fp2 f2_conj(const Fp2& a) { return {a.c0, f_neg(a.c1)}; }
-__device__ __forceinline__ Fp2 f2_mul_fp(const Fp2& a, const Fp& s) { return {f_mul(a.c0, s), f_mul(a.c1, s)}; }
-// (a0 + a1 i)(9 + i) = (9 a0 - a1) + (a0 + 9 a1) i
-__device__ __forceinline__ Fp2 f2_mul_xi(const Fp2& a) {
-  Fp t0 = f_add(f_dbl(f_dbl(f_dbl(a.c0))), a.c0);
-  Fp t1 = f_add(f_dbl(f_dbl(f_dbl(a.c1))), a.c1);
-  return {f_sub(t0, a.c1), f_add(a.c0, t1)};
-}
-
-// ------------------------------------------------------------------ Fp6
-// The out-of-line tower functions take their operands by reference and copy them into
-// locals on entry: with a 384-byte by-value Fp12 parameter read again after nested
-// out-of-line calls, the exponentiation by u returned wrong values on sm_103a (found
-// against the oracle; the same loop inlined into its caller was correct).
-__device__ __forceinline__ Fp6 f6_add(const Fp6& a, const Fp6& b) {
-  return {f_add(a.c0, b.c0), f_add(a.c1, b.c1), f_add(a.c2, b.c2)};
-}
-__device__ __forceinline__ Fp6 f6_sub(const Fp6& a, const Fp6& b) {
-  return {f_sub(a.c0, b.c0), f_sub(a.c1, b.c1), f_sub(a.c2, b.c2)};
-}
-__device__ __forceinline__ Fp6 f6_neg(const Fp6& a) { return {f_neg(a.c0), f_neg(a.c1), f_neg(a.c2)}; }
-// (c0, c1, c2) v = (xi c2, c0, c1)
-__device__ __forceinline__ Fp6 f6_mul_v(const Fp6& a) { return {f2_mul_xi(a.c2), a.c0, a.c1}; }
-
-static __device__ __noinline__ Fp6 f6_mul(const Fp6& a_in, const Fp6& b_in) {
-  const Fp6 a = a_in, b = b_in;
-  Fp2 t0 = f_mul(a.c0, b.c0), t1 = f_mul(a.c1, b.c1), t2 = f_mul(a.c2, b.c2);
-  Fp2 c0 = f_add(t0, f2_mul_xi(f_sub(f_sub(f_mul(f_add(a.c1, a.c2), f_add(b.c1, b.c2)), t1), t2)));
-  Fp2 c1 = f_add(f_sub(f_sub(f_mul(f_add(a.c0, a.c1), f_add(b.c0, b.c1)), t0), t1), f2_mul_xi(t2));
-  Fp2 c2 = f_add(f_sub(f_sub(f_mul(f_add(a.c0, a.c2), f_add(b.c0, b.c2)), t0), t2), t1);
-  return {c0, c1, c2};
-}
-
-__device__ __forceinline__ Fp6 f6_inv(const Fp6& a) {
-  Fp2 A = f_sub(f_sqr(a.c0), f2_mul_xi(f_mul(a.c1, a.c2)));
-  Fp2 B = f_sub(f2_mul_xi(f_sqr(a.c2)), f_mul(a.c0, a.c1));
-  Fp2 C = f_sub(f_sqr(a.c1), f_mul(a.c0, a.c2));
-  Fp2 F = f_add(f_mul(a.c0, A), f2_mul_xi(f_add(f_mul(a.c2, B), f_mul(a.c1, C))));
-  Fp2 fi = f_inv(F);
-  return {f_mul(A, fi), f_mul(B, fi), f_mul(C, fi)};
-}
-
-// ------------------------------------------------------------------ Fp12
-__device__ __forceinline__ Fp12 f12_one() {
-  Fp12 r;
-  r.c0 = {Fp2::one(), Fp2::zero(), Fp2::zero()};
-  r.c1 = {Fp2::zero(), Fp2::zero(), Fp2::zero()};
-  return r;
-}
-
-static __device__ __noinline__ Fp12 f12_mul(const Fp12& a_in, const Fp12& b_in) {
-  const Fp12 a = a_in, b = b_in;
-  Fp6 t0 = f6_mul(a.c0, b.c0), t1 = f6_mul(a.c1, b.c1);
-  Fp12 r;
-  r.c0 = f6_add(t0, f6_mul_v(t1));
-  r.c1 = f6_sub(f6_sub(f6_mul(f6_add(a.c0, a.c1), f6_add(b.c0, b.c1)), t0), t1);
-  return r;
-}
-
-// (a0 + a1 w)^2 = (a0 + a1)(a0 + v a1) - t - v t + 2 t w, t = a0 a1
-static __device__ __noinline__ Fp12 f12_sqr(const Fp12& a_in) {
-  const Fp12 a = a_in;
-  Fp6 t = f6_mul(a.c0, a.c1);
-  Fp12 r;
-  r.c0 = f6_sub(f6_sub(f6_mul(f6_add(a.c0, a.c1), f6_add(a.c0, f6_mul_v(a.c1))), t), f6_mul_v(t));
-  r.c1 = f6_add(t, t);
-  return r;
-}
-
-__device__ __forceinline__ Fp12 f12_conj(const Fp12& a) { return {a.c0, f6_neg(a.c1)}; }
-
-// (a0 + a1 w)^-1 = (a0 - a1 w) / (a0^2 - v a1^2)
-__device__ __forceinline__ Fp12 f12_inv(const Fp12& a) {
-  Fp6 t = f6_sub(f6_mul(a.c0, a.c0), f6_mul_v(f6_mul(a.c1, a.c1)));
-  Fp6 ti = f6_inv(t);
-  return {f6_mul(a.c0, ti), f6_neg(f6_mul(a.c1, ti))};
-}
-
-__device__ __forceinline__ bool f12_is_one(const Fp12& a) {
-  Fp12 o = f12_one();
-  return a.c0.c0 == o.c0.c0 && a.c0.c1 == o.c0.c1 && a.c0.c2 == o.c0.c2 && a.c1.c0 == o.c1.c0 &&
-         a.c1.c1 == o.c1.c1 && a.c1.c2 == o.c1.c2;
-}
-
-// Frobenius constants: gam[k][m] = xi^(m (p^k - 1) / 6) for k = 1, 2, 3 and m < 6 (index k-1).
-struct FrobTab {
-  Fp2 g[3][6];
-};
-
-// f^(p^k): c_m -> c_m^(p^k) gam[k][m] with c^(p^k) = conj(c) for odd k
-__device__ __forceinline__ Fp12 f12_frob(const Fp12& a, const FrobTab& T, int k) {
-  const Fp2* g = T.g[k - 1];
-  const bool cj = (k & 1) != 0;
-  auto tw = [&](const Fp2& c, int m) { return f_mul(cj ? f2_conj(c) : c, g[m]); };
-  Fp12 r;
-  r.c0 = {tw(a.c0.c0, 0), tw(a.c0.c1, 2), tw(a.c0.c2, 4)};
-  r.c1 = {tw(a.c1.c0, 1), tw(a.c1.c1, 3), tw(a.c1.c2, 5)};
-  return r;
-}
-
-// ------------------------------------------------------------------ Miller loop
-struct G2Jac {
-  Fp2 X, Y, Z;
-};
-
-// l = l0 + l1 w + l3 w^3 = (l0, 0, 0) + (l1, l3, 0) w
-__device__ __forceinline__ Fp12 line_to_f12(const Fp2& l0, const Fp2& l1, const Fp2& l3) {
-  Fp12 r;
-  r.c0 = {l0, Fp2::zero(), Fp2::zero()};
-  r.c1 = {l1, l3, Fp2::zero()};
-  return r;
-}
-
-// tangent at T evaluated at P (scaled by 2 Y Z^3), and T <- 2T
-__device__ __forceinline__ Fp12 miller_dbl(G2Jac& T, const Fp& xP, const Fp& yP) {
-  Fp2 A = f_sqr(T.X), B = f_sqr(T.Y), C = f_sqr(B);
-  Fp2 ZZ = f_sqr(T.Z);
-  Fp2 D = f_dbl(f_sub(f_sub(f_sqr(f_add(T.X, B)), A), C));
-  Fp2 E = f_add(f_dbl(A), A);
-  Fp2 F = f_sqr(E);
-  Fp2 l3 = f_sub(f_mul(E, T.X), f_dbl(B));   // 3 X^3 - 2 Y^2
-  Fp2 X3 = f_sub(F, f_dbl(D));
-  Fp2 Y3 = f_sub(f_mul(E, f_sub(D, X3)), f_dbl(f_dbl(f_dbl(C))));
-  Fp2 Z3 = f_dbl(f_mul(T.Y, T.Z));
-  Fp2 l0 = f2_mul_fp(f_mul(Z3, ZZ), yP);     // 2 Y Z^3 yP
-  Fp2 l1 = f_neg(f2_mul_fp(f_mul(E, ZZ), xP));  // -3 X^2 Z^2 xP
-  T = {X3, Y3, Z3};
-  return line_to_f12(l0, l1, l3);
-}
-
-// chord through T and Q (affine) evaluated at P (scaled by Z3), and T <- T + Q
-__device__ __forceinline__ Fp12 miller_add(G2Jac& T, const G2A& Q, const Fp& xP, const Fp& yP) {
-  Fp2 ZZ = f_sqr(T.Z), ZZZ = f_mul(T.Z, ZZ);
-  Fp2 H = f_sub(f_mul(Q.x, ZZ), T.X);
-  Fp2 R = f_sub(f_mul(Q.y, ZZZ), T.Y);
-  Fp2 HH = f_sqr(H), HHH = f_mul(H, HH), V = f_mul(T.X, HH);
-  Fp2 X3 = f_sub(f_sub(f_sqr(R), HHH), f_dbl(V));
-  Fp2 Y3 = f_sub(f_mul(R, f_sub(V, X3)), f_mul(T.Y, HHH));
-  Fp2 Z3 = f_mul(T.Z, H);
-  Fp2 l0 = f2_mul_fp(Z3, yP);
-  Fp2 l1 = f_neg(f2_mul_fp(R, xP));
-  Fp2 l3 = f_sub(f_mul(R, Q.x), f_mul(Z3, Q.y));
-  T = {X3, Y3, Z3};
-  return line_to_f12(l0, l1, l3);
-}
-
 static constexpr uint64_t BN_U = 4965661367192848881ull;  // the curve parameter u
 
-// bit i of the loop scalar 6u + 2 (65 bits; bit 64 is set, the low 64 bits wrap)
-__device__ __forceinline__ bool ate_bit(int i) {
-  const uint64_t lo = 6ull * BN_U + 2ull;
-  return i == 64 ? true : ((lo >> i) & 1ull) != 0;
+__device__ __forceinline__ Fp2 f2_conj(const Fp2& a) { return {a.c0, f_neg(a.c1)}; }
+
+// an element of Fp12: c[2 m + part] the real or imaginary part of the coefficient of w^m
+struct alignas(16) E12 {
+  Fp c[12];
+};
+
+// Frobenius constants gam[k][m] = xi^(m (p^k - 1) / 6) for k = 1, 2, 3 and m < 6 (index
+// k-1), and the twist's b' and 3 b'
+struct FrobTab {
+  Fp2 g[3][6];
+  Fp2 b, b3;
+};
+
+// signed digits (non-adjacent form) of a positive number, least significant first
+struct Naf {
+  int8_t d[72];
+  int n;
+};
+constexpr Naf naf_digits(uint64_t lo, bool bit64) {
+  Naf r{};
+  // the number as lo + 2^64 bit64: halve, taking out +-1 where odd
+  uint64_t x = lo;
+  uint64_t top = bit64 ? 1 : 0;
+  while (x || top) {
+    int8_t z = 0;
+    if (x & 1) {
+      z = (x & 3) == 3 ? -1 : 1;
+      if (z == 1) {
+        x -= 1;
+      } else {
+        x += 1;
+        if (x == 0) top += 1;
+      }
+    }
+    r.d[r.n++] = z;
+    x = (x >> 1) | (top << 63);
+    top >>= 1;
+  }
+  return r;
+}
+// 6u + 2 has 65 bits: the low 64 wrap, bit 64 is set
+__device__ constexpr Naf ATE_NAF = naf_digits(6ull * BN_U + 2ull, true);
+__device__ constexpr Naf U_NAF = naf_digits(BN_U, false);
+
+// ------------------------------------------------------------------ Fp12 on three warps
+constexpr int PAIR_F = 96;   // threads of the Fp12 arithmetic
+constexpr int PAIR_BT = 128;  // and a warp of point arithmetic in the Miller loop
+
+__device__ __forceinline__ void f12_bar() { asm volatile("bar.sync 1, 96;" ::: "memory"); }
+
+// t < 64 N (nine limbs) mod N: the quotient from the top bits, at most one short
+__device__ __forceinline__ Fp f_mod9(const uint32_t (&t)[9]) {
+  const uint32_t h = (t[7] >> 16) | (t[8] << 16);  // t / 2^240 < 2^20
+  const uint32_t q = __umulhi(h, 346675u);         // 2^32 / 12389, N / 2^240 in (12388, 12389)
+  uint32_t p[8];
+  Fp r, x;
+  uint64_t c = 0;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    c += (uint64_t)q * mod_limb<FpCfg>(i);
+    p[i] = (uint32_t)c;
+    c >>= 32;
+    x.v[i] = t[i];
+  }
+  sub8(r.v, x.v, p);  // below 2N: the ninth limbs cancel
+  return f_once(r);
 }
 
-// f_(6u+2, Q)(P) with the two Frobenius additions; P, Q affine (Montgomery), not infinity
-static __device__ __noinline__ Fp12 miller_loop(const G1A& P_in, const G2A& Q_in, const FrobTab& T) {
-  const G1A P = P_in;
-  const G2A Q = Q_in;
-  Fp12 f = f12_one();
-  if (P.is_inf() || Q.is_inf()) return f;
-  G2Jac R{Q.x, Q.y, Fp2::one()};
-  for (int i = 63; i >= 0; i--) {
-    f = f12_mul(f12_sqr(f), miller_dbl(R, P.x, P.y));
-    if (ate_bit(i)) f = f12_mul(f, miller_add(R, Q, P.x, P.y));
+// t += x over nine limbs
+__device__ __forceinline__ void add9(uint32_t (&t)[9], const uint32_t (&x)[9]) {
+  asm("add.cc.u32  %0, %0, %9;\n\taddc.cc.u32 %1, %1, %10;\n\taddc.cc.u32 %2, %2, %11;\n\t"
+      "addc.cc.u32 %3, %3, %12;\n\taddc.cc.u32 %4, %4, %13;\n\taddc.cc.u32 %5, %5, %14;\n\t"
+      "addc.cc.u32 %6, %6, %15;\n\taddc.cc.u32 %7, %7, %16;\n\taddc.u32 %8, %8, %17;"
+      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8])
+      : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]), "r"(x[8]));
+}
+
+// dst = a b on threads 0 .. 95 (dst may be a or b).  Lane 6 g + i of warp w (g < 4, i < 6)
+// computes part g & 1 of a_i b_(m-i), m = 2 w + (g >> 1), b's index modulo 6; the terms that
+// wrap (i > m) carry w^6 = xi: xi (x + y i) = (9 x - y) + (x + 9 y) i.  The six lanes' values
+// (each below 10 N) are summed unreduced.
+static __device__ __noinline__ void f12_mul(E12* dst, const E12* a, const E12* b) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = lane < 24 ? lane / 6 : 3, i = lane < 24 ? lane % 6 : 5;
+  const int m = 2 * w + (g >> 1), part = g & 1;
+  const bool wrap = i > m;
+  const int j = wrap ? m - i + 6 : m - i;
+  const Fp a0 = ld_field(&a->c[2 * i]), a1 = ld_field(&a->c[2 * i + 1]);
+  const Fp b0 = ld_field(&b->c[2 * j + part]), b1 = ld_field(&b->c[2 * j + 1 - part]);
+  // part 0: a0 b.re + (N - a1) b.im; part 1: a0 b.im + a1 b.re
+  Fp n1 = f_comp(a1);
+#pragma unroll
+  for (int l = 0; l < 8; l++) n1.v[l] = part ? a1.v[l] : n1.v[l];
+  const Fp v = f_mul2(a0, b0, n1, b1);
+  // the other part of the same product
+  Fp o;
+  const int mate = part ? lane - 6 : lane + 6;
+#pragma unroll
+  for (int l = 0; l < 8; l++) o.v[l] = __shfl_sync(0xffffffffu, v.v[l], mate & 31);
+  uint32_t t[9];
+  {
+    // wrapped: 9 v + (part ? o : N - o)
+    const Fp co = f_comp(o);
+    const uint32_t k = wrap ? 9u : 1u;
+    uint64_t c = 0;
+#pragma unroll
+    for (int l = 0; l < 8; l++) {
+      c += (uint64_t)k * v.v[l] + (wrap ? (part ? o.v[l] : co.v[l]) : 0u);
+      t[l] = (uint32_t)c;
+      c >>= 32;
+    }
+    t[8] = (uint32_t)c;
   }
-  // pi(Q) = (conj(x) xi^((p-1)/3), conj(y) xi^((p-1)/2)); pi^2(Q) = (x xi^((p^2-1)/3), y xi^((p^2-1)/2))
-  G2A Q1{f_mul(f2_conj(Q.x), T.g[0][2]), f_mul(f2_conj(Q.y), T.g[0][3])};
-  G2A Q2n{f_mul(Q.x, T.g[1][2]), f_neg(f_mul(Q.y, T.g[1][3]))};
-  f = f12_mul(f, miller_add(R, Q1, P.x, P.y));
-  f = f12_mul(f, miller_add(R, Q2n, P.x, P.y));
-  return f;
+  uint32_t x[9], y[9];
+#pragma unroll
+  for (int l = 0; l < 9; l++) x[l] = __shfl_sync(0xffffffffu, t[l], (lane + 3) & 31);
+  add9(t, x);  // i < 3: terms i and i + 3
+#pragma unroll
+  for (int l = 0; l < 9; l++) {
+    x[l] = __shfl_sync(0xffffffffu, t[l], (lane + 1) & 31);
+    y[l] = __shfl_sync(0xffffffffu, t[l], (lane + 2) & 31);
+  }
+  add9(x, y);
+  add9(t, x);
+  const Fp r = f_mod9(t);
+  f12_bar();  // every operand has been read
+  if (lane < 24 && i == 0) st_field(&dst->c[2 * m + part], r);
+  f12_bar();
+}
+
+__device__ __forceinline__ void f12_set_one(E12* dst) {  // threads 0 .. 11 of the caller
+  if (threadIdx.x < 12) st_field(&dst->c[threadIdx.x], threadIdx.x == 0 ? Fp::one() : Fp::zero());
+}
+__device__ __forceinline__ void f12_copy(E12* dst, const E12* a) {
+  if (threadIdx.x < 12) st_field(&dst->c[threadIdx.x], ld_field(&a->c[threadIdx.x]));
+  f12_bar();
+}
+// a -> conj(a): the odd powers of w change sign (f^(p^6))
+__device__ __forceinline__ void f12_conj(E12* dst, const E12* a) {
+  if (threadIdx.x < 12) {
+    const Fp x = ld_field(&a->c[threadIdx.x]);
+    st_field(&dst->c[threadIdx.x], (threadIdx.x >> 1) & 1 ? f_neg(x) : x);
+  }
+  f12_bar();
+}
+// f^(p^k): c_m -> c_m^(p^k) gam[k][m] with c^(p^k) = conj(c) for odd k
+static __device__ __noinline__ void f12_frob(E12* dst, const E12* a, const FrobTab* T, int k) {
+  const int t = threadIdx.x;
+  Fp r = Fp::zero();
+  if (t < 12) {
+    const int m = t >> 1, part = t & 1;
+    const Fp x = ld_field(&a->c[2 * m]);
+    Fp y = ld_field(&a->c[2 * m + 1]);
+    if (k & 1) y = f_neg(y);
+    const Fp2 g = ld_field(&T->g[k - 1][m]);
+    r = part ? f_mul2(x, g.c1, y, g.c0) : f_mul2(x, g.c0, f_comp(y), g.c1);
+  }
+  f12_bar();
+  if (t < 12) st_field(&dst->c[t], r);
+  f12_bar();
 }
 
 // ------------------------------------------------------------------ final exponentiation
-static __device__ __noinline__ Fp12 f12_pow_u(const Fp12& a_in) {  // a^u
-  const Fp12 a = a_in;
-  const uint64_t u = BN_U;
-  Fp12 r = a;
-  for (int i = 61; i >= 0; i--) {  // u has 63 bits: top bit 62
-    r = f12_sqr(r);
-    if ((u >> i) & 1ull) r = f12_mul(r, a);
+// r = a^u for a in the cyclotomic subgroup (conj(a) = a^-1 in ac)
+static __device__ __noinline__ void f12_pow_u(E12* r, const E12* a, E12* ac) {
+  f12_conj(ac, a);
+  f12_copy(r, a);
+  for (int i = U_NAF.n - 2; i >= 0; i--) {
+    f12_mul(r, r, r);
+    const int d = U_NAF.d[i];
+    if (d) f12_mul(r, r, d > 0 ? a : ac);
   }
-  return r;
 }
 
-static __device__ __noinline__ Fp12 final_exp(const Fp12& f_in, const FrobTab& T) {
-  const Fp12 f = f_in;
-  // easy part: f^(p^6 - 1) = conj(f) / f, then ^(p^2 + 1)
-  Fp12 t = f12_mul(f12_conj(f), f12_inv(f));
-  t = f12_mul(f12_frob(t, T, 2), t);
-  // hard part
-  Fp12 a = f12_pow_u(t), b = f12_pow_u(a), c = f12_pow_u(b);  // t^u, t^u^2, t^u^3
-  Fp12 t2 = f12_sqr(t);
-  Fp12 a2 = f12_sqr(a), a3 = f12_mul(a2, a), a6 = f12_sqr(a3), a12 = f12_sqr(a6), a18 = f12_mul(a12, a6);
-  Fp12 b2 = f12_sqr(b), b3 = f12_mul(b2, b), b6 = f12_sqr(b3), b12 = f12_sqr(b6), b18 = f12_mul(b12, b6);
-  Fp12 b30 = f12_mul(b18, b12);
-  Fp12 c2 = f12_sqr(c), c4 = f12_sqr(c2), c8 = f12_sqr(c4), c9 = f12_mul(c8, c), c18 = f12_sqr(c9), c36 = f12_sqr(c18);
-  Fp12 y0 = f12_conj(f12_mul(f12_mul(c36, b30), f12_mul(a18, t2)));  // t^l0
-  Fp12 y1 = f12_mul(f12_conj(f12_mul(f12_mul(c36, b18), a12)), t);   // t^l1
-  Fp12 y2 = f12_mul(b6, t);                                          // t^l2
-  Fp12 r = f12_mul(f12_frob(t, T, 3), f12_frob(y2, T, 2));
-  r = f12_mul(r, f12_frob(y1, T, 1));
-  return f12_mul(r, y0);
+// f <- f^((p^12 - 1)/r) on threads 0 .. 95; s: scratch
+struct alignas(16) FinalScratch {
+  E12 t, a, b, c, x, y, z;
+  Fp inv;
+};
+static __device__ __noinline__ void final_exp(E12* f, FinalScratch* s, const FrobTab* T) {
+  // f^-1 = conj(f) g^(p^2) g^(p^4) / n, g = f conj(f) in Fp6 and n = g g^(p^2) g^(p^4) in Fp2
+  f12_conj(&s->x, f);
+  f12_mul(&s->y, f, &s->x);
+  f12_frob(&s->a, &s->y, T, 2);
+  f12_frob(&s->b, &s->a, T, 2);
+  f12_mul(&s->a, &s->a, &s->b);
+  f12_mul(&s->z, &s->y, &s->a);
+  if (threadIdx.x == 0) {
+    const Fp2 n{ld_field(&s->z.c[0]), ld_field(&s->z.c[1])}, ni = f_inv(n);
+    for (int i = 0; i < 12; i++) st_field(&s->z.c[i], i == 0 ? ni.c0 : i == 1 ? ni.c1 : Fp::zero());
+  }
+  f12_bar();
+  f12_mul(&s->a, &s->a, &s->z);
+  f12_mul(&s->a, &s->a, &s->x);
+  // easy part: t = f^(p^6 - 1) = conj(f) / f, then ^(p^2 + 1)
+  f12_mul(&s->x, &s->x, &s->a);
+  f12_frob(&s->y, &s->x, T, 2);
+  f12_mul(&s->t, &s->x, &s->y);
+  // hard part: a = t^u, b = t^(u^2), c = t^(u^3)
+  f12_pow_u(&s->a, &s->t, &s->x);
+  f12_pow_u(&s->b, &s->a, &s->x);
+  f12_pow_u(&s->c, &s->b, &s->x);
+  E12 *x = &s->x, *y = &s->y, *z = &s->z, *a = &s->a, *b = &s->b, *c = &s->c, *t = &s->t;
+  // c <- c^36
+  f12_mul(x, c, c);
+  f12_mul(x, x, x);
+  f12_mul(x, x, x);
+  f12_mul(c, x, c);  // c^9
+  f12_mul(c, c, c);
+  f12_mul(c, c, c);
+  // b: y = b^6, b <- b^18
+  f12_mul(x, b, b);
+  f12_mul(x, x, b);
+  f12_mul(y, x, x);     // b^6
+  f12_mul(z, y, y);     // b^12
+  f12_mul(b, z, y);     // b^18
+  f12_mul(z, b, z);     // b^30
+  f12_mul(y, y, t);     // t^l2 = b^6 t
+  f12_frob(f, y, T, 2);
+  f12_mul(z, z, c);     // c^36 b^30
+  f12_mul(b, b, c);     // c^36 b^18
+  // a: x = a^12, a <- a^18
+  f12_mul(x, a, a);
+  f12_mul(a, x, a);     // a^3
+  f12_mul(a, a, a);     // a^6
+  f12_mul(x, a, a);     // a^12
+  f12_mul(a, x, a);     // a^18
+  f12_mul(b, b, x);     // c^36 b^18 a^12
+  f12_conj(b, b);
+  f12_mul(b, b, t);     // t^l1
+  f12_frob(b, b, T, 1);
+  f12_mul(z, z, a);
+  f12_mul(x, t, t);
+  f12_mul(z, z, x);     // c^36 b^30 a^18 t^2
+  f12_conj(z, z);       // t^l0
+  f12_frob(t, t, T, 3);
+  f12_mul(f, f, t);
+  f12_mul(f, f, b);
+  f12_mul(f, f, z);
+}
+
+// ------------------------------------------------------------------ Miller loop
+// The point warp's variables (Fp2 each); lane 2 s + part of the warp handles part `part` of
+// slot s of a round.
+enum MillerVar : uint8_t {
+  MV_X, MV_Y, MV_Z, MV_QX, MV_QY, MV_XN, MV_YP, MV_B3,  // T, the point added, (-xP, 0), (yP, 0), 3 b'
+  MV_0, MV_1, MV_2, MV_3, MV_4, MV_5, MV_6, MV_7, MV_8, MV_9, MV_L0, MV_L1, MV_L3, MV_COUNT
+};
+struct MillerOp {
+  uint8_t dst, a, b, op;
+};
+enum : uint8_t { OP_NONE, OP_MUL, OP_ADD, OP_SUB };
+
+// A program is a list of rounds of up to five operations of one kind.
+// Doubling: B = Y^2, E = 3 b' Z^2, F = 3 E; X3 = 2 X Y (B - F), Y3 = (B + F)^2 - 12 E^2,
+// Z3 = 8 B Y Z (four times the usual coordinates); l0 = 2 Y Z yP, l1 = -3 X^2 xP, l3 = B - E.
+constexpr int MILLER_OPS = 5;
+static __device__ const MillerOp MILLER_DBL[][MILLER_OPS] = {
+    {{MV_0, MV_X, MV_Y, OP_MUL}, {MV_1, MV_Y, MV_Y, OP_MUL}, {MV_2, MV_Z, MV_Z, OP_MUL}, {MV_3, MV_Y, MV_Z, OP_MUL},
+     {MV_4, MV_X, MV_X, OP_MUL}},
+    {{MV_0, MV_0, MV_0, OP_ADD}, {MV_5, MV_1, MV_1, OP_ADD}, {MV_3, MV_3, MV_3, OP_ADD}, {MV_6, MV_4, MV_4, OP_ADD}},
+    {{MV_4, MV_6, MV_4, OP_ADD}, {MV_7, MV_3, MV_3, OP_ADD}},
+    {{MV_2, MV_B3, MV_2, OP_MUL}, {MV_L0, MV_3, MV_YP, OP_MUL}, {MV_L1, MV_4, MV_XN, OP_MUL}},
+    {{MV_6, MV_2, MV_2, OP_ADD}, {MV_L3, MV_1, MV_2, OP_SUB}},
+    {{MV_8, MV_6, MV_2, OP_ADD}},
+    {{MV_2, MV_1, MV_8, OP_ADD}, {MV_1, MV_1, MV_8, OP_SUB}, {MV_8, MV_8, MV_8, OP_ADD}},
+    {{MV_X, MV_0, MV_1, OP_MUL}, {MV_2, MV_2, MV_2, OP_MUL}, {MV_6, MV_6, MV_8, OP_MUL}, {MV_Z, MV_5, MV_7, OP_MUL}},
+    {{MV_Y, MV_2, MV_6, OP_SUB}},
+};
+// Addition of Q: th = Y - yQ Z, la = X - xQ Z, C = th^2, D = la^2, E = la D, F = Z C,
+// G = X D, H = E + F - 2 G; X3 = la H, Y3 = th (G - H) - E Y, Z3 = Z E; l0 = la yP,
+// l1 = -th xP, l3 = th xQ - la yQ.
+static __device__ const MillerOp MILLER_ADD[][MILLER_OPS] = {
+    {{MV_0, MV_QY, MV_Z, OP_MUL}, {MV_1, MV_QX, MV_Z, OP_MUL}},
+    {{MV_0, MV_Y, MV_0, OP_SUB}, {MV_1, MV_X, MV_1, OP_SUB}},
+    {{MV_2, MV_0, MV_0, OP_MUL}, {MV_3, MV_1, MV_1, OP_MUL}, {MV_4, MV_0, MV_QX, OP_MUL}, {MV_5, MV_1, MV_QY, OP_MUL},
+     {MV_L0, MV_1, MV_YP, OP_MUL}},
+    {{MV_L3, MV_4, MV_5, OP_SUB}},
+    {{MV_4, MV_1, MV_3, OP_MUL}, {MV_5, MV_Z, MV_2, OP_MUL}, {MV_6, MV_X, MV_3, OP_MUL}, {MV_L1, MV_0, MV_XN, OP_MUL}},
+    {{MV_7, MV_4, MV_5, OP_ADD}, {MV_8, MV_6, MV_6, OP_ADD}},
+    {{MV_7, MV_7, MV_8, OP_SUB}},
+    {{MV_8, MV_6, MV_7, OP_SUB}},
+    {{MV_X, MV_1, MV_7, OP_MUL}, {MV_2, MV_0, MV_8, OP_MUL}, {MV_3, MV_4, MV_Y, OP_MUL}, {MV_Z, MV_Z, MV_4, OP_MUL}},
+    {{MV_Y, MV_2, MV_3, OP_SUB}},
+};
+
+// one round on the calling warp: every lane calls; rounds are uniform in kind
+__device__ __forceinline__ void miller_round(Fp2* V, const MillerOp* ops) {
+  const int lane = threadIdx.x & 31, s = lane >> 1, part = lane & 1;
+  const MillerOp o = ops[s < MILLER_OPS ? s : 0];
+  const bool mul = ops[0].op == OP_MUL;
+  const Fp* const A = &V[o.a].c0;
+  const Fp* const B = &V[o.b].c0;
+  Fp r;
+  if (mul) {
+    const Fp a0 = ld_field(A), a1 = ld_field(A + 1), b0 = ld_field(B + part), b1 = ld_field(B + 1 - part);
+    Fp n1 = f_comp(a1);
+#pragma unroll
+    for (int l = 0; l < 8; l++) n1.v[l] = part ? a1.v[l] : n1.v[l];
+    r = f_mul2(a0, b0, n1, b1);
+  } else {
+    const Fp x = ld_field(A + part), y = ld_field(B + part);
+    const Fp add = f_add(x, y), sub = f_sub(x, y);
+#pragma unroll
+    for (int l = 0; l < 8; l++) r.v[l] = o.op == OP_ADD ? add.v[l] : sub.v[l];
+  }
+  __syncwarp();
+  if (s < MILLER_OPS && o.op != OP_NONE) st_field(&V[o.dst].c0 + part, r);
+  __syncwarp();
+}
+
+struct alignas(16) MillerShared {
+  E12 f, line[2];
+  Fp2 V[MV_COUNT];
+  Fp2 Q[2], nQy;   // Q, -yQ
+  Fp2 Q1[2], Q2[2];  // pi(Q), -pi^2(Q)
+};
+
+// steps of the loop: for each digit below the top a doubling (0), then +-Q (1, 2) where the
+// digit is not zero, then pi(Q) (3) and -pi^2(Q) (4)
+struct AteSteps {
+  uint8_t k[96];
+  int n;
+};
+constexpr AteSteps ate_steps() {
+  AteSteps s{};
+  const Naf d = naf_digits(6ull * BN_U + 2ull, true);
+  for (int i = d.n - 2; i >= 0; i--) {
+    s.k[s.n++] = 0;
+    if (d.d[i]) s.k[s.n++] = d.d[i] > 0 ? 1 : 2;
+  }
+  s.k[s.n++] = 3;
+  s.k[s.n++] = 4;
+  return s;
+}
+__device__ constexpr AteSteps ATE_STEPS = ate_steps();
+
+// f_(6u+2, Q)(P) with the two closing additions into sh->f, by a block of PAIR_BT threads; P,
+// Q affine (Montgomery), one at infinity: one.  Returns (to every thread of the fourth warp)
+// whether [6u + 2]Q + pi(Q) - pi^2(Q) = -pi^3(Q): as pi satisfies X^2 - t X + p on the twist
+// and the norm of X^3 - X^2 + X + 6u + 2 modulo that polynomial is r times a number prime to
+// the twist's order (checked by the tests), the equation holds exactly for the points of
+// order r.  (An addition that meets T = +-Q or O, which no point of order r does, leaves
+// Z = 0 for good, and the test fails.)
+__device__ __forceinline__ bool miller_loop(MillerShared* sh, const G1A& P, const G2A& Q, const FrobTab* T) {
+  const int t = threadIdx.x, warp = t >> 5;
+  Fp2* const V = sh->V;
+  f12_set_one(&sh->f);
+  if (t < 24) st_field(&sh->line[t / 12].c[t % 12], Fp::zero());
+  if (P.is_inf() || Q.is_inf()) {
+    __syncthreads();
+    return true;
+  }
+  if (t == 96) {
+    V[MV_X] = Q.x;
+    V[MV_Y] = Q.y;
+    V[MV_Z] = Fp2::one();
+    V[MV_XN] = {f_neg(P.x), Fp::zero()};
+    V[MV_YP] = {P.y, Fp::zero()};
+    V[MV_B3] = T->b3;
+    sh->Q[0] = Q.x;
+    sh->Q[1] = Q.y;
+    sh->nQy = f_neg(Q.y);
+    // pi(Q) = (conj(x) xi^((p-1)/3), conj(y) xi^((p-1)/2)), pi^2(Q) = (x xi^((p^2-1)/3), y xi^((p^2-1)/2))
+    sh->Q1[0] = f_mul(f2_conj(Q.x), T->g[0][2]);
+    sh->Q1[1] = f_mul(f2_conj(Q.y), T->g[0][3]);
+    sh->Q2[0] = f_mul(Q.x, T->g[1][2]);
+    sh->Q2[1] = f_neg(f_mul(Q.y, T->g[1][3]));
+  }
+  __syncthreads();
+  const int n = ATE_STEPS.n;
+  for (int s = 0; s <= n; s++) {
+    if (warp == 3) {  // the point warp, one step ahead
+      if (s < n) {
+        const int k = ATE_STEPS.k[s], lane = t & 31;
+        if (k) {
+          if (lane < 4) {
+            const Fp2* const q = k == 3 ? sh->Q1 : k == 4 ? sh->Q2 : sh->Q;
+            const Fp2* const y = k == 2 ? &sh->nQy : q + 1;
+            const Fp* const src = lane < 2 ? &q->c0 : &y->c0;
+            st_field(&V[lane < 2 ? MV_QX : MV_QY].c0 + (lane & 1), ld_field(src + (lane & 1)));
+          }
+          __syncwarp();
+          for (const auto& r : MILLER_ADD) miller_round(V, r);
+        } else {
+          for (const auto& r : MILLER_DBL) miller_round(V, r);
+        }
+        E12* const L = &sh->line[s & 1];
+        if (lane < 6) {  // l0, l1 w, l3 w^3
+          const int c = lane >> 1, part = lane & 1;
+          st_field(&L->c[(c == 2 ? 6 : 2 * c) + part], ld_field(&V[MV_L0 + c].c0 + part));
+        }
+      }
+    } else if (s > 0) {
+      if (s > 1 && ATE_STEPS.k[s - 1] == 0) f12_mul(&sh->f, &sh->f, &sh->f);
+      f12_mul(&sh->f, &sh->f, &sh->line[(s - 1) & 1]);
+    }
+    __syncthreads();
+  }
+  if (warp != 3) return true;
+  // T = -pi^3(Q) = (conj(x) xi^((p^3-1)/3), -conj(y) xi^((p^3-1)/2))?
+  if ((t & 31) == 0) {
+    V[MV_0] = f_mul(f_mul(f2_conj(Q.x), T->g[2][2]), V[MV_Z]);
+    V[MV_1] = f_neg(f_mul(f_mul(f2_conj(Q.y), T->g[2][3]), V[MV_Z]));
+  }
+  __syncwarp();
+  return V[MV_0] == V[MV_X] && V[MV_1] == V[MV_Y] && !V[MV_Z].is_zero();
 }
 
 }  // namespace zkvc

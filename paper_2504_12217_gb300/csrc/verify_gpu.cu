@@ -5,10 +5,10 @@
 // checked as e(-A, B) e(alpha, beta) e(IC(x), gamma) e(C, delta) = 1 with one shared final
 // exponentiation per proof.  IC(x) for every proof comes from one merged multi-output MSM
 // (each output reads its own verifying key's IC points; X int8 and Y int32 scalars in 8-bit
-// windows); each (proof, pair) gets a thread for its Miller loop; a last kernel multiplies a
-// proof's four Miller values and runs the final exponentiation.  Proof points are checked
-// as the host verifier checks them: canonical coordinates, on the curve, and B in the
-// order-r subgroup ([r] B = O, a 254-bit multiplication on the twist).
+// windows); each (proof, pair) gets a block for its Miller loop; a last kernel multiplies a
+// proof's four Miller values and runs the final exponentiation, a block per proof.  Proof
+// points are checked as the host verifier checks them: canonical coordinates, on the curve,
+// and B in the order-r subgroup (from its Miller loop's last point, pairing.cuh).
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -56,6 +56,8 @@ __global__ void k_frob_init(FrobTab* T) {
       acc = f_mul(acc, base[k]);
     }
   }
+  T->b = g2_b();
+  T->b3 = f_add(f_dbl(T->b), T->b);
 }
 
 static std::mutex g_frob_mu;
@@ -118,25 +120,24 @@ __device__ __forceinline__ G2A ld_g2(const uint8_t* p, int* ok) {
   return {{f_to_mont(a), f_to_mont(b)}, {f_to_mont(c), f_to_mont(d)}};
 }
 
-__device__ __forceinline__ void st_f12(uint8_t* out, const Fp12& f) {
-  const Fp2* c[6] = {&f.c0.c0, &f.c0.c1, &f.c0.c2, &f.c1.c0, &f.c1.c1, &f.c1.c2};
-  for (int j = 0; j < 6; j++) {
-    st_canon(out + 64 * j, c[j]->c0);
-    st_canon(out + 64 * j + 32, c[j]->c1);
-  }
-}
-
-// e(P_i, Q_i) for canonical points; out: 12 canonical Fp coefficients per pairing in tower
-// order (c0.c0, c0.c1, c0.c2, c1.c0, c1.c1, c1.c2; each Fp2 as c0 then c1)
-__global__ void __launch_bounds__(64) k_pairing(const uint8_t* __restrict__ P, const uint8_t* __restrict__ Q, size_t n,
-                                                const FrobTab* __restrict__ T, uint8_t* out) {
-  size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// e(P_i, Q_i) for canonical points, a block each; out: 12 canonical Fp coefficients per
+// pairing in tower order (c0.c0, c0.c1, c0.c2, c1.c0, c1.c1, c1.c2 = w^0, 2, 4, 1, 3, 5; each
+// Fp2 as c0 then c1)
+__global__ void __launch_bounds__(PAIR_BT) k_pairing(const uint8_t* __restrict__ P, const uint8_t* __restrict__ Q,
+                                                     const FrobTab* __restrict__ T, uint8_t* out) {
+  __shared__ MillerShared sh;
+  __shared__ FinalScratch fs;
+  const size_t i = blockIdx.x;
   int ok = 1;
-  G1A p = ld_g1(P + 64 * i, &ok);
-  G2A q = ld_g2(Q + 128 * i, &ok);
-  FrobTab t = *T;
-  st_f12(out + 384 * i, final_exp(miller_loop(p, q, t), t));
+  const G1A p = ld_g1(P + 64 * i, &ok);
+  const G2A q = ld_g2(Q + 128 * i, &ok);
+  miller_loop(&sh, p, q, T);
+  if (threadIdx.x >= PAIR_F) return;
+  final_exp(&sh.f, &fs, T);
+  if (threadIdx.x < 12) {
+    const int j = threadIdx.x >> 1, m = j < 3 ? 2 * j : 2 * j - 5;
+    st_canon(out + 384 * i + 32 * threadIdx.x, ld_field(&sh.f.c[2 * m + (threadIdx.x & 1)]));
+  }
 }
 
 // ------------------------------------------------------------------ batched verification
@@ -154,7 +155,7 @@ struct VfyItem {
 };
 
 __global__ void k_vfy_load(const uint8_t* __restrict__ proofs, const int* __restrict__ vk_of, const VkDev* __restrict__ vks,
-                           int count, VfyItem* items) {
+                           int count, const FrobTab* __restrict__ T, VfyItem* items) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= count) return;
   const uint8_t* pr = proofs + 256 * size_t(t);
@@ -162,7 +163,7 @@ __global__ void k_vfy_load(const uint8_t* __restrict__ proofs, const int* __rest
   G1A A = ld_g1(pr, &ok);
   G2A B = ld_g2(pr + 64, &ok);
   G1A C = ld_g1(pr + 192, &ok);
-  if (ok && (!p_on_curve(A, g1_b()) || !p_on_curve(C, g1_b()) || !p_on_curve(B, g2_b()))) ok = 0;
+  if (ok && (!p_on_curve(A, g1_b()) || !p_on_curve(C, g1_b()) || !p_on_curve(B, T->b))) ok = 0;
   const VkDev& vk = vks[vk_of[t]];
   VfyItem it;
   it.P[0] = p_neg(A);
@@ -188,38 +189,45 @@ __global__ void k_vfy_ic(const int* __restrict__ vk_of, const VkDev* __restrict_
   items[t].P[2] = p_to_affine(acc);
 }
 
-// B in the order-r subgroup: [r] B = O
-__global__ void __launch_bounds__(64) k_vfy_subgroup(int count, VfyItem* items) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= count) return;
-  G2A B = items[t].Q[0];
-  if (B.is_inf() || !items[t].ok) return;
-  uint32_t r[8];
-#pragma unroll
-  for (int i = 0; i < 8; i++) r[i] = mod_limb<FrCfg>(i);
-  if (!p_mul_scalar_w4(G2J::from_affine(B), r).is_inf()) items[t].ok = 0;
+// a block per (proof, pair); the block of pair 0 also decides whether B has order r
+__global__ void __launch_bounds__(PAIR_BT) k_vfy_miller(const VfyItem* __restrict__ items,
+                                                        const FrobTab* __restrict__ T, E12* f, int* in_group) {
+  __shared__ MillerShared sh;
+  const int i = blockIdx.x >> 2, k = blockIdx.x & 3;
+  if (!items[i].ok) return;
+  G1A P = items[i].P[k];
+  const G2A Q = items[i].Q[k];
+  // A at infinity would skip the loop, and with it B's test: run it on any other coordinates
+  const bool skip = k == 0 && P.is_inf();
+  if (skip) P = {Fp::one(), Fp::one()};
+  const bool sub = miller_loop(&sh, P, Q, T);
+  if (k == 0 && threadIdx.x == 96) in_group[i] = sub;
+  if (skip) f12_set_one(&sh.f);
+  __syncthreads();
+  if (threadIdx.x < 12) st_field(&f[blockIdx.x].c[threadIdx.x], ld_field(&sh.f.c[threadIdx.x]));
 }
 
-__global__ void __launch_bounds__(64) k_vfy_miller(const VfyItem* __restrict__ items, int count,
-                                                   const FrobTab* __restrict__ T, Fp12* f) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 4 * count) return;
-  const int i = t >> 2, k = t & 3;
-  FrobTab tab = *T;
-  f[t] = items[i].ok ? miller_loop(items[i].P[k], items[i].Q[k], tab) : f12_one();
-}
-
-__global__ void __launch_bounds__(64) k_vfy_final(const VfyItem* __restrict__ items, const Fp12* __restrict__ f, int count,
-                                                  const FrobTab* __restrict__ T, int* ok) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= count) return;
-  if (!items[t].ok) {
-    ok[t] = 0;
+__global__ void __launch_bounds__(PAIR_F) k_vfy_final(const VfyItem* __restrict__ items, const E12* __restrict__ f,
+                                                      const int* __restrict__ in_group, const FrobTab* __restrict__ T,
+                                                      int* ok) {
+  __shared__ E12 g[4];
+  __shared__ FinalScratch fs;
+  const int i = blockIdx.x, t = threadIdx.x;
+  if (!items[i].ok || !in_group[i]) {
+    if (t == 0) ok[i] = 0;
     return;
   }
-  FrobTab tab = *T;
-  Fp12 g = f12_mul(f12_mul(f[4 * t], f[4 * t + 1]), f12_mul(f[4 * t + 2], f[4 * t + 3]));
-  ok[t] = f12_is_one(final_exp(g, tab)) ? 1 : 0;
+  if (t < 48) st_field(&g[t / 12].c[t % 12], ld_field(&f[4 * i + t / 12].c[t % 12]));
+  f12_bar();
+  f12_mul(g, g, g + 1);
+  f12_mul(g + 2, g + 2, g + 3);
+  f12_mul(g, g, g + 2);
+  final_exp(g, &fs, T);
+  const bool one = t >= 12 || ld_field(&g->c[t]) == (t == 0 ? Fp::one() : Fp::zero());
+  if (t < 32) {
+    const bool all = __all_sync(0xffffffffu, one);
+    if (t == 0) ok[i] = all ? 1 : 0;
+  }
 }
 
 __global__ void k_canon_to_mont_g1(G1A* p, size_t n) {
@@ -367,24 +375,24 @@ int verify_batch_impl(const zkvc_vk* const* vks, const int8_t* const* X, const i
   }
   // points, IC, subgroup, Miller loops, final exponentiations
   uint8_t* d_proofs = nullptr;
-  int *d_vk_of = nullptr, *d_slot = nullptr, *d_ok = nullptr;
+  int *d_vk_of = nullptr, *d_slot = nullptr, *d_ok = nullptr, *d_group = nullptr;
   VfyItem* d_items = nullptr;
-  Fp12* d_f = nullptr;
+  E12* d_f = nullptr;
   ZK_TRY(buf.get(&d_proofs, size_t(count) * 256));
   ZK_TRY(buf.get(&d_vk_of, count));
   ZK_TRY(buf.get(&d_slot, count));
   ZK_TRY(buf.get(&d_ok, count));
+  ZK_TRY(buf.get(&d_group, count));
   ZK_TRY(buf.get(&d_items, count));
   ZK_TRY(buf.get(&d_f, 4 * size_t(count)));
   ZK_CUDA(cudaMemcpyAsync(d_proofs, proofs, size_t(count) * 256, cudaMemcpyHostToDevice, st));
   ZK_CUDA(cudaMemcpyAsync(d_vk_of, vk_of.data(), count * sizeof(int), cudaMemcpyHostToDevice, st));
   ZK_CUDA(cudaMemcpyAsync(d_slot, slot.data(), count * sizeof(int), cudaMemcpyHostToDevice, st));
   const unsigned g = (unsigned)((count + 63) / 64);
-  k_vfy_load<<<g, 64, 0, st>>>(d_proofs, d_vk_of, d_vk, count, d_items); ZK_COUNT_LAUNCH();
+  k_vfy_load<<<g, 64, 0, st>>>(d_proofs, d_vk_of, d_vk, count, T, d_items); ZK_COUNT_LAUNCH();
   k_vfy_ic<<<g, 64, 0, st>>>(d_vk_of, d_vk, d_slot, d_msm, count, d_items); ZK_COUNT_LAUNCH();
-  k_vfy_subgroup<<<g, 64, 0, st>>>(count, d_items); ZK_COUNT_LAUNCH();
-  k_vfy_miller<<<(unsigned)((4 * count + 63) / 64), 64, 0, st>>>(d_items, count, T, d_f); ZK_COUNT_LAUNCH();
-  k_vfy_final<<<g, 64, 0, st>>>(d_items, d_f, count, T, d_ok); ZK_COUNT_LAUNCH();
+  k_vfy_miller<<<4 * (unsigned)count, PAIR_BT, 0, st>>>(d_items, T, d_f, d_group); ZK_COUNT_LAUNCH();
+  k_vfy_final<<<(unsigned)count, PAIR_F, 0, st>>>(d_items, d_f, d_group, T, d_ok); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   ZK_CUDA(cudaMemcpyAsync(ok, d_ok, count * sizeof(int), cudaMemcpyDeviceToHost, st));
   ZK_TRY(wait_stream(st, "verify_batch"));
@@ -396,7 +404,7 @@ int pairing_impl(const uint8_t* d_P, const uint8_t* d_Q, size_t n, uint8_t* d_ou
   ZK_CHECK(d_P && d_Q && d_out, ZKVC_EINVAL, "pairing: null pointer");
   const FrobTab* T = nullptr;
   ZK_TRY(frob_table(&T, st));
-  k_pairing<<<(unsigned)((n + 63) / 64), 64, 0, st>>>(d_P, d_Q, n, T, d_out); ZK_COUNT_LAUNCH();
+  k_pairing<<<(unsigned)n, PAIR_BT, 0, st>>>(d_P, d_Q, T, d_out); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   return ZKVC_OK;
 }
