@@ -657,7 +657,7 @@ int zkvc_ntt(uint8_t* d_data, uint32_t log_n, int kind, void* stream) {
   int load_scale = kind == ZKVC_NTT_COSET_FORWARD ? SC_G : SC_NONE;
   int out_scale = kind == ZKVC_NTT_INVERSE ? SC_N : (kind == ZKVC_NTT_COSET_INVERSE ? SC_NGI : SC_NONE);
   ZK_TRY(ntt_dif(x, 1, 0, d, inverse, load_scale, SC_NONE, true, st));
-  ZK_TRY(ntt_bitrev(x, d, out_scale, true, st));
+  ZK_TRY(ntt_bitrev(x, d, out_scale, st));
   return ZKVC_OK;
 }
 

@@ -54,6 +54,12 @@ constexpr U256c cx_pow2_mod(int k, U256c m) {
   return x;
 }
 
+constexpr U256c cx_twice(U256c x) {  // 2x below 2^256
+  U256c r{};
+  for (int i = 0; i < 8; i++) r.w[i] = (x.w[i] << 1) | (i ? x.w[i - 1] >> 31 : 0u);
+  return r;
+}
+
 constexpr uint32_t cx_neg_inv32(uint32_t m0) {
   uint32_t x = m0;  // Newton iteration for m0^-1 mod 2^32 (m0 odd)
   for (int i = 0; i < 5; i++) x = x * (2u - m0 * x);
@@ -65,6 +71,7 @@ constexpr uint32_t cx_neg_inv32(uint32_t m0) {
 struct FpCfg {
   static constexpr U256c MOD = {{0xd87cfd47u, 0x3c208c16u, 0x6871ca8du, 0x97816a91u,
                                  0x8181585du, 0xb85045b6u, 0xe131a029u, 0x30644e72u}};
+  static constexpr U256c MOD2 = cx_twice(MOD);
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
@@ -73,6 +80,7 @@ struct FpCfg {
 struct FrCfg {
   static constexpr U256c MOD = {{0xf0000001u, 0x43e1f593u, 0x79b97091u, 0x2833e848u,
                                  0x8181585du, 0xb85045b6u, 0xe131a029u, 0x30644e72u}};
+  static constexpr U256c MOD2 = cx_twice(MOD);
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
@@ -92,6 +100,8 @@ struct FrCfg {
 
 template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t mod_limb(int i) { ZKVC_LIMB_SWITCH(C::MOD, i) }
+template <class C>
+__host__ __device__ __forceinline__ constexpr uint32_t mod2_limb(int i) { ZKVC_LIMB_SWITCH(C::MOD2, i) }
 template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t r1_limb(int i) { ZKVC_LIMB_SWITCH(C::R1, i) }
 template <class C>
@@ -537,12 +547,12 @@ __device__ __forceinline__ Field<C> f_once(const Field<C>& r) {
   return br ? r : d;
 }
 
-// Montgomery product a b R^-1 mod N for a < 2N and any b < 2^256: after each row the state
-// is below a + N < 2^256 and before the division below 2^288, so nothing leaves limb 8; the
-// result is below a b / R + N < 2N for b < 2N, and for any b where a < N.  (Values that may
-// exceed N come second: f_to_mont reduces an arbitrary 256-bit value.)
+// Montgomery product a b R^-1 mod N, not brought below N.  For a <= 4N and any b < 2^256:
+// after each row the state is below a + N <= 5N < 2^256 and before the division below
+// 2^288, so nothing leaves limb 8; the result is below a b / R + N: below 2N for a < 4N and
+// b < N, for a, b < 2N, and for a < N and any b.
 template <class C>
-__device__ __forceinline__ Field<C> f_mul(const Field<C>& a, const Field<C>& b) {
+__device__ __forceinline__ Field<C> f_mul_lazy(const Field<C>& a, const Field<C>& b) {
   uint32_t e[8], o[8], pend;
   eo::mul4(e, a.v, 0, b.v[0]);
   eo::mul4(o, a.v, 1, b.v[0]);
@@ -557,7 +567,42 @@ __device__ __forceinline__ Field<C> f_mul(const Field<C>& a, const Field<C>& b) 
   }
   Field<C> r;
   eo::merge(r.v, e, o, pend);
-  return f_once(r);
+  return r;
+}
+
+// the product below N, for operands whose lazy product is below 2N.  (Values that may exceed
+// N come second: f_to_mont reduces an arbitrary 256-bit value.)
+template <class C>
+__device__ __forceinline__ Field<C> f_mul(const Field<C>& a, const Field<C>& b) {
+  return f_once(f_mul_lazy(a, b));
+}
+
+// Lazy butterfly arithmetic: x < 4N brought below 2N; a + b below 2N and a - b + 2N below 4N
+// for a, b < 2N
+template <class C>
+__device__ __forceinline__ Field<C> f_red2(const Field<C>& x) {
+  Field<C> m, d;
+#pragma unroll
+  for (int i = 0; i < 8; i++) m.v[i] = mod2_limb<C>(i);
+  const uint32_t br = sub8(d.v, x.v, m.v);
+  return br ? x : d;
+}
+template <class C>
+__device__ __forceinline__ Field<C> f_add_raw(const Field<C>& a, const Field<C>& b) {
+  Field<C> s;
+  add8(s.v, a.v, b.v);
+  return s;
+}
+template <class C>
+__device__ __forceinline__ Field<C> f_add2(const Field<C>& a, const Field<C>& b) { return f_red2(f_add_raw(a, b)); }
+template <class C>
+__device__ __forceinline__ Field<C> f_sub2(const Field<C>& a, const Field<C>& b) {
+  Field<C> m, s, d;
+#pragma unroll
+  for (int i = 0; i < 8; i++) m.v[i] = mod2_limb<C>(i);
+  add8(s.v, a.v, m.v);
+  sub8(d.v, s.v, b.v);
+  return d;
 }
 
 // (a b + c d) R^-1 mod N with one reduction, for operands up to N: the state stays below
@@ -695,6 +740,27 @@ __device__ __noinline__ Field<C> f_sqrc(Field<C> a) {
 template <class C>
 __device__ __noinline__ Field<C> f_mul2c(Field<C> a, Field<C> b, Field<C> c, Field<C> d) {
   return f_mul2(a, b, c, d);
+}
+
+// t < 64 N (nine limbs) mod N: the quotient from the top bits, at most one short (both
+// moduli begin with the same bits: N / 2^240 lies in (12388, 12389))
+template <class C>
+__device__ __forceinline__ Field<C> f_mod9(const uint32_t (&t)[9]) {
+  static_assert(C::MOD.w[7] >> 16 == 12388, "the quotient estimate's divisor");
+  const uint32_t h = (t[7] >> 16) | (t[8] << 16);  // t / 2^240 < 2^20
+  const uint32_t q = __umulhi(h, 346675u);         // 2^32 / 12389
+  uint32_t p[8];
+  Field<C> r, x;
+  uint64_t c = 0;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    c += (uint64_t)q * mod_limb<C>(i);
+    p[i] = (uint32_t)c;
+    c >>= 32;
+    x.v[i] = t[i];
+  }
+  sub8(r.v, x.v, p);  // below 2N: the ninth limbs cancel
+  return f_once(r);
 }
 
 // a R mod N for any a < 2^256 (the second operand of f_mul may exceed N)

@@ -3,15 +3,15 @@
 // t(x) = x^N - 1 through evaluations on the coset gH).
 //
 // GB300 design: every pass takes k <= 10 consecutive radix-2 stages of one group of 2^k
-// elements, staged through shared memory in a limb-major (structure-of-arrays) layout
-// so that the 8 words of neighbouring elements fall in different banks.  A block holds
+// elements, staged through shared memory as two planes of 16-byte halves.  A block holds
 // G groups whose global indices differ in the low bits, so each global load or store of
 // the block touches G consecutive elements (G * 32 contiguous bytes).  N = 2^16 takes
 // two passes (two HBM round trips), N = 2^24 three.  Decimation in frequency maps
 // natural order to bit-reversed order and decimation in time maps it back, so the prove
 // path (INTT -> coset NTT -> pointwise -> coset INTT) never runs a bit-reversal pass:
 // the coset shift g^i and 1/N are applied at the bit-reversed store of the inverse
-// transforms.  Twiddles are read from a table omega^e (e < N/2), L2-resident for the
+// transforms.  The transform is linear and its twiddles are in Montgomery form, so data in
+// either form goes through unconverted.  Twiddles are read from a table omega^e (e < N/2), L2-resident for the
 // proof domains.
 #include <algorithm>
 #include <map>
@@ -157,81 +157,97 @@ static ScaleTabs tabs_of(const NttDomain* d) {
 }
 
 // One pass: k consecutive radix-2 stages from stage s0, over G = 2^logG groups of 2^k
-// elements per block (E = G 2^k elements, staged limb-major in shared memory).
+// elements per block (E = G 2^k elements, staged in shared memory as two planes of 16-byte
+// halves: an element is two vector accesses, and neighbouring elements are conflict-free).
 struct PassGeo {
   uint32_t L, s0, k, logG;
 };
 
-// global index of the block's e-th staged element
+// global index of the block's e-th staged element (N <= 2^28)
 template <bool DIT>
-__device__ __forceinline__ size_t pass_index(const PassGeo& g, size_t gid0, uint32_t e) {
-  const uint32_t G = 1u << g.logG;
-  const uint32_t gg = e & (G - 1), j = e >> g.logG;
-  const size_t gid = gid0 + gg;
+__device__ __forceinline__ uint32_t pass_index(const PassGeo& g, uint32_t gid0, uint32_t e) {
+  const uint32_t gg = e & ((1u << g.logG) - 1u), j = e >> g.logG;
+  const uint32_t gid = gid0 + gg;
   const uint32_t sbits = DIT ? g.s0 : (g.L - g.s0 - g.k);
-  const size_t lo = gid & ((size_t(1) << sbits) - 1), hi = gid >> sbits;
-  const size_t base = DIT ? ((hi << (g.s0 + g.k)) | lo) : ((hi << (g.L - g.s0)) | lo);
-  return base + (size_t(j) << sbits);
+  const uint32_t lo = gid & ((1u << sbits) - 1u), hi = gid >> sbits;
+  const uint32_t base = DIT ? ((hi << (g.s0 + g.k)) | lo) : ((hi << (g.L - g.s0)) | lo);
+  return base + (j << sbits);
 }
 
-__device__ __forceinline__ Fr sm_get(const uint32_t* sm, uint32_t E, uint32_t e) {
-  Fr x;
-#pragma unroll
-  for (int l = 0; l < 8; l++) x.v[l] = sm[l * E + e];
-  return x;
+__device__ __forceinline__ Fr sm_get(const uint4* sm, uint32_t E, uint32_t e) {
+  const uint4 a = sm[e], b = sm[E + e];
+  return {{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
 }
-__device__ __forceinline__ void sm_put(uint32_t* sm, uint32_t E, uint32_t e, const Fr& x) {
-#pragma unroll
-  for (int l = 0; l < 8; l++) sm[l * E + e] = x.v[l];
+__device__ __forceinline__ void sm_put(uint4* sm, uint32_t E, uint32_t e, const Fr& x) {
+  sm[e] = make_uint4(x.v[0], x.v[1], x.v[2], x.v[3]);
+  sm[E + e] = make_uint4(x.v[4], x.v[5], x.v[6], x.v[7]);
 }
 
+// What bounds a pass on a large grid: the products, at 0.74 of the multiplier's rate (289
+// instructions per warp of butterflies, 136 of them the product's multiply-adds; 405 with
+// eight scalar shared-memory accesses per element, full reductions and 64-bit indices).
+// Measured at 2^22, passes of 8 + 7 + 7 stages: 306 + 257 + 226 us (378 + 296 + 293 before);
+// the first is slower by its twiddles, whose table leaves L2 between stages.
+//
+// Values stay lazily reduced between loads and stores: below 2N in a decimation-in-frequency
+// pass, below 4N in a decimation-in-time pass, so a butterfly's product needs no
+// conditional subtraction and its sums one at most.  raw: the input is any 256-bit value.
 template <bool DIT>
-__device__ __forceinline__ void pass_load(const Fr* arr, const PassGeo& g, size_t gid0, uint32_t* sm, int load_scale,
-                                          int to_mont, const ScaleTabs& tabs) {
+__device__ __forceinline__ void pass_load(const Fr* arr, const PassGeo& g, uint32_t gid0, uint4* sm, int load_scale,
+                                          int raw, const ScaleTabs& tabs) {
   const uint32_t E = 1u << (g.logG + g.k);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-    const size_t idx = pass_index<DIT>(g, gid0, e);
+    const uint32_t idx = pass_index<DIT>(g, gid0, e);
     Fr x = ld_field(arr + idx);
-    if (to_mont) x = f_to_mont(x);
-    if (load_scale) x = f_mul(x, scale_factor(tabs, load_scale, (uint32_t)idx));
+    if (load_scale) {  // (the product reduces a raw value too)
+      x = f_mul_lazy(scale_factor(tabs, load_scale, idx), x);
+    } else if (raw) {
+      const uint32_t t[9] = {x.v[0], x.v[1], x.v[2], x.v[3], x.v[4], x.v[5], x.v[6], x.v[7], 0};
+      x = f_mod9<FrCfg>(t);
+    }
     sm_put(sm, E, e, x);
   }
 }
 
+// last: the transform's last pass, whose values go out below N
 template <bool DIT>
-__device__ __forceinline__ void pass_store(Fr* arr, const PassGeo& g, size_t gid0, const uint32_t* sm, int store_scale,
-                                           const ScaleTabs& tabs) {
+__device__ __forceinline__ void pass_store(Fr* arr, const PassGeo& g, uint32_t gid0, const uint4* sm, int store_scale,
+                                           bool last, const ScaleTabs& tabs) {
   const uint32_t E = 1u << (g.logG + g.k);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-    const size_t idx = pass_index<DIT>(g, gid0, e);
+    const uint32_t idx = pass_index<DIT>(g, gid0, e);
     Fr x = sm_get(sm, E, e);
-    if (store_scale) x = f_mul(x, scale_factor(tabs, store_scale, brev_bits((uint32_t)idx, g.L)));
+    if (store_scale) {
+      x = f_mul(scale_factor(tabs, store_scale, brev_bits(idx, g.L)), x);
+    } else if (last) {
+      if (DIT) x = f_red2(x);
+      x = f_once(x);
+    }
     st_field(arr + idx, x);
   }
 }
 
-// The pass's k stages on NPOLY staged arrays (8 E words apart).  Radix 2 (R4 false):
+// The pass's k stages on NPOLY staged arrays (2 E vectors apart).  Radix 2 (R4 false):
 // one stage per shared-memory round trip, one butterfly per element pair.  R4: two stages
 // at a time: a radix-4 unit reads four elements, runs their four butterflies of stages t
 // and t + 1 in registers (two independent products per stage) and writes them back, so a
 // pair of stages costs one round trip and one barrier instead of two; an odd last stage
-// runs as radix 2.  R4 holds more registers (112 against 64: two blocks of 256 per SM
-// instead of four), which pays where the grid is too small to fill the GPU (the latency of
-// a thread's serial stages decides) and costs a few per cent where it is large.  Barriers
-// between rounds (the first one orders the loads before it).
+// runs as radix 2.  Barriers between rounds (the first one orders the loads before it).
 //   DIF, stage t of half h (block 2h), then h/2: a unit is j0 = blk 2h + off (off < h/2)
 //     and j0 + h/2, j0 + h, j0 + 3h/2; twiddles w_t(off), w_t(off + h/2), w_(t+1)(off).
 //   DIT, stage t of half h (block 2h), then 2h: a unit is j0 = blk 4h + off (off < h) and
 //     j0 + h, j0 + 2h, j0 + 3h; twiddles w_t(off), w_(t+1)(off), w_(t+1)(off + h).
 // w_t(q) is the table entry of the radix-2 form: DIF ((q << sbits) + lo) << s, DIT
-// ((q << s0) + lo) << (L - 1 - s), lo the group's low index bits, s = s0 + t.
+// ((q << s0) + lo) << (L - 1 - s), lo the group's low index bits, s = s0 + t.  The
+// transform's stage of half 1 over neighbouring elements (DIF s = L - 1, DIT s = 0) has
+// w = 1 throughout and takes no product.
 template <bool DIT, int NPOLY, bool R4>
-__device__ __forceinline__ void pass_stages(uint32_t* sm, const PassGeo& g, size_t gid0, const Fr* tw) {
+__device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_t gid0, const Fr* tw) {
   const uint32_t G = 1u << g.logG, E = G << g.k, L = g.L, logG = g.logG;
   const uint32_t sbits = DIT ? g.s0 : (L - g.s0 - g.k);
-  const size_t smask = (size_t(1) << sbits) - 1;
-  auto twi = [&](uint32_t s, uint32_t q, size_t lo) -> size_t {
-    return DIT ? ((((size_t)q << g.s0) + lo) << (L - 1 - s)) : ((((size_t)q << sbits) + lo) << s);
+  const uint32_t smask = (1u << sbits) - 1u;
+  auto twi = [&](uint32_t s, uint32_t q, uint32_t lo) -> const Fr* {
+    return tw + (DIT ? (((q << g.s0) + lo) << (L - 1 - s)) : (((q << sbits) + lo) << s));
   };
   __syncthreads();
   uint32_t t = 0;
@@ -240,39 +256,62 @@ __device__ __forceinline__ void pass_stages(uint32_t* sm, const PassGeo& g, size
     const uint32_t s = g.s0 + t;
     for (uint32_t ua = threadIdx.x; ua < nq * (uint32_t)NPOLY; ua += blockDim.x) {
       const uint32_t poly = NPOLY == 1 ? 0u : ua / nq, u = ua - poly * nq;
-      uint32_t* smp = sm + size_t(poly) * 8 * E;
+      uint4* smp = sm + size_t(poly) * 2 * E;
       const uint32_t gg = u & (G - 1), q = u >> logG;
-      const size_t lo = (gid0 + gg) & smask;
+      const uint32_t lo = (gid0 + gg) & smask;
       if (DIT) {
         const uint32_t lh = t, h = 1u << lh;  // stage t: half h; stage t + 1: half 2h
         const uint32_t off = q & (h - 1), j0 = ((q >> lh) << (lh + 2)) + off;
         const uint32_t p0 = (j0 << logG) + gg, p1 = ((j0 + h) << logG) + gg, p2 = ((j0 + 2 * h) << logG) + gg,
                        p3 = ((j0 + 3 * h) << logG) + gg;
-        const Fr w0 = ld_field(tw + twi(s, off, lo));
-        Fr x0 = sm_get(smp, E, p0), x1 = sm_get(smp, E, p1), x2 = sm_get(smp, E, p2), x3 = sm_get(smp, E, p3);
-        x1 = f_mul(x1, w0);
-        x3 = f_mul(x3, w0);
-        const Fr a = f_add(x0, x1), b = f_sub(x0, x1), c = f_add(x2, x3), d = f_sub(x2, x3);
-        const Fr w1 = ld_field(tw + twi(s + 1, off, lo)), w2 = ld_field(tw + twi(s + 1, off + h, lo));
-        const Fr vc = f_mul(c, w1), vd = f_mul(d, w2);
-        sm_put(smp, E, p0, f_add(a, vc));
-        sm_put(smp, E, p2, f_sub(a, vc));
-        sm_put(smp, E, p1, f_add(b, vd));
-        sm_put(smp, E, p3, f_sub(b, vd));
+        Fr x1 = sm_get(smp, E, p1), x3 = sm_get(smp, E, p3);
+        if (s == 0) {
+          x1 = f_red2(x1);
+          x3 = f_red2(x3);
+        } else {
+          const Fr w0 = ld_field(twi(s, off, lo));
+          x1 = f_mul_lazy(x1, w0);
+          x3 = f_mul_lazy(x3, w0);
+        }
+        const Fr x0 = f_red2(sm_get(smp, E, p0)), x2 = f_red2(sm_get(smp, E, p2));
+        const Fr vc = f_mul_lazy(f_add_raw(x2, x3), ld_field(twi(s + 1, off, lo)));
+        const Fr a = f_red2(f_add_raw(x0, x1));
+        sm_put(smp, E, p0, f_add_raw(a, vc));
+        sm_put(smp, E, p2, f_sub2(a, vc));
+        const Fr vd = f_mul_lazy(f_sub2(x2, x3), ld_field(twi(s + 1, off + h, lo)));
+        const Fr b = f_red2(f_sub2(x0, x1));
+        sm_put(smp, E, p1, f_add_raw(b, vd));
+        sm_put(smp, E, p3, f_sub2(b, vd));
       } else {
         const uint32_t lh = g.k - 1 - t, h = 1u << lh, hq = h >> 1;  // stage t: half h; t + 1: h/2
         const uint32_t off = q & (hq - 1), j0 = ((q >> (lh - 1)) << (lh + 1)) + off;
         const uint32_t p0 = (j0 << logG) + gg, p1 = ((j0 + hq) << logG) + gg, p2 = ((j0 + h) << logG) + gg,
                        p3 = ((j0 + h + hq) << logG) + gg;
-        const Fr w0 = ld_field(tw + twi(s, off, lo)), w1 = ld_field(tw + twi(s, off + hq, lo));
-        const Fr x0 = sm_get(smp, E, p0), x1 = sm_get(smp, E, p1), x2 = sm_get(smp, E, p2), x3 = sm_get(smp, E, p3);
-        const Fr a = f_add(x0, x2), b = f_mul(f_sub(x0, x2), w0);
-        const Fr c = f_add(x1, x3), d = f_mul(f_sub(x1, x3), w1);
-        const Fr w2 = ld_field(tw + twi(s + 1, off, lo));
-        sm_put(smp, E, p0, f_add(a, c));
-        sm_put(smp, E, p1, f_mul(f_sub(a, c), w2));
-        sm_put(smp, E, p2, f_add(b, d));
-        sm_put(smp, E, p3, f_mul(f_sub(b, d), w2));
+        Fr a, b, c, d;
+        {
+          const Fr x0 = sm_get(smp, E, p0), x2 = sm_get(smp, E, p2);
+          a = f_add2(x0, x2);
+          b = f_mul_lazy(f_sub2(x0, x2), ld_field(twi(s, off, lo)));
+        }
+        {
+          const Fr x1 = sm_get(smp, E, p1), x3 = sm_get(smp, E, p3);
+          c = f_add2(x1, x3);
+          d = f_mul_lazy(f_sub2(x1, x3), ld_field(twi(s, off + hq, lo)));
+        }
+        sm_put(smp, E, p0, f_add2(a, c));
+        sm_put(smp, E, p2, f_add2(b, d));
+        a = f_sub2(a, c);
+        b = f_sub2(b, d);
+        if (s + 1 == L - 1) {
+          a = f_red2(a);
+          b = f_red2(b);
+        } else {
+          const Fr w2 = ld_field(twi(s + 1, off, lo));
+          a = f_mul_lazy(a, w2);
+          b = f_mul_lazy(b, w2);
+        }
+        sm_put(smp, E, p1, a);
+        sm_put(smp, E, p3, b);
       }
     }
     __syncthreads();
@@ -280,44 +319,47 @@ __device__ __forceinline__ void pass_stages(uint32_t* sm, const PassGeo& g, size
   for (; t < g.k; t++) {  // radix 2: every stage, or the last of an odd count
     const uint32_t s = g.s0 + t, nbf = E >> 1;
     const uint32_t logh = DIT ? t : (g.k - 1 - t), h = 1u << logh;
+    const bool unit = DIT ? s == 0 : s == L - 1;
     for (uint32_t bfa = threadIdx.x; bfa < nbf * (uint32_t)NPOLY; bfa += blockDim.x) {
       const uint32_t poly = NPOLY == 1 ? 0u : bfa / nbf, bf = bfa - poly * nbf;
-      uint32_t* smp = sm + size_t(poly) * 8 * E;
+      uint4* smp = sm + size_t(poly) * 2 * E;
       const uint32_t gg = bf & (G - 1), q = bf >> logG;
       const uint32_t qh = q & (h - 1);
       const uint32_t ju = ((q >> logh) << (logh + 1)) + qh;
       const uint32_t pu = (ju << logG) + gg, pv = ((ju + h) << logG) + gg;
-      const size_t lo = (gid0 + gg) & smask;
-      const Fr w = ld_field(tw + twi(s, qh, lo));
-      Fr u = sm_get(smp, E, pu), v = sm_get(smp, E, pv);
-      Fr a, b;
+      const uint32_t lo = (gid0 + gg) & smask;
+      const Fr u = sm_get(smp, E, pu), v = sm_get(smp, E, pv);
       if (DIT) {
-        v = f_mul(v, w);
-        a = f_add(u, v);
-        b = f_sub(u, v);
+        const Fr x = f_red2(u), y = unit ? f_red2(v) : f_mul_lazy(v, ld_field(twi(s, qh, lo)));
+        sm_put(smp, E, pu, f_add_raw(x, y));
+        sm_put(smp, E, pv, f_sub2(x, y));
       } else {
-        a = f_add(u, v);
-        b = f_mul(f_sub(u, v), w);
+        sm_put(smp, E, pu, f_add2(u, v));
+        const Fr d = f_sub2(u, v);
+        sm_put(smp, E, pv, unit ? f_red2(d) : f_mul_lazy(d, ld_field(twi(s, qh, lo))));
       }
-      sm_put(smp, E, pu, a);
-      sm_put(smp, E, pv, b);
     }
     __syncthreads();
   }
 }
 
+// Resident blocks the registers are cut to: radix 2 at 64 registers (32 warps per SM, the
+// large grids), radix 4 at 128 (the small ones, which have fewer blocks than that).
+template <bool R4>
+constexpr int pass_min_blocks() { return R4 ? 2 : 4; }
+
 // One pass of k stages over G groups per block; see the file comment.
 template <bool DIT, bool R4>
-__global__ void __launch_bounds__(256) k_ntt_pass(Fr* data, size_t bstride, const Fr* __restrict__ tw,
-                                                  uint32_t logN, uint32_t s0, uint32_t k, uint32_t logG,
-                                                  int load_scale, int store_scale, int to_mont, ScaleTabs tabs) {
-  extern __shared__ uint32_t sm[];
+__global__ void __launch_bounds__(256, pass_min_blocks<R4>())
+    k_ntt_pass(Fr* data, size_t bstride, const Fr* __restrict__ tw, uint32_t logN, uint32_t s0, uint32_t k,
+               uint32_t logG, int load_scale, int store_scale, int raw, ScaleTabs tabs) {
+  extern __shared__ uint4 sm[];
   const PassGeo g{logN, s0, k, logG};
   Fr* arr = data + size_t(blockIdx.y) * bstride;
-  const size_t gid0 = size_t(blockIdx.x) << logG;
-  pass_load<DIT>(arr, g, gid0, sm, load_scale, to_mont, tabs);
+  const uint32_t gid0 = blockIdx.x << logG;
+  pass_load<DIT>(arr, g, gid0, sm, load_scale, raw, tabs);
   pass_stages<DIT, 1, R4>(sm, g, gid0, tw);
-  pass_store<DIT>(arr, g, gid0, sm, store_scale, tabs);
+  pass_store<DIT>(arr, g, gid0, sm, store_scale, s0 + k == logN, tabs);
 }
 
 // The turn of an inverse DIF transform into a forward DIT transform, in one pass: the
@@ -325,49 +367,49 @@ __global__ void __launch_bounds__(256) k_ntt_pass(Fr* data, size_t bstride, cons
 // the inverse's scaling by the factor of each element's natural index, and the DIT's
 // first pass over the same groups.  Saves a global round trip and a launch.
 template <bool R4>
-__global__ void __launch_bounds__(256) k_ntt_turn(Fr* data, size_t bstride, const Fr* __restrict__ tw_inv,
-                                                  const Fr* __restrict__ tw_fwd, uint32_t L, uint32_t k,
-                                                  uint32_t logG, int mid_scale, ScaleTabs tabs) {
-  extern __shared__ uint32_t sm[];
+__global__ void __launch_bounds__(256, pass_min_blocks<R4>())
+    k_ntt_turn(Fr* data, size_t bstride, const Fr* __restrict__ tw_inv, const Fr* __restrict__ tw_fwd, uint32_t L,
+               uint32_t k, uint32_t logG, int mid_scale, ScaleTabs tabs) {
+  extern __shared__ uint4 sm[];
   const PassGeo gdif{L, L - k, k, logG}, gdit{L, 0, k, logG};
   Fr* arr = data + size_t(blockIdx.y) * bstride;
-  const size_t gid0 = size_t(blockIdx.x) << logG;
+  const uint32_t gid0 = blockIdx.x << logG;
   const uint32_t E = 1u << (logG + k);
   pass_load<false>(arr, gdif, gid0, sm, SC_NONE, 0, tabs);
   pass_stages<false, 1, R4>(sm, gdif, gid0, tw_inv);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-    const size_t idx = pass_index<false>(gdif, gid0, e);
-    sm_put(sm, E, e, f_mul(sm_get(sm, E, e), scale_factor(tabs, mid_scale, brev_bits((uint32_t)idx, L))));
+    const uint32_t idx = pass_index<false>(gdif, gid0, e);
+    sm_put(sm, E, e, f_mul_lazy(scale_factor(tabs, mid_scale, brev_bits(idx, L)), sm_get(sm, E, e)));
   }
   pass_stages<true, 1, R4>(sm, gdit, gid0, tw_fwd);
-  pass_store<true>(arr, gdit, gid0, sm, SC_NONE, tabs);
+  pass_store<true>(arr, gdit, gid0, sm, SC_NONE, false, tabs);
 }
 
 // The quotient turn, one instance per blockIdx.y (arrays A_i, B_i, C_i, H_i of N
 // elements at i, m + i, 2m + i, 3m + i): the last DIT pass of A, B and C (strided groups),
 // h_ev = (A B - C) / (g^N - 1) on the staged elements, and the first DIF pass of the
-// inverse transform of h over the same groups; only H is written.  Small grids get up
-// to three times the threads of a single-array pass (the three forward passes side by
-// side), large ones one array's worth.
+// inverse transform of h over the same groups; only H is written.  Its three staged arrays
+// leave two blocks per SM: 512 threads of radix 2 on large grids, up to 768 (the three
+// forward passes side by side) of radix 4 on small ones.
 template <bool R4>
-__global__ void __launch_bounds__(768) k_ntt_quotient_turn(Fr* ev, uint32_t m, size_t N, const Fr* __restrict__ tw_fwd,
-                                                           const Fr* __restrict__ tw_inv, uint32_t L, uint32_t k,
-                                                           uint32_t logG, ScaleTabs tabs) {
-  extern __shared__ uint32_t sm[];
+__global__ void __launch_bounds__(R4 ? 768 : 512, R4 ? 1 : 2)
+    k_ntt_quotient_turn(Fr* ev, uint32_t m, size_t N, const Fr* __restrict__ tw_fwd, const Fr* __restrict__ tw_inv,
+                        uint32_t L, uint32_t k, uint32_t logG, ScaleTabs tabs) {
+  extern __shared__ uint4 sm[];
   const PassGeo gdit{L, L - k, k, logG}, gdif{L, 0, k, logG};
-  const size_t gid0 = size_t(blockIdx.x) << logG;
+  const uint32_t gid0 = blockIdx.x << logG;
   const uint32_t E = 1u << (logG + k);
   const size_t i = blockIdx.y;
   for (int p = 0; p < 3; p++)
-    pass_load<true>(ev + (size_t(p) * m + i) * N, gdit, gid0, sm + size_t(p) * 8 * E, SC_NONE, 0, tabs);
+    pass_load<true>(ev + (size_t(p) * m + i) * N, gdit, gid0, sm + size_t(p) * 2 * E, SC_NONE, 0, tabs);
   pass_stages<true, 3, R4>(sm, gdit, gid0, tw_fwd);
   const Fr zinv = ld_field(tabs.consts + 1);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-    const Fr a = sm_get(sm, E, e), b = sm_get(sm + 8 * E, E, e), c = sm_get(sm + 16 * E, E, e);
-    sm_put(sm, E, e, f_mul(f_sub(f_mul(a, b), c), zinv));
+    const Fr a = f_red2(sm_get(sm, E, e)), b = f_red2(sm_get(sm + 2 * E, E, e)), c = f_red2(sm_get(sm + 4 * E, E, e));
+    sm_put(sm, E, e, f_mul_lazy(f_sub2(f_mul_lazy(a, b), c), zinv));
   }
   pass_stages<false, 1, R4>(sm, gdif, gid0, tw_inv);
-  pass_store<false>(ev + (size_t(3) * m + i) * N, gdif, gid0, sm, SC_NONE, tabs);
+  pass_store<false>(ev + (size_t(3) * m + i) * N, gdif, gid0, sm, SC_NONE, false, tabs);
 }
 
 static std::once_flag g_smem_once;
@@ -444,7 +486,7 @@ static int launch_pass(bool dit, Fr* data, int batch, size_t bstride, const NttD
 }
 
 static int run_passes(bool dit, Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse,
-                      int load_scale, int store_scale, bool to_mont, int elog, cudaStream_t st) {
+                      int load_scale, int store_scale, bool raw, int elog, cudaStream_t st) {
   ZK_CHECK(elog >= 8 && elog <= 11, ZKVC_EINVAL, "ntt: 2^%d elements per block outside [2^8, 2^11]", elog);
   ZK_CHECK(batch >= 1 && batch <= 65535, ZKVC_EINVAL, "ntt: batch of %d arrays", batch);
   ntt_smem_attrs();
@@ -455,7 +497,7 @@ static int run_passes(bool dit, Fr* data, int batch, size_t bstride, const NttDo
   for (uint32_t p = 0; p < P; p++) {
     const bool first = p == 0, last = p + 1 == P;
     ZK_TRY(launch_pass(dit, data, batch, bstride, d, tw, s0, ks[p], elog, first ? load_scale : 0,
-                       last ? store_scale : 0, (first && to_mont) ? 1 : 0, st));
+                       last ? store_scale : 0, (first && raw) ? 1 : 0, st));
     s0 += ks[p];
   }
   return ZKVC_OK;
@@ -508,11 +550,11 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
   {
     const uint32_t k = ks[0];
     const PassShape sh = pass_shape(L, k, elog, m);
-    // three times the threads where the grid is too small to fill the GPU (latency-bound),
-    // one array's worth where it is large (more blocks per SM)
+    // three times the threads where the grid is too small to fill the GPU (latency-bound)
     const uint64_t blocks = uint64_t(sh.grid.x) * sh.grid.y;
-    const uint32_t threads =
-        blocks < 2 * uint64_t(device_sm_count()) ? std::min<uint32_t>(3 * sh.threads, 768) : sh.threads;
+    const uint32_t threads = blocks < 2 * uint64_t(device_sm_count()) ? std::min<uint32_t>(3 * sh.threads, 768)
+                             : radix4(sh.grid)                         ? sh.threads
+                                                                       : std::min<uint32_t>(2 * sh.threads, 512);
     if (radix4(sh.grid))
       k_ntt_quotient_turn<true><<<sh.grid, threads, size_t(3) * sh.E * 32, st>>>(ev, (uint32_t)m, N, d->tw_fwd,
                                                                                  d->tw_inv, L, k, sh.logG, tabs);
@@ -532,37 +574,56 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
 }
 
 int ntt_dif(Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse, int load_scale,
-            int store_scale, bool to_mont, cudaStream_t st, int elog) {
-  return run_passes(false, data, batch, bstride, d, inverse, load_scale, store_scale, to_mont, elog, st);
+            int store_scale, bool raw, cudaStream_t st, int elog) {
+  return run_passes(false, data, batch, bstride, d, inverse, load_scale, store_scale, raw, elog, st);
 }
 
 int ntt_dit(Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse, cudaStream_t st, int elog) {
   return run_passes(true, data, batch, bstride, d, inverse, 0, 0, false, elog, st);
 }
 
-__global__ void k_bitrev(Fr* a, uint32_t logN, int scale, int from_mont, ScaleTabs tabs) {
-  size_t N = size_t(1) << logN;
-  size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= N) return;
-  size_t q = brev_bits((uint32_t)p, logN);
-  if (p > q) return;
-  Fr x = ld_field(a + p), y = ld_field(a + q);
-  // natural index p receives the element at bit-reversed position q, and vice versa
-  if (scale) {
-    y = f_mul(y, scale_factor(tabs, scale, (uint32_t)p));
-    if (p != q) x = f_mul(x, scale_factor(tabs, scale, (uint32_t)q));
-  }
-  if (from_mont) {
-    x = f_from_mont(x);
-    y = f_from_mont(y);
-  }
-  st_field(a + p, y);
-  if (p != q) st_field(a + q, x);
+// The element at bit-reversed position q, natural index p, on its way out: times the factor
+// of p, below N (x: below 4N).
+__device__ __forceinline__ Fr bitrev_value(const Fr& x, int scale, uint32_t p, const ScaleTabs& tabs) {
+  return scale ? f_mul(scale_factor(tabs, scale, p), x) : f_once(f_red2(x));
 }
 
-int ntt_bitrev(Fr* data, const NttDomain* d, int scale, bool from_mont, cudaStream_t st) {
-  unsigned blocks = (unsigned)((d->N + 255) / 256);
-  k_bitrev<<<blocks, 256, 0, st>>>(data, d->logN, scale, from_mont ? 1 : 0, tabs_of(d)); ZK_COUNT_LAUNCH();
+__global__ void k_bitrev_small(Fr* a, uint32_t logN, int scale, ScaleTabs tabs) {
+  const uint32_t N = 1u << logN, p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= N) return;
+  const uint32_t q = brev_bits(p, logN);
+  if (p > q) return;
+  const Fr x = ld_field(a + p), y = ld_field(a + q);
+  st_field(a + p, bitrev_value(y, scale, p, tabs));
+  if (p != q) st_field(a + q, bitrev_value(x, scale, q, tabs));
+}
+
+// Bit reversal of N >= 256 elements in tiles: index (hi, mid, lo) with four bits in hi and
+// lo goes to (lo^r, mid^r, hi^r), so the 16 x 16 elements of one mid trade places with those
+// of mid^r, transposed and reversed, through shared memory; both sides move in runs of 512
+// bytes and every thread has work (one thread per index, half of them past the diagonal,
+// took 350 us at 2^22 with a scale, 131 now).
+constexpr int BR_ROW = 17;  // padded: a column's 16-byte halves fall in different banks
+__global__ void __launch_bounds__(256) k_bitrev_tiles(Fr* a, uint32_t logN, int scale, ScaleTabs tabs) {
+  __shared__ uint4 sm[2][2 * 16 * BR_ROW];
+  const uint32_t mid = blockIdx.x, mrev = logN == 8 ? 0u : brev_bits(mid, logN - 8);
+  if (mid > mrev) return;
+  const uint32_t hi = threadIdx.x >> 4, lo = threadIdx.x & 15, E = 16 * BR_ROW;
+  const uint32_t p = (hi << (logN - 4)) | (mid << 4) | lo, q = (hi << (logN - 4)) | (mrev << 4) | lo;
+  sm_put(sm[0], E, hi * BR_ROW + lo, ld_field(a + p));
+  sm_put(sm[1], E, hi * BR_ROW + lo, ld_field(a + q));
+  __syncthreads();
+  const uint32_t e = (__brev(lo) >> 28) * BR_ROW + (__brev(hi) >> 28);
+  st_field(a + q, bitrev_value(sm_get(sm[0], E, e), scale, q, tabs));
+  if (mid != mrev) st_field(a + p, bitrev_value(sm_get(sm[1], E, e), scale, p, tabs));
+}
+
+int ntt_bitrev(Fr* data, const NttDomain* d, int scale, cudaStream_t st) {
+  if (d->logN >= 8)
+    k_bitrev_tiles<<<1u << (d->logN - 8), 256, 0, st>>>(data, d->logN, scale, tabs_of(d));
+  else
+    k_bitrev_small<<<1, 128, 0, st>>>(data, d->logN, scale, tabs_of(d));
+  ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   return ZKVC_OK;
 }

@@ -38,19 +38,19 @@ int ntt_domain(uint32_t logN, const NttDomain** out);
 // Decimation-in-frequency: natural-order input, bit-reversed output, in place.
 //   load_scale  multiplies input i (natural index) before the first stage;
 //   store_scale multiplies output position p by the factor of natural index bitrev(p).
-//   to_mont     converts canonical input to Montgomery form on load.
+//   raw         reduces arbitrary 256-bit input values on load.
+// Data in Montgomery form or not (the transform is linear); output below N.
 // batch arrays of N elements each, batch_stride elements apart.  elog = log2 of the
 // elements a block stages in shared memory (8 .. 11; passes take min(elog, 10) stages).
 int ntt_dif(Fr* data, int batch, size_t batch_stride, const NttDomain* d, bool inverse, int load_scale,
-            int store_scale, bool to_mont, cudaStream_t st, int elog = 10);
+            int store_scale, bool raw, cudaStream_t st, int elog = 10);
 
 // Decimation-in-time: bit-reversed input, natural-order output, in place.
 int ntt_dit(Fr* data, int batch, size_t batch_stride, const NttDomain* d, bool inverse, cudaStream_t st,
             int elog = 10);
 
-// In-place bit-reversal permutation with an optional scale by natural index and an
-// optional conversion out of Montgomery form.
-int ntt_bitrev(Fr* data, const NttDomain* d, int scale, bool from_mont, cudaStream_t st);
+// In-place bit-reversal permutation with an optional scale by natural index.
+int ntt_bitrev(Fr* data, const NttDomain* d, int scale, cudaStream_t st);
 
 // The prover's quotient chain for m instances of one domain: ev holds the arrays A_0 ..
 // A_(m-1), B_0 .., C_0 .., H_0 .. (N_stride elements apart) with A, B, C the evaluations

@@ -90,24 +90,6 @@ constexpr int PAIR_BT = 128;  // and a warp of point arithmetic in the Miller lo
 
 __device__ __forceinline__ void f12_bar() { asm volatile("bar.sync 1, 96;" ::: "memory"); }
 
-// t < 64 N (nine limbs) mod N: the quotient from the top bits, at most one short
-__device__ __forceinline__ Fp f_mod9(const uint32_t (&t)[9]) {
-  const uint32_t h = (t[7] >> 16) | (t[8] << 16);  // t / 2^240 < 2^20
-  const uint32_t q = __umulhi(h, 346675u);         // 2^32 / 12389, N / 2^240 in (12388, 12389)
-  uint32_t p[8];
-  Fp r, x;
-  uint64_t c = 0;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    c += (uint64_t)q * mod_limb<FpCfg>(i);
-    p[i] = (uint32_t)c;
-    c >>= 32;
-    x.v[i] = t[i];
-  }
-  sub8(r.v, x.v, p);  // below 2N: the ninth limbs cancel
-  return f_once(r);
-}
-
 // t += x over nine limbs
 __device__ __forceinline__ void add9(uint32_t (&t)[9], const uint32_t (&x)[9]) {
   asm("add.cc.u32  %0, %0, %9;\n\taddc.cc.u32 %1, %1, %10;\n\taddc.cc.u32 %2, %2, %11;\n\t"
@@ -164,7 +146,7 @@ static __device__ __noinline__ void f12_mul(E12* dst, const E12* a, const E12* b
   }
   add9(x, y);
   add9(t, x);
-  const Fp r = f_mod9(t);
+  const Fp r = f_mod9<FpCfg>(t);
   f12_bar();  // every operand has been read
   if (lane < 24 && i == 0) st_field(&dst->c[2 * m + part], r);
   f12_bar();

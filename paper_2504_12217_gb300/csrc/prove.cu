@@ -770,7 +770,7 @@ int prove_graph(const zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW,
 int prove_autotune(zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, const uint8_t* rs, cudaStream_t st,
                    uint32_t* chosen) {
   static const uint32_t kCand[] = {2, 4, 8, 16, 32, 64};
-  static const uint32_t kElog[] = {8, 9, 10, 11};
+  static const uint32_t kElog[] = {8, 9, 0, 11};  // 0: the default, 2^10 elements
   static const uint32_t kRest[] = {0, 1, 2};
   static const uint32_t kBin[] = {0, 1};
   uint32_t saved[ZKVC_PK_TUNING_LEN];
@@ -875,7 +875,7 @@ int prove_autotune(zkvc_pk* pk, int mode, const int8_t* dX, const int8_t* dW, co
       uint32_t best = pk->prove_tune[r];
       for (int ci = 0; ci < ncand; ci++) {
         const uint32_t c = cand[ci];
-        if (c == best || (r == 4 && best == 0 && c == 10)) continue;
+        if (c == best) continue;
         pk->prove_tune[r] = c;
         float ms = 0;
         ZK_TRY(timed(m, &ms));
