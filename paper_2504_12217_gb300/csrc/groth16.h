@@ -26,6 +26,9 @@
 
 namespace zkvc {
 
+constexpr int CHAIN_THREADS = 160;  // of each of k_chains' two blocks (prove.cu)
+
+
 // Regions of the G1 base array, in order.  An entry stores nwin consecutive bases
 // 2^(c w) P (w < nwin) so that every window of one MSM shares one bucket set.
 enum G1Region : int {

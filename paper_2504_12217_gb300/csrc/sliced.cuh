@@ -225,35 +225,70 @@ static __device__ __noinline__ SlG1 sl_padd(SlG1 p, SlG1 q) {
   return {X3, Y3, ZZ3, sl_from(m, 2)};
 }
 
-// k P for one half of a GLV-split scalar (|k| < 2^128 with its sign; glv.h) on one warp:
-// the 15 multiples of +-P in shared memory T[1..15] (this warp's own table), then 4-bit
-// windows from the top: four doublings and at most one addition per window.
+// Signed digits of n (below 2^127) for width-4 windows: odd digits in [-7, 7], any two
+// nonzero ones at least four places apart, into d[0 ..] (zeroed by the caller); returns the
+// place of the top one (-1: n = 0).  Every lane computes the same.
+__device__ __forceinline__ int sl_wnaf4(uint32_t (&n)[4], int8_t* d) {
+  int pos = 0, top = -1;
+  while (n[0] | n[1] | n[2] | n[3]) {
+    int z = n[0] ? __ffs((int)n[0]) - 1 : 31;
+    pos += z;
+#pragma unroll
+    for (int i = 0; i < 4; i++) n[i] = __funnelshift_r(n[i], i < 3 ? n[i + 1] : 0u, z);
+    if ((n[0] & 1u) == 0) continue;
+    const int v = (int)(n[0] & 15u), s = v >= 8 ? v - 16 : v;
+    if ((threadIdx.x & 31) == 0) d[pos] = (int8_t)s;
+    top = pos;
+    n[0] &= ~15u;
+    uint64_t c = v >= 8 ? 16 : 0;  // n - s: the low four bits clear, plus 16 for a negative digit
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      c += n[i];
+      n[i] = (uint32_t)c;
+      c >>= 32;
+    }
+  }
+  return top;
+}
+
+// 2^shift k P for bits [lo, lo + count) of a GLV-split half scalar (|k| < 2^127 with its sign;
+// glv.h) on one warp: the odd multiples P .. 7P in shared memory T[0..3], then a doubling per
+// place and an addition per nonzero digit from the top, then the shift's doublings.
 template <class Half>
-__device__ __forceinline__ SlG1 sl_mul_half(SlG1 P, const Half& h, G1J* T) {
+__device__ __forceinline__ SlG1 sl_mul_piece(SlG1 P, const Half& h, uint32_t lo, uint32_t count, uint32_t shift,
+                                             G1J* T, int8_t* digits) {
   if (h.neg) P.Y = sl_neg(P.Y);
-  SlG1 prev = P;
-  sl_st(T + 1, P);
-  for (int i = 2; i < 16; i++) {
-    prev = sl_padd(prev, P);
-    sl_st(T + i, prev);
+  for (int i = threadIdx.x & 31; i < 132; i += 32) digits[i] = 0;
+  sl_st(T, P);
+  const SlG1 P2 = sl_pdbl(P);
+  SlG1 odd = P;
+  for (int i = 1; i < 4; i++) {
+    odd = sl_padd(odd, P2);
+    sl_st(T + i, odd);
+  }
+  uint32_t n[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) {  // (k >> lo) mod 2^count
+    const uint32_t w = (lo >> 5) + i;
+    const uint32_t x = w < 4 ? h.mag[w] : 0u, y = w + 1 < 4 ? h.mag[w + 1] : 0u;
+    n[i] = __funnelshift_r(x, y, lo & 31);
+    n[i] = count >= 32u * i + 32 ? n[i] : count > 32u * i ? n[i] & ((1u << (count - 32u * i)) - 1u) : 0u;
   }
   __syncwarp();
+  const int top = sl_wnaf4(n, digits);
+  __syncwarp();
   SlG1 acc = sl_inf();
-  bool started = false;
-  for (int w = 31; w >= 0; w--) {
-    if (started) {
-      acc = sl_pdbl(acc);
-      acc = sl_pdbl(acc);
-      acc = sl_pdbl(acc);
-      acc = sl_pdbl(acc);
-    }
-    const uint32_t nib = (h.mag[w >> 3] >> ((w & 7) * 4)) & 15u;
-    if (nib) {
-      const SlG1 t = sl_ld(T + nib);
-      acc = started ? sl_padd(acc, t) : t;
-      started = true;
+  if (top < 0) return acc;
+  for (int i = top; i >= 0; i--) {
+    if (i != top) acc = sl_pdbl(acc);
+    const int d = digits[i];
+    if (d) {
+      SlG1 t = sl_ld(T + (d > 0 ? d : -d) / 2);
+      if (d < 0) t.Y = sl_neg(t.Y);
+      acc = i == top ? t : sl_padd(acc, t);
     }
   }
+  for (uint32_t i = 0; i < shift; i++) acc = sl_pdbl(acc);
   return acc;
 }
 
