@@ -191,6 +191,7 @@ constexpr uint64_t TREE_MIN_TERMS = 1ull << 22;
 constexpr uint32_t TREE_MAX_ROUNDS = 5;
 constexpr uint32_t TREE_NONE = 0xffffffffu;        // a padding term of a bucket
 constexpr uint64_t TREE_NONE_BASE = 0x7fffffffull;  // base indices stay below: no term equals TREE_NONE
+constexpr uint64_t MSM_SMALL_TERMS = 65536;
 // Threads of the G1 accumulation kernel resident on the whole GPU at `at` threads per
 // block (one per chunk), from the occupancy of its register use; cached per block size.
 static uint64_t accum_resident_threads(uint32_t at);
@@ -262,7 +263,9 @@ int msm_plan_finalize(MsmPlan& p) {
   p.pad_slots = p.rounds ? key * ((1u << p.rounds) - 1u) : 0u;
   // default chunk: about two chunks per bucket, but at least ~40 k chunks so that the
   // accumulation fills the GPU, and 16 at the least (8 after affine rounds, where level 0
-  // is a small part); and at least the chunk that puts every point into one wave of
+  // is a small part; 8 or 4 for runs of up to a few thousand chunks, where a
+  // chunk's serial additions are the run's latency: a proof of [4,16] x [16,8] 467 us with
+  // 16, 362 with 8, 326 with 4); and at least the chunk that puts every point into one wave of
   // resident accumulation threads (the chunks are balanced, so a second, partial wave
   // would only add a tail).  Counted in the points that the affine rounds leave.
   const uint64_t pts0 = (slot + p.pad_slots) >> p.rounds;
@@ -276,7 +279,10 @@ int msm_plan_finalize(MsmPlan& p) {
     // (7/8 of the resident threads: the prover's other streams hold some SM slots)
     const uint64_t resident = accum_resident_threads(p.tune.accum_threads) * 7 / 8;
     const uint64_t one_wave = resident ? (pts0 + resident - 1) / resident : 0;
-    const uint64_t least = p.rounds ? 8 : 16;
+    const uint64_t least = p.rounds                     ? 8
+                           : slot < MSM_SMALL_TERMS / 8 ? 4
+                           : slot < MSM_SMALL_TERMS     ? 8
+                                                        : p.tune.least;
     p.chunk_pts = (uint32_t)std::min<uint64_t>(
         std::max<uint64_t>(std::max<uint64_t>(least, std::min(per_bucket, fill)), one_wave), 1024u >> p.rounds);
     p.chunk = p.chunk_pts << p.rounds;

@@ -45,6 +45,7 @@ struct MsmOut {
 // Launch-shape knobs of a run (chosen by the batch autotuner; defaults otherwise).
 struct MsmTune {
   uint32_t chunk = 0;          // terms per level-0 chunk (0: the default rule of msm_plan_finalize)
+  uint32_t least = 16;         // the default rule's smallest chunk
   uint32_t accum_threads = 128;
   uint32_t lanes = 0;          // lanes per chunk: 1, 4 (a quad), 0 = by the run's size
 };

@@ -316,6 +316,10 @@ static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* 
   P->rest.tune.chunk = pk->prove_tune[1];
   P->h.tune.chunk = pk->prove_tune[2];
   P->g2.tune.chunk = pk->prove_tune[3];
+  // serial additions of a default chunk: 8 where the run's latency is on a critical path (the
+  // G2 run, and the small-digit run that the chains wait for), 16 where it fills gaps
+  P->g2.tune.least = 8;
+  P->small.tune.least = chain ? 8 : 16;
   P->h.tune.lanes = pk->prove_tune[8] ? 4 : 1;
   P->small.tune.lanes = pk->prove_tune[9] ? 4 : 1;
   P->rest.tune.lanes = 1;
