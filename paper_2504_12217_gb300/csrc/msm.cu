@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "coop.cuh"
+#include "fp2_rounds.cuh"
 #include "msm.h"
 #include "sliced.cuh"
 
@@ -1244,10 +1245,11 @@ struct OutItem {
 //   slice  block per slice of one bit's buckets: the slice's sum (serial per thread, then
 //          the block's tree) into S;
 //   bit    the last slice block of a bit to finish sums the bit's slices (U_b) and doubles
-//          it b times (2^b U_b; G1 on one warp in limb-sliced arithmetic, G2 on a quad);
+//          it b times (2^b U_b; G1 on one warp in limb-sliced arithmetic, G2 on one warp's
+//          rounds of shared products, fp2_rounds.cuh);
 //   window the last bit of a window sums the window's c terms 2^b U_b;
 //   output the last window of an output applies Horner's rule over the output's windows
-//          (variable base; G1 on a sliced warp, G2 on a quad) or copies its one window.
+//          (variable base; doublings as for the bits) or copies its one window.
 // Each hand-over: the finishing block's stores, a fence by every storing thread, a
 // barrier, then a fetch-and-add on the level's counter (zeroed before the launch) by one
 // thread; the block that brings the count to the total goes on, after a fence, reading
@@ -1261,6 +1263,7 @@ __global__ void __launch_bounds__(SliceBT<F>::value) k_bits_chain(
   constexpr int BT = SliceBT<F>::value;
   __shared__ XYZZ<F> sh[BT];
   __shared__ XYZZ<F> xs;
+  __shared__ __align__(16) Fp2 gv[GV_COUNT];  // G2: the doublings' variables
   __shared__ uint32_t last;
   const uint32_t sl = blockIdx.x;
   uint32_t lo = 0, hi = nseg - 1;
@@ -1302,9 +1305,11 @@ __global__ void __launch_bounds__(SliceBT<F>::value) k_bits_chain(
         sl_st(D + g.dslot, y);  // eight lanes store a word of each coordinate
       }
     } else {
-      if (threadIdx.x < 4) {
-        for (uint32_t i = 0; i < shift; i++) x = p_dbl_quad(x);
-        if (threadIdx.x == 0) st_field(D + g.dslot, x);
+      if (threadIdx.x == 0) st_field(reinterpret_cast<XYZZ<F>*>(gv), x);
+      __syncthreads();
+      if (threadIdx.x < 32) {
+        g2_doublings(gv, shift);
+        if (threadIdx.x == 0) st_field(D + g.dslot, ld_field(reinterpret_cast<const XYZZ<F>*>(gv)));
       }
     }
     __threadfence();  // by every storing lane, before the barrier and the count below
@@ -1344,13 +1349,21 @@ __global__ void __launch_bounds__(SliceBT<F>::value) k_bits_chain(
     }
     sl_st(results + w.out, acc);
   } else {
-    if (threadIdx.x >= 4) return;
-    XYZZ<F> acc = ld_field(sh + it.nwin - 1);
+    // doublings on a warp, the windows' additions on its first quad
+    if (threadIdx.x >= 32) return;
+    XYZZ<F>* const pt = reinterpret_cast<XYZZ<F>*>(gv);
+    if (threadIdx.x == 0) st_field(pt, ld_field(sh + it.nwin - 1));
+    __syncwarp();
     for (int v = (int)it.nwin - 2; v >= 0; v--) {
-      for (uint32_t i = 0; i < it.c; i++) acc = p_dbl_quad(acc);
-      acc = p_add_quad(acc, ld_field(sh + v));
+      g2_doublings(gv, it.c);
+      if (threadIdx.x < 4) {
+        const XYZZ<F> acc = p_add_quad(ld_field(pt), ld_field(sh + v));
+        __syncwarp(quad_mask());
+        if (threadIdx.x == 0) st_field(pt, acc);
+      }
+      __syncwarp();
     }
-    if (threadIdx.x == 0) st_field(results + w.out, acc);
+    if (threadIdx.x == 0) st_field(results + w.out, ld_field(pt));
   }
 }
 

@@ -33,7 +33,7 @@
 // cyclotomic subgroup an inverse is a conjugation.  The result is exactly the pairing
 // value, not a power of it.
 #pragma once
-#include "curve.cuh"
+#include "fp2_rounds.cuh"
 
 namespace zkvc {
 
@@ -264,22 +264,14 @@ static __device__ __noinline__ void final_exp(E12* f, FinalScratch* s, const Fro
 }
 
 // ------------------------------------------------------------------ Miller loop
-// The point warp's variables (Fp2 each); lane 2 s + part of the warp handles part `part` of
-// slot s of a round.
+// The point warp's variables (fp2_rounds.cuh)
 enum MillerVar : uint8_t {
   MV_X, MV_Y, MV_Z, MV_QX, MV_QY, MV_XN, MV_YP, MV_B3,  // T, the point added, (-xP, 0), (yP, 0), 3 b'
   MV_0, MV_1, MV_2, MV_3, MV_4, MV_5, MV_6, MV_7, MV_8, MV_9, MV_L0, MV_L1, MV_L3, MV_COUNT
 };
-struct MillerOp {
-  uint8_t dst, a, b, op;
-};
-enum : uint8_t { OP_NONE, OP_MUL, OP_ADD, OP_SUB };
-
-// A program is a list of rounds of up to five operations of one kind.
 // Doubling: B = Y^2, E = 3 b' Z^2, F = 3 E; X3 = 2 X Y (B - F), Y3 = (B + F)^2 - 12 E^2,
 // Z3 = 8 B Y Z (four times the usual coordinates); l0 = 2 Y Z yP, l1 = -3 X^2 xP, l3 = B - E.
-constexpr int MILLER_OPS = 5;
-static __device__ const MillerOp MILLER_DBL[][MILLER_OPS] = {
+static __device__ const RoundOp MILLER_DBL[][ROUND_OPS] = {
     {{MV_0, MV_X, MV_Y, OP_MUL}, {MV_1, MV_Y, MV_Y, OP_MUL}, {MV_2, MV_Z, MV_Z, OP_MUL}, {MV_3, MV_Y, MV_Z, OP_MUL},
      {MV_4, MV_X, MV_X, OP_MUL}},
     {{MV_0, MV_0, MV_0, OP_ADD}, {MV_5, MV_1, MV_1, OP_ADD}, {MV_3, MV_3, MV_3, OP_ADD}, {MV_6, MV_4, MV_4, OP_ADD}},
@@ -294,7 +286,7 @@ static __device__ const MillerOp MILLER_DBL[][MILLER_OPS] = {
 // Addition of Q: th = Y - yQ Z, la = X - xQ Z, C = th^2, D = la^2, E = la D, F = Z C,
 // G = X D, H = E + F - 2 G; X3 = la H, Y3 = th (G - H) - E Y, Z3 = Z E; l0 = la yP,
 // l1 = -th xP, l3 = th xQ - la yQ.
-static __device__ const MillerOp MILLER_ADD[][MILLER_OPS] = {
+static __device__ const RoundOp MILLER_ADD[][ROUND_OPS] = {
     {{MV_0, MV_QY, MV_Z, OP_MUL}, {MV_1, MV_QX, MV_Z, OP_MUL}},
     {{MV_0, MV_Y, MV_0, OP_SUB}, {MV_1, MV_X, MV_1, OP_SUB}},
     {{MV_2, MV_0, MV_0, OP_MUL}, {MV_3, MV_1, MV_1, OP_MUL}, {MV_4, MV_0, MV_QX, OP_MUL}, {MV_5, MV_1, MV_QY, OP_MUL},
@@ -307,31 +299,6 @@ static __device__ const MillerOp MILLER_ADD[][MILLER_OPS] = {
     {{MV_X, MV_1, MV_7, OP_MUL}, {MV_2, MV_0, MV_8, OP_MUL}, {MV_3, MV_4, MV_Y, OP_MUL}, {MV_Z, MV_Z, MV_4, OP_MUL}},
     {{MV_Y, MV_2, MV_3, OP_SUB}},
 };
-
-// one round on the calling warp: every lane calls; rounds are uniform in kind
-__device__ __forceinline__ void miller_round(Fp2* V, const MillerOp* ops) {
-  const int lane = threadIdx.x & 31, s = lane >> 1, part = lane & 1;
-  const MillerOp o = ops[s < MILLER_OPS ? s : 0];
-  const bool mul = ops[0].op == OP_MUL;
-  const Fp* const A = &V[o.a].c0;
-  const Fp* const B = &V[o.b].c0;
-  Fp r;
-  if (mul) {
-    const Fp a0 = ld_field(A), a1 = ld_field(A + 1), b0 = ld_field(B + part), b1 = ld_field(B + 1 - part);
-    Fp n1 = f_comp(a1);
-#pragma unroll
-    for (int l = 0; l < 8; l++) n1.v[l] = part ? a1.v[l] : n1.v[l];
-    r = f_mul2(a0, b0, n1, b1);
-  } else {
-    const Fp x = ld_field(A + part), y = ld_field(B + part);
-    const Fp add = f_add(x, y), sub = f_sub(x, y);
-#pragma unroll
-    for (int l = 0; l < 8; l++) r.v[l] = o.op == OP_ADD ? add.v[l] : sub.v[l];
-  }
-  __syncwarp();
-  if (s < MILLER_OPS && o.op != OP_NONE) st_field(&V[o.dst].c0 + part, r);
-  __syncwarp();
-}
 
 struct alignas(16) MillerShared {
   E12 f, line[2];
@@ -405,9 +372,9 @@ __device__ __forceinline__ bool miller_loop(MillerShared* sh, const G1A& P, cons
             st_field(&V[lane < 2 ? MV_QX : MV_QY].c0 + (lane & 1), ld_field(src + (lane & 1)));
           }
           __syncwarp();
-          for (const auto& r : MILLER_ADD) miller_round(V, r);
+          for (const auto& r : MILLER_ADD) fp2_round(V, r);
         } else {
-          for (const auto& r : MILLER_DBL) miller_round(V, r);
+          for (const auto& r : MILLER_DBL) fp2_round(V, r);
         }
         E12* const L = &sh->line[s & 1];
         if (lane < 6) {  // l0, l1 w, l3 w^3
