@@ -151,6 +151,7 @@ __global__ void k_b_encode(const G1J* __restrict__ small, const G1J* __restrict_
 struct BatchTune {
   MsmTune small, main, g2;
   int elog = 10;
+  BatchTune() { small.floor = main.floor = g2.floor = 8; }  // the workspaces are sized for chunks of 8
 };
 
 struct NttGroup {

@@ -281,7 +281,7 @@ int msm_plan_finalize(MsmPlan& p) {
     const uint64_t resident = accum_resident_threads(p.tune.accum_threads) * 7 / 8;
     const uint64_t one_wave = resident ? (pts0 + resident - 1) / resident : 0;
     const uint64_t least = p.rounds                     ? 8
-                           : slot < MSM_SMALL_TERMS / 8 ? 4
+                           : slot < MSM_SMALL_TERMS / 8 ? p.tune.floor
                            : slot < MSM_SMALL_TERMS     ? 8
                                                         : p.tune.least;
     p.chunk_pts = (uint32_t)std::min<uint64_t>(

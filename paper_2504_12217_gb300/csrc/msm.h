@@ -46,6 +46,7 @@ struct MsmOut {
 struct MsmTune {
   uint32_t chunk = 0;          // terms per level-0 chunk (0: the default rule of msm_plan_finalize)
   uint32_t least = 16;         // the default rule's smallest chunk
+  uint32_t floor = 4;          // and its smallest for a run of few terms
   uint32_t accum_threads = 128;
   uint32_t lanes = 0;          // lanes per chunk: 1, 4 (a quad), 0 = by the run's size
 };
