@@ -86,14 +86,14 @@ static void b_matmul_init() {
 }
 
 __global__ void __launch_bounds__(256) k_b_crpc_ab(const BInst* __restrict__ I) {
-  __shared__ Fr sh[256];
+  __shared__ Wide sh[8 * CRPC_ROWS];
   const BInst& in = I[blockIdx.y];
-  if ((int)blockIdx.x >= in.n) return;
-  crpc_ab_row(in.X, in.W, in.zA, in.zB, in.a, in.n, in.b, blockIdx.x, in.ak, in.bk, sh);
+  if ((int)blockIdx.x * CRPC_ROWS >= in.n) return;
+  crpc_ab_rows(in.X, in.W, in.zA, in.zB, in.a, in.n, in.b, blockIdx.x * CRPC_ROWS, in.ak, in.bk, sh);
 }
 
 __global__ void __launch_bounds__(256) k_b_crpc_y(const BInst* __restrict__ I) {
-  __shared__ Fr sh[256];
+  __shared__ Wide sh[8];
   const BInst& in = I[blockIdx.y];
   if ((int)blockIdx.x >= in.a) return;
   crpc_y_row(in.Y, in.zA, in.zB, in.b, blockIdx.x, in.yz, sh);
@@ -428,7 +428,7 @@ static int enqueue(zkvc_batch* B) {
   k_b_matmul<<<dim3((maxb + MM_M - 1) / MM_M, (maxa + MM_N - 1) / MM_N, n), MM_THREADS, sizeof(MatmulSmem), st>>>(
       B->dinst);
   ZK_COUNT_LAUNCH();
-  k_b_crpc_ab<<<dim3(maxn, n), 256, 0, st>>>(B->dinst); ZK_COUNT_LAUNCH();
+  k_b_crpc_ab<<<dim3((maxn + CRPC_ROWS - 1) / CRPC_ROWS, n), 256, 0, st>>>(B->dinst); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   // G2 run on side stream 0 (needs b_k and s)
   ZK_CUDA(cudaEventRecord(B->fork[0], st));

@@ -914,6 +914,19 @@ __global__ void k_gen_spmv(CsrView m, const Fr* __restrict__ tab, const Fr* __re
   }
 }
 
+// Sum over the block of per-thread Fr values (blockDim.x = 256, sh of 256 entries).
+__device__ __forceinline__ Fr block_sum(Fr v, Fr* sh) {
+  st_field(sh + threadIdx.x, v);
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) st_field(sh + threadIdx.x, f_add(ld_field(sh + threadIdx.x), ld_field(sh + threadIdx.x + s)));
+    __syncthreads();
+  }
+  Fr r = ld_field(sh);
+  __syncthreads();
+  return r;
+}
+
 // a block (256 threads) per long row
 __global__ void __launch_bounds__(256) k_gen_spmv_long(CsrView m, const uint32_t* __restrict__ rows,
                                                        const Fr* __restrict__ tab, const Fr* __restrict__ w, Fr* Aev,
@@ -1092,7 +1105,7 @@ int prove_generic(const zkvc_pk* pk, const int8_t* dX, const int8_t* dW, const u
     case ZKVC_CIRCUIT_CRPC:
     case ZKVC_CIRCUIT_SOFTMAX:
     case ZKVC_CIRCUIT_GELU:
-      k_crpc_ab<<<sh.n, 256, 0, st>>>(dX, dW, pk->zA, pk->zB, sh.a, sh.n, sh.b, B.ak, B.bk); ZK_COUNT_LAUNCH();
+      k_crpc_ab<<<(sh.n + CRPC_ROWS - 1) / CRPC_ROWS, 256, 0, st>>>(dX, dW, pk->zA, pk->zB, sh.a, sh.n, sh.b, B.ak, B.bk); ZK_COUNT_LAUNCH();
       if (sh.circuit != ZKVC_CIRCUIT_CRPC) {
         k_crpc_y<<<sh.a, 256, 0, st>>>(dY, pk->zA, pk->zB, sh.b, B.yz); ZK_COUNT_LAUNCH();
         // prefix sums into the auxiliary array; the first n evaluations land in ev and are

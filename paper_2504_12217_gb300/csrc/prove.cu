@@ -41,18 +41,18 @@
 namespace zkvc {
 
 // ------------------------------------------------------------------ witness
-// block k < n: a_k and b_k
+// block k: a and b of CRPC_ROWS rows
 __global__ void __launch_bounds__(256) k_crpc_ab(const int8_t* __restrict__ X, const int8_t* __restrict__ W,
                                                  const Fr* __restrict__ zA, const Fr* __restrict__ zB, int a, int n, int b,
                                                  Fr* ak, Fr* bk) {
-  __shared__ Fr sh[256];
-  crpc_ab_row(X, W, zA, zB, a, n, b, blockIdx.x, ak, bk, sh);
+  __shared__ Wide sh[8 * CRPC_ROWS];
+  crpc_ab_rows(X, W, zA, zB, a, n, b, blockIdx.x * CRPC_ROWS, ak, bk, sh);
 }
 
 // block i < a: z^(ib) sum_j z^j y_ij
 __global__ void __launch_bounds__(256) k_crpc_y(const int32_t* __restrict__ Y, const Fr* __restrict__ zA,
                                                 const Fr* __restrict__ zB, int b, Fr* part) {
-  __shared__ Fr sh[256];
+  __shared__ Wide sh[8];
   crpc_y_row(Y, zA, zB, b, blockIdx.x, part, sh);
 }
 
@@ -471,7 +471,7 @@ static int prove_enqueue_impl(const zkvc_pk* pk, int mode, const int8_t* dX, con
   cudaStream_t s3 = side->st[3];
   // 1. the CRPC sums a_k, b_k (side stream 3);  2. Y = X W (tensor cores), unless a
   // claimed Y is given
-  k_crpc_ab<<<sh.n, 256, 0, s3>>>(dX, dW, pk->zA, pk->zB, sh.a, sh.n, sh.b, B.ak, B.bk); ZK_COUNT_LAUNCH();
+  k_crpc_ab<<<(sh.n + CRPC_ROWS - 1) / CRPC_ROWS, 256, 0, s3>>>(dX, dW, pk->zA, pk->zB, sh.a, sh.n, sh.b, B.ak, B.bk); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   ZK_CUDA(cudaEventRecord(side->fork[0], s3));  // G2 MSM: needs b_k and s
   if (!y_given) ZK_TRY(matmul_i8(dX, dW, dY, sh.a, sh.n, sh.b, B.flags, st));
