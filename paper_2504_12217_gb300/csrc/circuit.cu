@@ -628,7 +628,7 @@ int setup_generic(int a, int n, int b, int circuit, int pub, const uint8_t* toxi
     Fr* Bt = At + sh.n_vars;
     Fr* Ct = Bt + sh.n_vars;
     size_t lag_threads = (sh.n_rows + LAG_CHUNK - 1) / LAG_CHUNK;
-    k_lagrange<<<(unsigned)((lag_threads + 127) / 128), 128, 0, st>>>(d_sc, dom->tw_fwd, sh.N, (uint32_t)sh.n_rows, d_L); ZK_COUNT_LAUNCH();
+    k_lagrange<<<(unsigned)((lag_threads + 127) / 128), 128, 0, st>>>(d_sc, dom->tw, sh.N, (uint32_t)sh.n_rows, d_L); ZK_COUNT_LAUNCH();
     for (int mi = 0; mi < 3 && rc == ZKVC_OK; mi++) {
       uint64_t* cp = nullptr;
       uint32_t *rw = nullptr, *cf = nullptr;

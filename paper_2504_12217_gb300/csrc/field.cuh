@@ -570,6 +570,128 @@ __device__ __forceinline__ Field<C> f_mul_lazy(const Field<C>& a, const Field<C>
   return r;
 }
 
+// Products by a constant w known ahead (a transform's twiddles) with its quotient
+// wq = floor(w 2^256 / N) beside it (Shoup's method, as in Harvey, "Faster arithmetic for
+// number-theoretic transforms", 2014): q = floor(x wq / 2^256) is the quotient of x w / N or
+// a little less, so x w - q N is found from its low 256 bits alone.  Neither product is
+// needed whole: q from the columns 6 .. 14 of x wq (43 multiply-adds, short of the true
+// quotient by less than x / 2^256 + 1 + 2^-29), and the columns 0 .. 7 of x w and of
+// q (2^256 - N), summed in one pair of accumulators (28 and 8 low products each): 99
+// multiply-adds and 16 low products against the Montgomery product's 128 and 8.
+namespace eo {
+// N products x0 y, x1 y, x2 y into t[0 .. 2N - 1], the carry out dropped; LOW: one more
+// whose low half alone goes to t[2N]
+template <int N, bool LOW>
+__device__ __forceinline__ void chain_low(uint32_t* t, const uint32_t* x, uint32_t y) {
+  if constexpr (N == 3 && LOW)
+    asm("mad.lo.cc.u32  %0, %7, %11, %0;\n\tmadc.hi.cc.u32 %1, %7, %11, %1;\n\t"
+        "madc.lo.cc.u32 %2, %8, %11, %2;\n\tmadc.hi.cc.u32 %3, %8, %11, %3;\n\t"
+        "madc.lo.cc.u32 %4, %9, %11, %4;\n\tmadc.hi.cc.u32 %5, %9, %11, %5;\n\tmadc.lo.u32 %6, %10, %11, %6;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6])
+        : "r"(x[0]), "r"(x[2]), "r"(x[4]), "r"(x[6]), "r"(y));
+  else if constexpr (N == 2 && LOW)
+    asm("mad.lo.cc.u32  %0, %5, %8, %0;\n\tmadc.hi.cc.u32 %1, %5, %8, %1;\n\t"
+        "madc.lo.cc.u32 %2, %6, %8, %2;\n\tmadc.hi.cc.u32 %3, %6, %8, %3;\n\tmadc.lo.u32 %4, %7, %8, %4;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4])
+        : "r"(x[0]), "r"(x[2]), "r"(x[4]), "r"(y));
+  else if constexpr (N == 1 && LOW)
+    asm("mad.lo.cc.u32 %0, %3, %5, %0;\n\tmadc.hi.cc.u32 %1, %3, %5, %1;\n\tmadc.lo.u32 %2, %4, %5, %2;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2])
+        : "r"(x[0]), "r"(x[2]), "r"(y));
+  else if constexpr (LOW)
+    t[0] += x[0] * y;
+  else if constexpr (N == 4)
+    chain(t, x, 0, y);
+  else if constexpr (N == 3)
+    asm("mad.lo.cc.u32  %0, %6, %9, %0;\n\tmadc.hi.cc.u32 %1, %6, %9, %1;\n\t"
+        "madc.lo.cc.u32 %2, %7, %9, %2;\n\tmadc.hi.cc.u32 %3, %7, %9, %3;\n\t"
+        "madc.lo.cc.u32 %4, %8, %9, %4;\n\tmadc.hi.u32 %5, %8, %9, %5;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5])
+        : "r"(x[0]), "r"(x[2]), "r"(x[4]), "r"(y));
+  else if constexpr (N == 2)
+    asm("mad.lo.cc.u32  %0, %4, %6, %0;\n\tmadc.hi.cc.u32 %1, %4, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %6, %2;\n\tmadc.hi.u32 %3, %5, %6, %3;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3])
+        : "r"(x[0]), "r"(x[2]), "r"(y));
+  else
+    asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;"
+        : "+r"(t[0]), "+r"(t[1])
+        : "r"(x[0]), "r"(y));
+}
+// rows I .. 7 of the low half of x y: e[0..7] + 2^32 o[0..6] += x y_I 2^(32 I) + .. mod 2^256
+template <int I>
+__device__ __forceinline__ void low_rows(uint32_t* e, uint32_t* o, const uint32_t* x, const uint32_t* y) {
+  if constexpr (I < 8) {
+    // even columns I + j <= 6 and odd ones I + j <= 7 (the last by its low half)
+    if constexpr (I % 2 == 0) {
+      chain_low<4 - I / 2, false>(e + I, x, y[I]);
+      chain_low<3 - I / 2, true>(o + I, x + 1, y[I]);
+    } else {
+      if constexpr (I < 7) chain_low<3 - I / 2, false>(e + I + 1, x + 1, y[I]);
+      chain_low<3 - I / 2, true>(o + I - 1, x, y[I]);
+    }
+    low_rows<I + 1>(e, o, x, y);
+  }
+}
+}  // namespace eo
+
+// x w mod N, not brought below N: below 2N for x < 4N (w < N in plain form, wq its quotient)
+template <class C>
+__device__ __forceinline__ Field<C> f_mul_const(const Field<C>& x, const Field<C>& w, const Field<C>& wq) {
+  uint32_t e[10], o[9], q[8], n[8];
+  const uint32_t* a = x.v;
+  {  // columns 6 .. 14 of x wq: e[c - 6], e[c - 5] even c; o[c - 7], o[c - 6] odd c
+    const uint64_t p6 = (uint64_t)a[6] * wq.v[0], p7 = (uint64_t)a[7] * wq.v[0];
+    e[0] = (uint32_t)p6;
+    e[1] = (uint32_t)(p6 >> 32);
+    e[2] = 0;
+    o[0] = (uint32_t)p7;
+    o[1] = (uint32_t)(p7 >> 32);
+    eo::chain_s<2, 1>(e, a[5], a[7], 0, wq.v[1]);
+    eo::chain_s<1, 0>(o, a[6], 0, 0, wq.v[1]);
+    eo::chain_s<2, 0>(e, a[4], a[6], 0, wq.v[2]);
+    eo::chain_s<2, 1>(o, a[5], a[7], 0, wq.v[2]);
+    eo::chain_s<3, 1>(e, a[3], a[5], a[7], wq.v[3]);
+    eo::chain_s<2, 0>(o, a[4], a[6], 0, wq.v[3]);
+    eo::chain_s<3, 0>(e, a[2], a[4], a[6], wq.v[4]);
+    eo::chain_s<3, 1>(o, a[3], a[5], a[7], wq.v[4]);
+    eo::chain_f1(e, a, 1, wq.v[5]);
+    eo::chain_s<3, 0>(o, a[2], a[4], a[6], wq.v[5]);
+    eo::chain_cf(e, e[8], a, 0, wq.v[6]);
+    eo::chain_f1(o, a, 1, wq.v[6]);
+    eo::chain_f1(e + 2, a, 1, wq.v[7]);
+    eo::chain_cf(o, o[8], a, 0, wq.v[7]);
+    asm("{\n\t.reg .u32 c;\n\tadd.cc.u32 c, %8, %17;\n\t"
+        "addc.cc.u32 %0, %9,  %18;\n\taddc.cc.u32 %1, %10, %19;\n\taddc.cc.u32 %2, %11, %20;\n\t"
+        "addc.cc.u32 %3, %12, %21;\n\taddc.cc.u32 %4, %13, %22;\n\taddc.cc.u32 %5, %14, %23;\n\t"
+        "addc.cc.u32 %6, %15, %24;\n\taddc.u32 %7, %16, %25;\n\t}"
+        : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7])
+        : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(e[8]), "r"(e[9]), "r"(o[0]),
+          "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]), "r"(o[8]));
+  }
+#pragma unroll
+  for (int i = 0; i < 8; i++) n[i] = i == 0 ? 0u - mod_limb<C>(0) : ~mod_limb<C>(i);  // 2^256 - N (N is odd)
+  eo::mul4(e, a, 0, w.v[0]);
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    const uint64_t p = (uint64_t)a[1 + 2 * j] * w.v[0];
+    o[2 * j] = (uint32_t)p;
+    o[2 * j + 1] = (uint32_t)(p >> 32);
+  }
+  o[6] = a[7] * w.v[0];
+  eo::low_rows<1>(e, o, a, w.v);
+  eo::low_rows<0>(e, o, n, q);
+  Field<C> r;
+  r.v[0] = e[0];
+  asm("add.cc.u32  %0, %7,  %14;\n\taddc.cc.u32 %1, %8,  %15;\n\taddc.cc.u32 %2, %9, %16;\n\t"
+      "addc.cc.u32 %3, %10, %17;\n\taddc.cc.u32 %4, %11, %18;\n\taddc.cc.u32 %5, %12, %19;\n\t"
+      "addc.u32 %6, %13, %20;"
+      : "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]), "=r"(r.v[7])
+      : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+        "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]));
+  return r;
+}
+
 // the product below N, for operands whose lazy product is below 2N.  (Values that may exceed
 // N come second: f_to_mont reduces an arbitrary 256-bit value.)
 template <class C>

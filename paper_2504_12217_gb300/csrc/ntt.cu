@@ -10,9 +10,17 @@
 // natural order to bit-reversed order and decimation in time maps it back, so the prove
 // path (INTT -> coset NTT -> pointwise -> coset INTT) never runs a bit-reversal pass:
 // the coset shift g^i and 1/N are applied at the bit-reversed store of the inverse
-// transforms.  The transform is linear and its twiddles are in Montgomery form, so data in
-// either form goes through unconverted.  Twiddles are read from a table omega^e (e < N/2), L2-resident for the
-// proof domains.
+// transforms.  The transform is linear and its twiddles are in plain form, so data in
+// either form (Montgomery or not) goes through unconverted.
+//
+// Each stage reads its twiddles omega^(j 2^s) from a table of its own, so neighbouring
+// butterflies read neighbouring entries at every stage (out of one table of N/2, the entries
+// of a later stage lie in a line each), and a second table holds their quotients
+// floor(omega^e 2^256 / r) (f_mul_const).  The inverse transforms read the same tables:
+// omega^-e = -omega^(N/2 - e), the sign taken by exchanging the operands of the butterfly's
+// difference.  2^22 coset inverse: Montgomery twiddles from one table 950 us, quotients from
+// one table 977, Montgomery twiddles by stages 928, quotients by stages 875; 2^24: 3,769 us
+// with Montgomery twiddles by stages, 3,493 with quotients.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -22,6 +30,12 @@
 #include "ntt.h"
 
 namespace zkvc {
+
+// first entry of the twiddle table of decimation-in-frequency stage s (2^(L - 1 - s) + 1
+// entries omega^(j 2^s), in whole 128-byte lines); s = L: all of them
+__host__ __device__ __forceinline__ size_t tw_offset(uint32_t L, uint32_t s) {
+  return (size_t(1) << L) - (size_t(1) << (L - s)) + 4 * s;
+}
 
 struct ScaleTabs {
   const Fr* g_lo;
@@ -99,6 +113,44 @@ __global__ void k_fill_pows(Fr* out, size_t count, const Fr* base_p, const Fr* m
   }
 }
 
+// From the Montgomery forms m = w 2^256 mod r of the twiddles in out[0 .. total): the plain w
+// there and out[total + e] = floor(w 2^256 / r) = (w 2^256 - m) / r, which is -m / r mod 2^256
+// (limb by limb, as in a reduction).
+__global__ void k_fill_twiddles(Fr* out, size_t total) {
+  const size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const Fr m = ld_field(out + e);
+  st_field(out + e, f_from_mont(m));
+  uint32_t t[8];
+  Fr q;
+#pragma unroll
+  for (int i = 0; i < 8; i++) t[i] = m.v[i];
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    q.v[i] = t[i] * FrCfg::INV;
+    uint64_t c = 0;
+#pragma unroll
+    for (int j = 0; i + j < 8; j++) {
+      c += (uint64_t)q.v[i] * mod_limb<FrCfg>(j) + t[i + j];
+      t[i + j] = (uint32_t)c;
+      c >>= 32;
+    }
+  }
+  st_field(out + total + e, q);
+}
+
+// the tables of the stages s >= 1: every 2^s-th entry of stage 0's
+__global__ void k_fill_stages(Fr* out, uint32_t L) {
+  const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;  // 2^(L - 1 - s) + j, j < 2^(L - 1 - s); 0: the last entries
+  if (e >= 1u << (L - 1)) return;
+  if (e == 0) {
+    for (uint32_t s = 1; s < L; s++) st_field(out + tw_offset(L, s) + (1u << (L - 1 - s)), ld_field(out + (1u << (L - 1))));
+    return;
+  }
+  const uint32_t lg = 31 - __clz(e), s = L - 1 - lg, j = e - (1u << lg);
+  if (s >= 1) st_field(out + tw_offset(L, s) + j, ld_field(out + (size_t(j) << s)));
+}
+
 static int fill_pows(Fr* out, size_t count, const Fr* base, const Fr* mult, cudaStream_t st) {
   size_t runs = (count + 15) / 16;
   unsigned blocks = (unsigned)((runs + 127) / 128);
@@ -128,8 +180,7 @@ int ntt_domain(uint32_t logN, const NttDomain** out) {
   cudaStream_t st;
   ZK_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   ZK_CUDA(cudaMalloc(&d->consts, 16 * sizeof(Fr)));
-  ZK_CUDA(cudaMalloc(&d->tw_fwd, half * sizeof(Fr)));
-  ZK_CUDA(cudaMalloc(&d->tw_inv, half * sizeof(Fr)));
+  ZK_CUDA(cudaMalloc(&d->tw, 2 * tw_offset(logN, logN) * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->g_lo, 1024 * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->gi_lo, 1024 * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->g_hi, hi * sizeof(Fr)));
@@ -138,8 +189,10 @@ int ntt_domain(uint32_t logN, const NttDomain** out) {
   k_domain_consts<<<1, 1, 0, st>>>(d->consts, logN); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   const Fr* c = d->consts;
-  ZK_TRY(fill_pows(d->tw_fwd, half, c + 2, c + 8, st));
-  ZK_TRY(fill_pows(d->tw_inv, half, c + 3, c + 8, st));
+  ZK_TRY(fill_pows(d->tw, half + 1, c + 2, c + 8, st));
+  k_fill_stages<<<(unsigned)((half + 255) / 256), 256, 0, st>>>(d->tw, logN); ZK_COUNT_LAUNCH();
+  k_fill_twiddles<<<(unsigned)((tw_offset(logN, logN) + 255) / 256), 256, 0, st>>>(d->tw, tw_offset(logN, logN)); ZK_COUNT_LAUNCH();
+  ZK_CUDA(cudaGetLastError());
   ZK_TRY(fill_pows(d->g_lo, 1024, c + 4, c + 8, st));
   ZK_TRY(fill_pows(d->gi_lo, 1024, c + 5, c + 8, st));
   ZK_TRY(fill_pows(d->g_hi, hi, c + 6, c + 8, st));
@@ -183,11 +236,12 @@ __device__ __forceinline__ void sm_put(uint4* sm, uint32_t E, uint32_t e, const 
   sm[E + e] = make_uint4(x.v[4], x.v[5], x.v[6], x.v[7]);
 }
 
-// What bounds a pass on a large grid: the products, at 0.74 of the multiplier's rate (289
-// instructions per warp of butterflies, 136 of them the product's multiply-adds; 405 with
-// eight scalar shared-memory accesses per element, full reductions and 64-bit indices).
-// Measured at 2^22, passes of 8 + 7 + 7 stages: 306 + 257 + 226 us (378 + 296 + 293 before);
-// the first is slower by its twiddles, whose table leaves L2 between stages.
+// What bounds a pass on a large grid: the products, at 0.8 of the multiplier's rate where
+// the twiddles stay in L1 (the passes after the first).  Measured at 2^22, passes of 8 + 7 +
+// 7 stages: 285 + 228 + 217 us (306 + 257 + 226 with Montgomery products by twiddles from
+// one table; 378 + 296 + 293 with eight scalar shared-memory accesses per element, full
+// reductions and 64-bit indices before that); the first reads its twiddles from memory, as
+// many bytes as the data.
 //
 // Values stay lazily reduced between loads and stores: below 2N in a decimation-in-frequency
 // pass, below 4N in a decimation-in-time pass, so a butterfly's product needs no
@@ -237,23 +291,35 @@ __device__ __forceinline__ void pass_store(Fr* arr, const PassGeo& g, uint32_t g
 //     and j0 + h/2, j0 + h, j0 + 3h/2; twiddles w_t(off), w_t(off + h/2), w_(t+1)(off).
 //   DIT, stage t of half h (block 2h), then 2h: a unit is j0 = blk 4h + off (off < h) and
 //     j0 + h, j0 + 2h, j0 + 3h; twiddles w_t(off), w_(t+1)(off), w_(t+1)(off + h).
-// w_t(q) is the table entry of the radix-2 form: DIF ((q << sbits) + lo) << s, DIT
-// ((q << s0) + lo) << (L - 1 - s), lo the group's low index bits, s = s0 + t.  The
+// w_t(q) is entry (q << sbits) + lo of the table of DIF stage s = s0 + t, in DIT entry
+// (q << s0) + lo of that of stage L - 1 - s, lo the group's low index bits; INV (DIF only): minus
+// the entry as far from the table's end, so the difference is taken the other way round.  The
 // transform's stage of half 1 over neighbouring elements (DIF s = L - 1, DIT s = 0) has
 // w = 1 throughout and takes no product.
-template <bool DIT, int NPOLY, bool R4>
+template <bool DIT, int NPOLY, bool R4, bool INV>
 __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_t gid0, const Fr* tw) {
   const uint32_t G = 1u << g.logG, E = G << g.k, L = g.L, logG = g.logG;
   const uint32_t sbits = DIT ? g.s0 : (L - g.s0 - g.k);
   const uint32_t smask = (1u << sbits) - 1u;
-  auto twi = [&](uint32_t s, uint32_t q, uint32_t lo) -> const Fr* {
-    return tw + (DIT ? (((q << g.s0) + lo) << (L - 1 - s)) : (((q << sbits) + lo) << s));
+  static_assert(!(DIT && INV), "the forward transforms alone run by decimation in time");
+  // the table of stage s and its entry for a butterfly
+  auto stage_tab = [&](uint32_t s) -> const Fr* {
+    const uint32_t sd = DIT ? L - 1 - s : s;
+    return tw + tw_offset(L, sd) + (INV ? 1u << (L - 1 - sd) : 0u);
   };
+  const size_t total = tw_offset(L, L);
+  auto mul_tw = [&](const Fr& x, const Fr* tab, uint32_t q, uint32_t lo) -> Fr {
+    const uint32_t p = DIT ? (q << g.s0) + lo : (q << sbits) + lo;
+    const Fr* w = INV ? tab - p : tab + p;
+    return f_mul_const(x, ld_field(w), ld_field(w + total));
+  };
+  auto diff = [&](const Fr& x, const Fr& y) -> Fr { return INV ? f_sub2(y, x) : f_sub2(x, y); };
   __syncthreads();
   uint32_t t = 0;
   const uint32_t nq = E >> 2;
   for (; R4 && t + 1 < g.k; t += 2) {
     const uint32_t s = g.s0 + t;
+    const Fr *tab0 = stage_tab(s), *tab1 = stage_tab(s + 1);
     for (uint32_t ua = threadIdx.x; ua < nq * (uint32_t)NPOLY; ua += blockDim.x) {
       const uint32_t poly = NPOLY == 1 ? 0u : ua / nq, u = ua - poly * nq;
       uint4* smp = sm + size_t(poly) * 2 * E;
@@ -269,16 +335,15 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
           x1 = f_red2(x1);
           x3 = f_red2(x3);
         } else {
-          const Fr w0 = ld_field(twi(s, off, lo));
-          x1 = f_mul_lazy(x1, w0);
-          x3 = f_mul_lazy(x3, w0);
+          x1 = mul_tw(x1, tab0, off, lo);
+          x3 = mul_tw(x3, tab0, off, lo);
         }
         const Fr x0 = f_red2(sm_get(smp, E, p0)), x2 = f_red2(sm_get(smp, E, p2));
-        const Fr vc = f_mul_lazy(f_add_raw(x2, x3), ld_field(twi(s + 1, off, lo)));
+        const Fr vc = mul_tw(f_add_raw(x2, x3), tab1, off, lo);
         const Fr a = f_red2(f_add_raw(x0, x1));
         sm_put(smp, E, p0, f_add_raw(a, vc));
         sm_put(smp, E, p2, f_sub2(a, vc));
-        const Fr vd = f_mul_lazy(f_sub2(x2, x3), ld_field(twi(s + 1, off + h, lo)));
+        const Fr vd = mul_tw(f_sub2(x2, x3), tab1, off + h, lo);
         const Fr b = f_red2(f_sub2(x0, x1));
         sm_put(smp, E, p1, f_add_raw(b, vd));
         sm_put(smp, E, p3, f_sub2(b, vd));
@@ -291,24 +356,21 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
         {
           const Fr x0 = sm_get(smp, E, p0), x2 = sm_get(smp, E, p2);
           a = f_add2(x0, x2);
-          b = f_mul_lazy(f_sub2(x0, x2), ld_field(twi(s, off, lo)));
+          b = mul_tw(diff(x0, x2), tab0, off, lo);
         }
         {
           const Fr x1 = sm_get(smp, E, p1), x3 = sm_get(smp, E, p3);
           c = f_add2(x1, x3);
-          d = f_mul_lazy(f_sub2(x1, x3), ld_field(twi(s, off + hq, lo)));
+          d = mul_tw(diff(x1, x3), tab0, off + hq, lo);
         }
         sm_put(smp, E, p0, f_add2(a, c));
         sm_put(smp, E, p2, f_add2(b, d));
-        a = f_sub2(a, c);
-        b = f_sub2(b, d);
         if (s + 1 == L - 1) {
-          a = f_red2(a);
-          b = f_red2(b);
+          a = f_red2(f_sub2(a, c));
+          b = f_red2(f_sub2(b, d));
         } else {
-          const Fr w2 = ld_field(twi(s + 1, off, lo));
-          a = f_mul_lazy(a, w2);
-          b = f_mul_lazy(b, w2);
+          a = mul_tw(diff(a, c), tab1, off, lo);
+          b = mul_tw(diff(b, d), tab1, off, lo);
         }
         sm_put(smp, E, p1, a);
         sm_put(smp, E, p3, b);
@@ -318,6 +380,7 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
   }
   for (; t < g.k; t++) {  // radix 2: every stage, or the last of an odd count
     const uint32_t s = g.s0 + t, nbf = E >> 1;
+    const Fr* tab = stage_tab(s);
     const uint32_t logh = DIT ? t : (g.k - 1 - t), h = 1u << logh;
     const bool unit = DIT ? s == 0 : s == L - 1;
     for (uint32_t bfa = threadIdx.x; bfa < nbf * (uint32_t)NPOLY; bfa += blockDim.x) {
@@ -330,13 +393,12 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
       const uint32_t lo = (gid0 + gg) & smask;
       const Fr u = sm_get(smp, E, pu), v = sm_get(smp, E, pv);
       if (DIT) {
-        const Fr x = f_red2(u), y = unit ? f_red2(v) : f_mul_lazy(v, ld_field(twi(s, qh, lo)));
+        const Fr x = f_red2(u), y = unit ? f_red2(v) : mul_tw(v, tab, qh, lo);
         sm_put(smp, E, pu, f_add_raw(x, y));
         sm_put(smp, E, pv, f_sub2(x, y));
       } else {
         sm_put(smp, E, pu, f_add2(u, v));
-        const Fr d = f_sub2(u, v);
-        sm_put(smp, E, pv, unit ? f_red2(d) : f_mul_lazy(d, ld_field(twi(s, qh, lo))));
+        sm_put(smp, E, pv, unit ? f_red2(f_sub2(u, v)) : mul_tw(diff(u, v), tab, qh, lo));
       }
     }
     __syncthreads();
@@ -349,7 +411,7 @@ template <bool R4>
 constexpr int pass_min_blocks() { return R4 ? 2 : 4; }
 
 // One pass of k stages over G groups per block; see the file comment.
-template <bool DIT, bool R4>
+template <bool DIT, bool R4, bool INV>
 __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
     k_ntt_pass(Fr* data, size_t bstride, const Fr* __restrict__ tw, uint32_t logN, uint32_t s0, uint32_t k,
                uint32_t logG, int load_scale, int store_scale, int raw, ScaleTabs tabs) {
@@ -358,7 +420,7 @@ __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
   Fr* arr = data + size_t(blockIdx.y) * bstride;
   const uint32_t gid0 = blockIdx.x << logG;
   pass_load<DIT>(arr, g, gid0, sm, load_scale, raw, tabs);
-  pass_stages<DIT, 1, R4>(sm, g, gid0, tw);
+  pass_stages<DIT, 1, R4, INV>(sm, g, gid0, tw);
   pass_store<DIT>(arr, g, gid0, sm, store_scale, s0 + k == logN, tabs);
 }
 
@@ -368,20 +430,20 @@ __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
 // first pass over the same groups.  Saves a global round trip and a launch.
 template <bool R4>
 __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
-    k_ntt_turn(Fr* data, size_t bstride, const Fr* __restrict__ tw_inv, const Fr* __restrict__ tw_fwd, uint32_t L,
-               uint32_t k, uint32_t logG, int mid_scale, ScaleTabs tabs) {
+    k_ntt_turn(Fr* data, size_t bstride, const Fr* __restrict__ tw, uint32_t L, uint32_t k,
+               uint32_t logG, int mid_scale, ScaleTabs tabs) {
   extern __shared__ uint4 sm[];
   const PassGeo gdif{L, L - k, k, logG}, gdit{L, 0, k, logG};
   Fr* arr = data + size_t(blockIdx.y) * bstride;
   const uint32_t gid0 = blockIdx.x << logG;
   const uint32_t E = 1u << (logG + k);
   pass_load<false>(arr, gdif, gid0, sm, SC_NONE, 0, tabs);
-  pass_stages<false, 1, R4>(sm, gdif, gid0, tw_inv);
+  pass_stages<false, 1, R4, true>(sm, gdif, gid0, tw);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
     const uint32_t idx = pass_index<false>(gdif, gid0, e);
     sm_put(sm, E, e, f_mul_lazy(scale_factor(tabs, mid_scale, brev_bits(idx, L)), sm_get(sm, E, e)));
   }
-  pass_stages<true, 1, R4>(sm, gdit, gid0, tw_fwd);
+  pass_stages<true, 1, R4, false>(sm, gdit, gid0, tw);
   pass_store<true>(arr, gdit, gid0, sm, SC_NONE, false, tabs);
 }
 
@@ -393,8 +455,8 @@ __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
 // forward passes side by side) of radix 4 on small ones.
 template <bool R4>
 __global__ void __launch_bounds__(R4 ? 768 : 512, R4 ? 1 : 2)
-    k_ntt_quotient_turn(Fr* ev, uint32_t m, size_t N, const Fr* __restrict__ tw_fwd, const Fr* __restrict__ tw_inv,
-                        uint32_t L, uint32_t k, uint32_t logG, ScaleTabs tabs) {
+    k_ntt_quotient_turn(Fr* ev, uint32_t m, size_t N, const Fr* __restrict__ tw, uint32_t L, uint32_t k,
+                        uint32_t logG, ScaleTabs tabs) {
   extern __shared__ uint4 sm[];
   const PassGeo gdit{L, L - k, k, logG}, gdif{L, 0, k, logG};
   const uint32_t gid0 = blockIdx.x << logG;
@@ -402,13 +464,13 @@ __global__ void __launch_bounds__(R4 ? 768 : 512, R4 ? 1 : 2)
   const size_t i = blockIdx.y;
   for (int p = 0; p < 3; p++)
     pass_load<true>(ev + (size_t(p) * m + i) * N, gdit, gid0, sm + size_t(p) * 2 * E, SC_NONE, 0, tabs);
-  pass_stages<true, 3, R4>(sm, gdit, gid0, tw_fwd);
+  pass_stages<true, 3, R4, false>(sm, gdit, gid0, tw);
   const Fr zinv = ld_field(tabs.consts + 1);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
     const Fr a = f_red2(sm_get(sm, E, e)), b = f_red2(sm_get(sm + 2 * E, E, e)), c = f_red2(sm_get(sm + 4 * E, E, e));
     sm_put(sm, E, e, f_mul_lazy(f_sub2(f_mul_lazy(a, b), c), zinv));
   }
-  pass_stages<false, 1, R4>(sm, gdif, gid0, tw_inv);
+  pass_stages<false, 1, R4, true>(sm, gdif, gid0, tw);
   pass_store<false>(ev + (size_t(3) * m + i) * N, gdif, gid0, sm, SC_NONE, false, tabs);
 }
 
@@ -416,10 +478,12 @@ static std::once_flag g_smem_once;
 
 static void ntt_smem_attrs() {
   std::call_once(g_smem_once, [] {
-    cudaFuncSetAttribute(k_ntt_pass<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
+    cudaFuncSetAttribute(k_ntt_pass<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
     cudaFuncSetAttribute(k_ntt_turn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
     cudaFuncSetAttribute(k_ntt_turn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
     cudaFuncSetAttribute(k_ntt_quotient_turn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 << 10);
@@ -465,21 +529,15 @@ static PassShape pass_shape(uint32_t L, uint32_t k, int elog, int batch) {
 // twice the resident warps).
 static bool radix4(dim3 grid) { return uint64_t(grid.x) * grid.y < 4ull * (uint64_t)device_sm_count(); }
 
-static int launch_pass(bool dit, Fr* data, int batch, size_t bstride, const NttDomain* d, const Fr* tw, uint32_t s0,
+static int launch_pass(bool dit, Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse, uint32_t s0,
                        uint32_t k, int elog, int ls, int ss, int tm, cudaStream_t st) {
   const uint32_t L = d->logN;
   const PassShape sh = pass_shape(L, k, elog, batch);
-  const size_t smem = size_t(sh.E) * 32;
-  const ScaleTabs tabs = tabs_of(d);
   const bool r4 = radix4(sh.grid);
-  if (dit && r4)
-    k_ntt_pass<true, true><<<sh.grid, sh.threads, smem, st>>>(data, bstride, tw, L, s0, k, sh.logG, ls, ss, tm, tabs);
-  else if (dit)
-    k_ntt_pass<true, false><<<sh.grid, sh.threads, smem, st>>>(data, bstride, tw, L, s0, k, sh.logG, ls, ss, tm, tabs);
-  else if (r4)
-    k_ntt_pass<false, true><<<sh.grid, sh.threads, smem, st>>>(data, bstride, tw, L, s0, k, sh.logG, ls, ss, tm, tabs);
-  else
-    k_ntt_pass<false, false><<<sh.grid, sh.threads, smem, st>>>(data, bstride, tw, L, s0, k, sh.logG, ls, ss, tm, tabs);
+  auto* f = dit ? (r4 ? k_ntt_pass<true, true, false> : k_ntt_pass<true, false, false>)
+          : inverse ? (r4 ? k_ntt_pass<false, true, true> : k_ntt_pass<false, false, true>)
+                    : (r4 ? k_ntt_pass<false, true, false> : k_ntt_pass<false, false, false>);
+  f<<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(data, bstride, d->tw, L, s0, k, sh.logG, ls, ss, tm, tabs_of(d));
   ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   return ZKVC_OK;
@@ -492,11 +550,10 @@ static int run_passes(bool dit, Fr* data, int batch, size_t bstride, const NttDo
   ntt_smem_attrs();
   const std::vector<uint32_t> ks = pass_split(d->logN, elog);
   const uint32_t P = (uint32_t)ks.size();
-  const Fr* tw = inverse ? d->tw_inv : d->tw_fwd;
   uint32_t s0 = 0;
   for (uint32_t p = 0; p < P; p++) {
     const bool first = p == 0, last = p + 1 == P;
-    ZK_TRY(launch_pass(dit, data, batch, bstride, d, tw, s0, ks[p], elog, first ? load_scale : 0,
+    ZK_TRY(launch_pass(dit, data, batch, bstride, d, inverse, s0, ks[p], elog, first ? load_scale : 0,
                        last ? store_scale : 0, (first && raw) ? 1 : 0, st));
     s0 += ks[p];
   }
@@ -522,7 +579,7 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
   // inverse DIF transforms of A, B, C up to their last pass
   uint32_t s0 = 0;
   for (uint32_t p = 0; p + 1 < P; p++) {
-    ZK_TRY(launch_pass(false, ev, 3 * m, N, d, d->tw_inv, s0, ks[p], elog, 0, 0, 0, st));
+    ZK_TRY(launch_pass(false, ev, 3 * m, N, d, true, s0, ks[p], elog, 0, 0, 0, st));
     s0 += ks[p];
   }
   // turn: the inverse's last pass, x N^-1 g^i, the forward DIT's first pass
@@ -530,11 +587,9 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
     const uint32_t k = ks[P - 1];
     const PassShape sh = pass_shape(L, k, elog, 3 * m);
     if (radix4(sh.grid))
-      k_ntt_turn<true><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw_inv, d->tw_fwd, L, k, sh.logG,
-                                                                      SC_NG, tabs);
+      k_ntt_turn<true><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, SC_NG, tabs);
     else
-      k_ntt_turn<false><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw_inv, d->tw_fwd, L, k, sh.logG,
-                                                                       SC_NG, tabs);
+      k_ntt_turn<false><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, SC_NG, tabs);
     ZK_COUNT_LAUNCH();
     ZK_CUDA(cudaGetLastError());
   }
@@ -542,7 +597,7 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
   // groups of the DIF's pass P - 1 - q)
   uint32_t s0d = ks[P - 1];
   for (uint32_t q = 1; q + 1 < P; q++) {
-    ZK_TRY(launch_pass(true, ev, 3 * m, N, d, d->tw_fwd, s0d, ks[P - 1 - q], elog, 0, 0, 0, st));
+    ZK_TRY(launch_pass(true, ev, 3 * m, N, d, false, s0d, ks[P - 1 - q], elog, 0, 0, 0, st));
     s0d += ks[P - 1 - q];
   }
   // quotient turn: the forward's last pass of A, B, C, the quotient, the first inverse
@@ -556,18 +611,16 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
                              : radix4(sh.grid)                         ? sh.threads
                                                                        : std::min<uint32_t>(2 * sh.threads, 512);
     if (radix4(sh.grid))
-      k_ntt_quotient_turn<true><<<sh.grid, threads, size_t(3) * sh.E * 32, st>>>(ev, (uint32_t)m, N, d->tw_fwd,
-                                                                                 d->tw_inv, L, k, sh.logG, tabs);
+      k_ntt_quotient_turn<true><<<sh.grid, threads, size_t(3) * sh.E * 32, st>>>(ev, (uint32_t)m, N, d->tw, L, k, sh.logG, tabs);
     else
-      k_ntt_quotient_turn<false><<<sh.grid, threads, size_t(3) * sh.E * 32, st>>>(ev, (uint32_t)m, N, d->tw_fwd,
-                                                                                  d->tw_inv, L, k, sh.logG, tabs);
+      k_ntt_quotient_turn<false><<<sh.grid, threads, size_t(3) * sh.E * 32, st>>>(ev, (uint32_t)m, N, d->tw, L, k, sh.logG, tabs);
     ZK_COUNT_LAUNCH();
     ZK_CUDA(cudaGetLastError());
   }
   // the rest of h's inverse DIF transform, x N^-1 g^-i at the last store
   s0 = ks[0];
   for (uint32_t p = 1; p < P; p++) {
-    ZK_TRY(launch_pass(false, H, m, N, d, d->tw_inv, s0, ks[p], elog, 0, p + 1 == P ? SC_NGI : 0, 0, st));
+    ZK_TRY(launch_pass(false, H, m, N, d, true, s0, ks[p], elog, 0, p + 1 == P ? SC_NGI : 0, 0, st));
     s0 += ks[p];
   }
   return ZKVC_OK;
@@ -576,10 +629,6 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
 int ntt_dif(Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse, int load_scale,
             int store_scale, bool raw, cudaStream_t st, int elog) {
   return run_passes(false, data, batch, bstride, d, inverse, load_scale, store_scale, raw, elog, st);
-}
-
-int ntt_dit(Fr* data, int batch, size_t bstride, const NttDomain* d, bool inverse, cudaStream_t st, int elog) {
-  return run_passes(true, data, batch, bstride, d, inverse, 0, 0, false, elog, st);
 }
 
 // The element at bit-reversed position q, natural index p, on its way out: times the factor

@@ -5,13 +5,13 @@
 
 namespace zkvc {
 
-// Tables of one evaluation domain H = <omega_N>, N = 2^logN, all in Montgomery form and
+// Tables of one evaluation domain H = <omega_N>, N = 2^logN, in Montgomery form (but tw) and
 // resident on the device that built them.  The coset shift is g = 5.
 struct NttDomain {
   uint32_t logN = 0;
   size_t N = 0;
-  Fr* tw_fwd = nullptr;   // omega^e,  e < N/2
-  Fr* tw_inv = nullptr;   // omega^-e, e < N/2
+  Fr* tw = nullptr;       // per stage s: omega^(j 2^s), plain, j <= N / 2^(s + 1); then, for
+                          // all of them, floor(w 2^256 / r)
   Fr* g_lo = nullptr;     // g^l,           l < 1024
   Fr* gi_lo = nullptr;    // g^-l
   Fr* g_hi = nullptr;     // g^(1024 h),    h < max(1, N/1024)
@@ -44,10 +44,6 @@ int ntt_domain(uint32_t logN, const NttDomain** out);
 // elements a block stages in shared memory (8 .. 11; passes take min(elog, 10) stages).
 int ntt_dif(Fr* data, int batch, size_t batch_stride, const NttDomain* d, bool inverse, int load_scale,
             int store_scale, bool raw, cudaStream_t st, int elog = 10);
-
-// Decimation-in-time: bit-reversed input, natural-order output, in place.
-int ntt_dit(Fr* data, int batch, size_t batch_stride, const NttDomain* d, bool inverse, cudaStream_t st,
-            int elog = 10);
 
 // In-place bit-reversal permutation with an optional scale by natural index.
 int ntt_bitrev(Fr* data, const NttDomain* d, int scale, cudaStream_t st);

@@ -113,10 +113,11 @@ __global__ void k_zpows(const SetupConsts* sc, Fr* zA, int a, Fr* zB, int b) {
     st_field(zB + (t - a), pow_u32(z, (uint32_t)(t - a)));
 }
 
-// omega^k from the half table omega^e (e < N/2): omega^(k + N/2) = -omega^k
+// omega^k from the stage-0 table of plain omega^e (e <= N/2): omega^(k + N/2) = -omega^k
 __device__ __forceinline__ Fr omega_pow(const Fr* tw, size_t N, size_t k) {
   size_t h = N / 2;
-  return k < h ? ld_field(tw + k) : f_neg(ld_field(tw + (k - h)));
+  const Fr w = f_to_mont(ld_field(tw + (k < h ? k : k - h)));
+  return k < h ? w : f_neg(w);
 }
 
 __global__ void k_lagrange(const SetupConsts* sc, const Fr* tw, size_t N, uint32_t rows, Fr* L) {
@@ -499,7 +500,7 @@ int setup_impl(int a, int n, int b, const uint8_t* toxic, cudaStream_t st, zkvc_
   do {
     k_zpows<<<(sh.a + sh.b + 127) / 128, 128, 0, st>>>(d_sc, pk->zA, sh.a, pk->zB, sh.b); ZK_COUNT_LAUNCH();
     size_t lag_threads = (sh.rows + LAG_CHUNK - 1) / LAG_CHUNK;
-    k_lagrange<<<(unsigned)((lag_threads + 127) / 128), 128, 0, st>>>(d_sc, dom->tw_fwd, sh.N, sh.rows, d_L); ZK_COUNT_LAUNCH();
+    k_lagrange<<<(unsigned)((lag_threads + 127) / 128), 128, 0, st>>>(d_sc, dom->tw, sh.N, sh.rows, d_L); ZK_COUNT_LAUNCH();
     if (cudaGetLastError() != cudaSuccess) {
       rc = ZKVC_ECUDA;
       break;
