@@ -36,8 +36,13 @@ namespace zkvc {
 __host__ __device__ __forceinline__ size_t tw_offset(uint32_t L, uint32_t s) {
   return (size_t(1) << L) - (size_t(1) << (L - s)) + 4 * s;
 }
+// After them, at 2^t + j: the coset forms g^(2^s) omega^(j 2^s), s = L - 1 - t, of the DIT
+// stages t = 1 .. COSET_STAGES - 1; quotients this many entries further on
+constexpr uint32_t COSET_STAGES = 4;  // no transform of two passes has a shorter last pass
+__host__ __device__ __forceinline__ size_t tw_total(uint32_t L) { return tw_offset(L, L) + (1u << COSET_STAGES); }
 
 struct ScaleTabs {
+  const Fr* coset;
   const Fr* g_lo;
   const Fr* gi_lo;
   const Fr* g_hi;
@@ -139,16 +144,32 @@ __global__ void k_fill_twiddles(Fr* out, size_t total) {
   st_field(out + total + e, q);
 }
 
-// the tables of the stages s >= 1: every 2^s-th entry of stage 0's
-__global__ void k_fill_stages(Fr* out, uint32_t L) {
+// the tables of the stages s >= 1 (every 2^s-th entry of stage 0's) and the coset forms
+__global__ void k_fill_stages(Fr* out, uint32_t L, ScaleTabs tabs) {
   const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;  // 2^(L - 1 - s) + j, j < 2^(L - 1 - s); 0: the last entries
   if (e >= 1u << (L - 1)) return;
   if (e == 0) {
     for (uint32_t s = 1; s < L; s++) st_field(out + tw_offset(L, s) + (1u << (L - 1 - s)), ld_field(out + (1u << (L - 1))));
+    for (uint32_t k = 0; k < 1u << COSET_STAGES; k++) {
+      const uint32_t t = k < 2 ? 0u : 31 - __clz(k);
+      st_field(out + tw_offset(L, L) + k,
+               t && t < L ? f_mul(scale_factor(tabs, SC_G, 1u << (L - 1 - t)), ld_field(out + (size_t(k - (1u << t)) << (L - 1 - t))))
+                          : Fr::zero());
+    }
     return;
   }
   const uint32_t lg = 31 - __clz(e), s = L - 1 - lg, j = e - (1u << lg);
   if (s >= 1) st_field(out + tw_offset(L, s) + j, ld_field(out + (size_t(j) << s)));
+}
+
+// The factors left of N^-1 g^i when the DIT's first COSET_STAGES stages run in coset form:
+// for position p (natural index i = bit-reversed p) N^-1 g^(i mod N / 16), times g^(N/2) for
+// odd p (stage 0's coset factor, so that stage keeps no product); entry 2 (p / 16) + p mod 2.
+__global__ void k_fill_coset(Fr* out, uint32_t L, ScaleTabs tabs) {
+  const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x, lb = L - COSET_STAGES;
+  if (e >= 2u << lb) return;
+  const Fr c = scale_factor(tabs, SC_NG, brev_bits(e >> 1, lb));
+  st_field(out + e, (e & 1u) ? f_mul(c, scale_factor(tabs, SC_G, 1u << (L - 1))) : c);
 }
 
 static int fill_pows(Fr* out, size_t count, const Fr* base, const Fr* mult, cudaStream_t st) {
@@ -157,6 +178,10 @@ static int fill_pows(Fr* out, size_t count, const Fr* base, const Fr* mult, cuda
   k_fill_pows<<<blocks, 128, 0, st>>>(out, count, base, mult); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   return ZKVC_OK;
+}
+
+static ScaleTabs tabs_of(const NttDomain* d) {
+  return {d->coset, d->g_lo, d->gi_lo, d->g_hi, d->g_hi_n, d->gi_hi_n, d->consts};
 }
 
 static std::mutex g_dom_mu;
@@ -180,7 +205,9 @@ int ntt_domain(uint32_t logN, const NttDomain** out) {
   cudaStream_t st;
   ZK_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   ZK_CUDA(cudaMalloc(&d->consts, 16 * sizeof(Fr)));
-  ZK_CUDA(cudaMalloc(&d->tw, 2 * tw_offset(logN, logN) * sizeof(Fr)));
+  const size_t total = tw_total(logN), ncoset = logN > COSET_STAGES ? size_t(2) << (logN - COSET_STAGES) : 0;
+  ZK_CUDA(cudaMalloc(&d->tw, 2 * total * sizeof(Fr)));
+  if (ncoset) ZK_CUDA(cudaMalloc(&d->coset, 2 * ncoset * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->g_lo, 1024 * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->gi_lo, 1024 * sizeof(Fr)));
   ZK_CUDA(cudaMalloc(&d->g_hi, hi * sizeof(Fr)));
@@ -190,23 +217,24 @@ int ntt_domain(uint32_t logN, const NttDomain** out) {
   ZK_CUDA(cudaGetLastError());
   const Fr* c = d->consts;
   ZK_TRY(fill_pows(d->tw, half + 1, c + 2, c + 8, st));
-  k_fill_stages<<<(unsigned)((half + 255) / 256), 256, 0, st>>>(d->tw, logN); ZK_COUNT_LAUNCH();
-  k_fill_twiddles<<<(unsigned)((tw_offset(logN, logN) + 255) / 256), 256, 0, st>>>(d->tw, tw_offset(logN, logN)); ZK_COUNT_LAUNCH();
-  ZK_CUDA(cudaGetLastError());
   ZK_TRY(fill_pows(d->g_lo, 1024, c + 4, c + 8, st));
   ZK_TRY(fill_pows(d->gi_lo, 1024, c + 5, c + 8, st));
   ZK_TRY(fill_pows(d->g_hi, hi, c + 6, c + 8, st));
   ZK_TRY(fill_pows(d->g_hi_n, hi, c + 6, c + 0, st));
   ZK_TRY(fill_pows(d->gi_hi_n, hi, c + 7, c + 0, st));
+  const ScaleTabs tabs = tabs_of(d);
+  k_fill_stages<<<(unsigned)((half + 255) / 256), 256, 0, st>>>(d->tw, logN, tabs); ZK_COUNT_LAUNCH();
+  k_fill_twiddles<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(d->tw, total); ZK_COUNT_LAUNCH();
+  if (ncoset) {
+    k_fill_coset<<<(unsigned)((ncoset + 255) / 256), 256, 0, st>>>(d->coset, logN, tabs); ZK_COUNT_LAUNCH();
+    k_fill_twiddles<<<(unsigned)((ncoset + 255) / 256), 256, 0, st>>>(d->coset, ncoset); ZK_COUNT_LAUNCH();
+  }
+  ZK_CUDA(cudaGetLastError());
   ZK_CUDA(cudaStreamSynchronize(st));
   ZK_CUDA(cudaStreamDestroy(st));
   g_domains[{dev, logN}] = d;
   *out = d;
   return ZKVC_OK;
-}
-
-static ScaleTabs tabs_of(const NttDomain* d) {
-  return {d->g_lo, d->gi_lo, d->g_hi, d->g_hi_n, d->gi_hi_n, d->consts};
 }
 
 // One pass: k consecutive radix-2 stages from stage s0, over G = 2^logG groups of 2^k
@@ -296,7 +324,7 @@ __device__ __forceinline__ void pass_store(Fr* arr, const PassGeo& g, uint32_t g
 // the entry as far from the table's end, so the difference is taken the other way round.  The
 // transform's stage of half 1 over neighbouring elements (DIF s = L - 1, DIT s = 0) has
 // w = 1 throughout and takes no product.
-template <bool DIT, int NPOLY, bool R4, bool INV>
+template <bool DIT, int NPOLY, bool R4, bool INV, bool COSET = false>
 __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_t gid0, const Fr* tw) {
   const uint32_t G = 1u << g.logG, E = G << g.k, L = g.L, logG = g.logG;
   const uint32_t sbits = DIT ? g.s0 : (L - g.s0 - g.k);
@@ -304,13 +332,17 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
   static_assert(!(DIT && INV), "the forward transforms alone run by decimation in time");
   // the table of stage s and its entry for a butterfly
   auto stage_tab = [&](uint32_t s) -> const Fr* {
+    if (COSET && s > 0 && s < COSET_STAGES) return tw + tw_offset(L, L) + (1u << s);
     const uint32_t sd = DIT ? L - 1 - s : s;
     return tw + tw_offset(L, sd) + (INV ? 1u << (L - 1 - sd) : 0u);
   };
-  const size_t total = tw_offset(L, L);
-  auto mul_tw = [&](const Fr& x, const Fr* tab, uint32_t q, uint32_t lo) -> Fr {
+  const size_t total = tw_total(L);
+  auto entry = [&](const Fr* tab, uint32_t q, uint32_t lo) -> const Fr* {
     const uint32_t p = DIT ? (q << g.s0) + lo : (q << sbits) + lo;
-    const Fr* w = INV ? tab - p : tab + p;
+    return INV ? tab - p : tab + p;
+  };
+  auto mul_tw = [&](const Fr& x, const Fr* tab, uint32_t q, uint32_t lo) -> Fr {
+    const Fr* w = entry(tab, q, lo);
     return f_mul_const(x, ld_field(w), ld_field(w + total));
   };
   auto diff = [&](const Fr& x, const Fr& y) -> Fr { return INV ? f_sub2(y, x) : f_sub2(x, y); };
@@ -383,22 +415,44 @@ __device__ __forceinline__ void pass_stages(uint4* sm, const PassGeo& g, uint32_
     const Fr* tab = stage_tab(s);
     const uint32_t logh = DIT ? t : (g.k - 1 - t), h = 1u << logh;
     const bool unit = DIT ? s == 0 : s == L - 1;
-    for (uint32_t bfa = threadIdx.x; bfa < nbf * (uint32_t)NPOLY; bfa += blockDim.x) {
-      const uint32_t poly = NPOLY == 1 ? 0u : bfa / nbf, bf = bfa - poly * nbf;
-      uint4* smp = sm + size_t(poly) * 2 * E;
+    auto place = [&](uint32_t bf, uint32_t& pu, uint32_t& pv, uint32_t& qh, uint32_t& lo) {
       const uint32_t gg = bf & (G - 1), q = bf >> logG;
-      const uint32_t qh = q & (h - 1);
+      qh = q & (h - 1);
       const uint32_t ju = ((q >> logh) << (logh + 1)) + qh;
-      const uint32_t pu = (ju << logG) + gg, pv = ((ju + h) << logG) + gg;
-      const uint32_t lo = (gid0 + gg) & smask;
-      const Fr u = sm_get(smp, E, pu), v = sm_get(smp, E, pv);
+      pu = (ju << logG) + gg;
+      pv = ((ju + h) << logG) + gg;
+      lo = (gid0 + gg) & smask;
+    };
+    auto butterfly = [&](uint4* smp, uint32_t pu, uint32_t pv, auto&& mul) {
+      const Fr v = sm_get(smp, E, pv);
       if (DIT) {
-        const Fr x = f_red2(u), y = unit ? f_red2(v) : mul_tw(v, tab, qh, lo);
+        const Fr y = unit ? f_red2(v) : mul(v), x = f_red2(sm_get(smp, E, pu));
         sm_put(smp, E, pu, f_add_raw(x, y));
         sm_put(smp, E, pv, f_sub2(x, y));
       } else {
+        const Fr u = sm_get(smp, E, pu);
         sm_put(smp, E, pu, f_add2(u, v));
-        sm_put(smp, E, pv, unit ? f_red2(f_sub2(u, v)) : mul_tw(diff(u, v), tab, qh, lo));
+        sm_put(smp, E, pv, unit ? f_red2(f_sub2(u, v)) : mul(diff(u, v)));
+      }
+    };
+    if (NPOLY > 1 && !R4) {
+      // a thread takes a butterfly's place in each array, for one read of its twiddle
+      // (quotient turns of a 64-proof batch: 4,976 us with the arrays side by side, 4,716 so)
+      for (uint32_t bf = threadIdx.x; bf < nbf; bf += blockDim.x) {
+        uint32_t pu, pv, qh, lo;
+        place(bf, pu, pv, qh, lo);
+        const Fr* w = entry(tab, qh, lo);
+        const Fr w0 = ld_field(w), w1 = ld_field(w + total);
+#pragma unroll 1
+        for (uint32_t p = 0; p < NPOLY; p++)
+          butterfly(sm + size_t(p) * 2 * E, pu, pv, [&](const Fr& x) { return f_mul_const(x, w0, w1); });
+      }
+    } else {
+      for (uint32_t bfa = threadIdx.x; bfa < nbf * (uint32_t)NPOLY; bfa += blockDim.x) {
+        const uint32_t poly = NPOLY == 1 ? 0u : bfa / nbf;
+        uint32_t pu, pv, qh, lo;
+        place(bfa - poly * nbf, pu, pv, qh, lo);
+        butterfly(sm + size_t(poly) * 2 * E, pu, pv, [&](const Fr& x) { return mul_tw(x, tab, qh, lo); });
       }
     }
     __syncthreads();
@@ -426,24 +480,28 @@ __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
 
 // The turn of an inverse DIF transform into a forward DIT transform, in one pass: the
 // DIF's last pass (its k stages end at stage L - 1, groups of 2^k consecutive elements),
-// the inverse's scaling by the factor of each element's natural index, and the DIT's
-// first pass over the same groups.  Saves a global round trip and a launch.
+// the inverse's scaling by N^-1 and the coset's powers g^i, and the DIT's first pass over the
+// same groups.  Saves a global round trip and a launch.  Most of g^i goes into the twiddles of
+// the DIT's first stages (k_fill_coset), which leaves one product by a constant per element
+// out of a table of N / 8 (two Montgomery products before: the turns of a 64-proof batch took
+// 5,756 us, 5,172 so).
 template <bool R4>
 __global__ void __launch_bounds__(256, pass_min_blocks<R4>())
     k_ntt_turn(Fr* data, size_t bstride, const Fr* __restrict__ tw, uint32_t L, uint32_t k,
-               uint32_t logG, int mid_scale, ScaleTabs tabs) {
+               uint32_t logG, ScaleTabs tabs) {
   extern __shared__ uint4 sm[];
   const PassGeo gdif{L, L - k, k, logG}, gdit{L, 0, k, logG};
   Fr* arr = data + size_t(blockIdx.y) * bstride;
   const uint32_t gid0 = blockIdx.x << logG;
-  const uint32_t E = 1u << (logG + k);
+  const uint32_t E = 1u << (logG + k), ncoset = 2u << (L - COSET_STAGES);
   pass_load<false>(arr, gdif, gid0, sm, SC_NONE, 0, tabs);
   pass_stages<false, 1, R4, true>(sm, gdif, gid0, tw);
   for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
     const uint32_t idx = pass_index<false>(gdif, gid0, e);
-    sm_put(sm, E, e, f_mul_lazy(scale_factor(tabs, mid_scale, brev_bits(idx, L)), sm_get(sm, E, e)));
+    const Fr* c = tabs.coset + 2 * (idx / (1u << COSET_STAGES)) + (idx & 1u);
+    sm_put(sm, E, e, f_mul_const(sm_get(sm, E, e), ld_field(c), ld_field(c + ncoset)));
   }
-  pass_stages<true, 1, R4, false>(sm, gdit, gid0, tw);
+  pass_stages<true, 1, R4, false, true>(sm, gdit, gid0, tw);
   pass_store<true>(arr, gdit, gid0, sm, SC_NONE, false, tabs);
 }
 
@@ -587,9 +645,9 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
     const uint32_t k = ks[P - 1];
     const PassShape sh = pass_shape(L, k, elog, 3 * m);
     if (radix4(sh.grid))
-      k_ntt_turn<true><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, SC_NG, tabs);
+      k_ntt_turn<true><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, tabs);
     else
-      k_ntt_turn<false><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, SC_NG, tabs);
+      k_ntt_turn<false><<<sh.grid, sh.threads, size_t(sh.E) * 32, st>>>(ev, N, d->tw, L, k, sh.logG, tabs);
     ZK_COUNT_LAUNCH();
     ZK_CUDA(cudaGetLastError());
   }

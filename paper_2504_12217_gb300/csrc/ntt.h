@@ -5,13 +5,14 @@
 
 namespace zkvc {
 
-// Tables of one evaluation domain H = <omega_N>, N = 2^logN, in Montgomery form (but tw) and
-// resident on the device that built them.  The coset shift is g = 5.
+// Tables of one evaluation domain H = <omega_N>, N = 2^logN, resident on the device that
+// built them; Montgomery form but for tw and coset.  The coset shift is g = 5.
 struct NttDomain {
   uint32_t logN = 0;
   size_t N = 0;
   Fr* tw = nullptr;       // per stage s: omega^(j 2^s), plain, j <= N / 2^(s + 1); then, for
                           // all of them, floor(w 2^256 / r)
+  Fr* coset = nullptr;    // factors of the coset turn (k_fill_coset) and their quotients
   Fr* g_lo = nullptr;     // g^l,           l < 1024
   Fr* gi_lo = nullptr;    // g^-l
   Fr* g_hi = nullptr;     // g^(1024 h),    h < max(1, N/1024)
