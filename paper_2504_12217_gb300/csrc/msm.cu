@@ -4,7 +4,10 @@
 // Scalars are recoded into signed c-bit digits d in (-2^(c-1), 2^(c-1)], so a digit
 // selects bucket |d| and the sign negates the base's y coordinate.  Every nonzero digit
 // becomes one term (bucket key, base index | sign).  Terms are counting-sorted by key
-// (histogram, scan, atomic scatter), then the sorted terms are summed by a balanced
+// (counts, scan, scatter; the ranks within a bucket come from the counting atomics where
+// digits spread over many buckets).  Large runs first halve every bucket a few times by
+// affine additions that share their inversions (k_tree below, 6 products per addition
+// instead of 10).  Then the sorted terms are summed by a balanced
 // segmented reduction: every chunk of T0 consecutive sorted terms goes to one thread
 // (mixed XYZZ + affine additions), which stores a partial sum each time a bucket ends
 // inside its chunk, so every thread does the same number of additions whatever the
@@ -16,8 +19,9 @@
 // buckets whose index has bit b set: one block per slice of a bit's buckets reduces it
 // in shared memory, one block per bit adds the slices and doubles b times, one block per
 // window adds the bits -- log-depth instead of a running sum, since a point addition is
-// long-latency on the GPU (about 10 us for one thread).  Where few sums remain, the
-// additions and doublings run on quads of lanes (coop.cuh).
+// long-latency on the GPU (about 7 us for one thread).  Where few sums remain, the
+// additions run on quads of lanes (coop.cuh) and the doublings on a warp (sliced.cuh,
+// fp2_rounds.cuh).
 //
 // Fixed-base MSMs (proving-key queries) store the multiples 2^(c w) P of each base, so all
 // windows share one bucket set and no doubling chain follows; variable-base MSMs keep
@@ -1020,7 +1024,7 @@ __global__ void __launch_bounds__(256, AccumMinB<F>::value) k_accum0(const uint3
 
 // Buckets with at most FOLD_SERIAL partial sums (the common case of a balanced
 // accumulation: a bucket split by one or two chunk boundaries) are folded by one thread
-// (or quad) per bucket, serially, without counters; the tree (fold_tree_at) takes the
+// or quad (QL lanes) per bucket, serially, without counters; the tree (fold_tree_at) takes the
 // larger ones.
 // Where chunk boundaries are fewer than buckets (large chunks over many small buckets),
 // the quads go over the boundaries' fold list instead (flist non-null, nlist entries), so
@@ -1119,16 +1123,27 @@ __device__ __forceinline__ void fold_tree_at(uint32_t q, const uint32_t* __restr
 }
 
 // Both folds in one launch (disjoint buckets: at most FOLD_SERIAL partials go serially,
-// more along the tree): quad (or thread) i takes serial entry i (bucket i, or boundary i
-// of the fold list) and tree slot i.
-template <class F, int QL>
+// more along the tree): the first sblocks blocks take the serial entries (entry i: bucket i,
+// or boundary i of the fold list) on SL lanes each, the others a tree slot per quad.
+//
+// What bounds it: the latency of two or three additions one after another.  A quad's
+// addition takes half a thread's time, but more than FOLD_QUADS quads are several waves
+// of them, where as many threads are one: the folds of 32,768 buckets (H query,
+// [49,320]x[320,512]) FOLDH us on threads, 55.7 on quads; of 40,960 buckets in G2 (65,536
+// points) FOLDG2, 184 on quads.
+constexpr uint64_t FOLD_QUADS = 16384;
+template <class F, int SL>
 __global__ void __launch_bounds__(128) k_fold(const uint32_t* __restrict__ choff, const uint32_t* __restrict__ nch,
                                               const uint32_t* __restrict__ chunk_key, uint32_t K, XYZZ<F>* part,
                                               uint32_t* arrive, const uint32_t* __restrict__ flist, uint32_t nlist,
-                                              const uint32_t* __restrict__ offs, uint32_t T0, uint32_t n_serial) {
-  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / QL;
-  if (i < n_serial) fold_serial_at<F, QL>(i, choff, nch, K, part, flist, nlist, offs, T0);
-  fold_tree_at<F, QL>(i, choff, nch, chunk_key, K, part, arrive);
+                                              const uint32_t* __restrict__ offs, uint32_t T0, uint32_t n_serial,
+                                              uint32_t sblocks) {
+  if (blockIdx.x < sblocks) {
+    const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / SL;
+    if (i < n_serial) fold_serial_at<F, SL>(i, choff, nch, K, part, flist, nlist, offs, T0);
+  } else {
+    fold_tree_at<F, 4>(((blockIdx.x - sblocks) * blockDim.x + threadIdx.x) / 4, choff, nch, chunk_key, K, part, arrive);
+  }
 }
 
 template <class F>
@@ -1703,12 +1718,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   XYZZ<F>* part = reinterpret_cast<XYZZ<F>*>(L.part);
   const uint32_t at = p.tune.accum_threads;
   const int lanes = p.lanes == 4 ? 4 : 1;
-  // the folds run on quads whatever the accumulation uses: after a balanced accumulation
-  // they only see a few partial sums per bucket (or few, large buckets), so they are
-  // latency-bound, and a quad's addition has a third of a lone thread's latency
-  const int flanes = 4;
   unsigned qb = (unsigned)((uint64_t(L.qmax) * lanes + at - 1) / at);
-  unsigned fb = (unsigned)((uint64_t(L.qmax) * flanes + 127) / 128);
   if (accum_stage >= 0) prof_mark(accum_stage, true, st);
   const auto* ob = reinterpret_cast<const Affine<F>* const*>(L.obases);
   if (R) {
@@ -1748,14 +1758,11 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   const bool by_boundary = nlist < K;
   const uint32_t* fl = by_boundary ? L.flist : nullptr;
   const uint64_t n_serial = by_boundary ? nlist : uint64_t(K);
-  const unsigned sfb = (unsigned)((n_serial * flanes + 127) / 128);
-  const unsigned fab = std::max(sfb, fb);
-  if (flanes == 4)
-    k_fold<F, 4><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0,
-                                      (uint32_t)n_serial);
-  else
-    k_fold<F, 1><<<fab, 128, 0, st>>>(L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0,
-                                      (uint32_t)n_serial);
+  const int slanes = n_serial > FOLD_QUADS ? 1 : 4;
+  const unsigned sblocks = (unsigned)((n_serial * slanes + 127) / 128);
+  const unsigned tblocks = (unsigned)((uint64_t(L.qmax) * 4 + 127) / 128);
+  (slanes == 4 ? k_fold<F, 4> : k_fold<F, 1>)<<<sblocks + tblocks, 128, 0, st>>>(
+      L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0, (uint32_t)n_serial, sblocks);
   ZK_COUNT_LAUNCH();
   // sum_v v B_v per (output, window) by bit decomposition
   XYZZ<F>* Sl = reinterpret_cast<XYZZ<F>*>(L.S);
