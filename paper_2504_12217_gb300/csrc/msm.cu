@@ -1128,9 +1128,11 @@ __device__ __forceinline__ void fold_tree_at(uint32_t q, const uint32_t* __restr
 //
 // What bounds it: the latency of two or three additions one after another.  A quad's
 // addition takes half a thread's time, but more than FOLD_QUADS quads are several waves
-// of them, where as many threads are one: the folds of 32,768 buckets (H query,
-// [49,320]x[320,512]) FOLDH us on threads, 55.7 on quads; of 40,960 buckets in G2 (65,536
-// points) FOLDG2, 184 on quads.
+// of them, where as many threads are one.  And where there are many slots most have no part
+// in the tree, so a thread looks at each and the block's quads take those that have.
+// Measured: H query of [49,320]x[320,512] (32,768 buckets) 49 us, 55.7 with a quad per bucket
+// and slot; 65,536 points in G1 61.5 (75.8), in G2 163 (184); the rest query of a fold-mode
+// proof of [63,333]x[333,517] 105 (126); a 64-proof batch's main run 111 (259).
 constexpr uint64_t FOLD_QUADS = 16384;
 template <class F, int SL>
 __global__ void __launch_bounds__(128) k_fold(const uint32_t* __restrict__ choff, const uint32_t* __restrict__ nch,
@@ -1141,8 +1143,22 @@ __global__ void __launch_bounds__(128) k_fold(const uint32_t* __restrict__ choff
   if (blockIdx.x < sblocks) {
     const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / SL;
     if (i < n_serial) fold_serial_at<F, SL>(i, choff, nch, K, part, flist, nlist, offs, T0);
-  } else {
+  } else if (SL == 4) {
     fold_tree_at<F, 4>(((blockIdx.x - sblocks) * blockDim.x + threadIdx.x) / 4, choff, nch, chunk_key, K, part, arrive);
+  } else {
+    // many slots, few of them in the tree: a thread looks at each, quads take those that are;
+    // a block's warps look far apart, since the slots of large buckets lie side by side
+    __shared__ uint32_t list[128], n;
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    const uint32_t q = ((threadIdx.x / 32) * (gridDim.x - sblocks) + blockIdx.x - sblocks) * 32 + threadIdx.x % 32;
+    if (q < choff[K]) {
+      const uint32_t k = chunk_key[q];
+      if (k < K && q - choff[k] < nch[k] && nch[k] > FOLD_SERIAL) list[atomicAdd(&n, 1u)] = q;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x / 4; i < n; i += blockDim.x / 4)
+      fold_tree_at<F, 4>(list[i], choff, nch, chunk_key, K, part, arrive);
   }
 }
 
@@ -1760,7 +1776,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   const uint64_t n_serial = by_boundary ? nlist : uint64_t(K);
   const int slanes = n_serial > FOLD_QUADS ? 1 : 4;
   const unsigned sblocks = (unsigned)((n_serial * slanes + 127) / 128);
-  const unsigned tblocks = (unsigned)((uint64_t(L.qmax) * 4 + 127) / 128);
+  const unsigned tblocks = (unsigned)((uint64_t(L.qmax) * slanes + 127) / 128);
   (slanes == 4 ? k_fold<F, 4> : k_fold<F, 1>)<<<sblocks + tblocks, 128, 0, st>>>(
       L.choff, L.nch, L.chunk_key, K, part, L.arrive, fl, (uint32_t)nlist, offs, T0, (uint32_t)n_serial, sblocks);
   ZK_COUNT_LAUNCH();
