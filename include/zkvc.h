@@ -22,7 +22,10 @@
  *  - Every function returns ZKVC_OK (0) or a negative status; zkvc_last_error() then
  *    describes the failure (thread-local, valid until the next call on that thread).
  *  - Workspaces are caller-provided device buffers of at least the size the matching
- *    *_workspace_bytes() function reports; the library never allocates inside a call
+ *    *_workspace_bytes() function reports (MSMs and proofs also run, more slowly, in the
+ *    part of it that remains without the pairwise affine rounds' points and with chunks of
+ *    16 terms: the size that versions without these asked for; less returns ZKVC_EINVAL);
+ *    the library never allocates inside a call
  *    that takes a workspace, except for a per-device domain table built once on first
  *    use of each NTT size (so warm up before capturing such a call in a CUDA graph).
  */

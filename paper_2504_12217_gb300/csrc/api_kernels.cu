@@ -192,10 +192,10 @@ static uint32_t window_bits(size_t n) {
 template <class F>
 constexpr bool msm_api_glv() { return true; }
 
-static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* out, bool affine = true) {
+static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* out, bool lean = false) {
   MsmPlan& p = *out;
   p = MsmPlan();
-  p.affine = affine;
+  p.lean = lean;
   const size_t pts = glv ? 2 * n : n;
   const uint32_t bits = glv ? 128 : 255;
   // the window rule's c, then the smallest c with the same window count, so that the top
@@ -219,11 +219,11 @@ static int variable_base_plan(size_t n, const void* scalars, bool glv, MsmPlan* 
 }
 
 template <class F>
-size_t msm_api_ws(size_t n, bool affine) {
+size_t msm_api_ws(size_t n, bool lean) {
   constexpr bool glv = msm_api_glv<F>();
   const size_t pts = glv ? 2 * n : n;
   MsmPlan p;
-  if (n > ZKVC_MSM_MAX_POINTS || variable_base_plan(n, nullptr, glv, &p, affine) != ZKVC_OK) return 0;
+  if (n > ZKVC_MSM_MAX_POINTS || variable_base_plan(n, nullptr, glv, &p, lean) != ZKVC_OK) return 0;
   return msm_workspace_bytes<F>(p) + round256(pts * sizeof(Affine<F>)) + (glv ? round256(pts * sizeof(uint4)) : 0) +
          2 * 256 + sizeof(XYZZ<F>) + sizeof(Affine<F>);
 }
@@ -312,9 +312,9 @@ int msm_api(const uint8_t* d_points, const uint8_t* d_scalars, size_t n, void* d
   MsmPlan p;
   ZK_TRY(variable_base_plan(n, nullptr, glv, &p));
   size_t need = msm_api_ws<F>(n);
-  if (ws_bytes < need && p.rounds) {  // short scratch: without the affine rounds
-    ZK_TRY(variable_base_plan(n, nullptr, glv, &p, false));
-    need = msm_api_ws<F>(n, false);
+  if (ws_bytes < need) {
+    ZK_TRY(variable_base_plan(n, nullptr, glv, &p, true));
+    need = msm_api_ws<F>(n, true);
   }
   ZK_CHECK(ws_bytes >= need, ZKVC_EINVAL, "msm: workspace %zu < %zu bytes", ws_bytes, need);
   Arena a;

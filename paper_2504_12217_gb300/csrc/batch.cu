@@ -186,7 +186,7 @@ struct zkvc_batch {
   uint8_t* dproofs = nullptr;
   std::vector<NttGroup> groups;
   MsmPlan p_small, p_main, p_g2;
-  bool lean = false;  // MSM runs without affine rounds, for memory too small for them
+  bool lean = false;  // MSM runs in their smaller form, for memory too small for the other
   MsmExec x_small, x_main, x_g2;
   void *ws_small = nullptr, *ws_main = nullptr, *ws_g2 = nullptr;
   size_t ws_small_bytes = 0, ws_main_bytes = 0, ws_g2_bytes = 0;
@@ -254,7 +254,7 @@ static void batch_plans(zkvc_batch* B) {
   B->p_small = MsmPlan();
   B->p_main = MsmPlan();
   B->p_g2 = MsmPlan();
-  B->p_small.affine = B->p_main.affine = B->p_g2.affine = !B->lean;
+  B->p_small.lean = B->p_main.lean = B->p_g2.lean = B->lean;
   for (int i = 0; i < B->count; i++) {
     const zkvc_pk* pk = B->pks[i];
     const Shape& sh = pk->shape;

@@ -1007,7 +1007,7 @@ static void gen_plans(const GenericKey& G, const void* src[G_COUNT], const Fr* h
     if (G.B2[g].count) P->g2.segs.push_back(gseg(G.B2[g], sh.count[g], 0, sh.kind[g], src[g]));
   P->g2.segs.push_back(gseg(G.BETA2, 1, 0, SK_ONE, nullptr));
   P->g2.segs.push_back(gseg(G.DELTA2, 1, 0, SK_FR_CANON, rs + 1));
-  P->pre.affine = P->h.affine = P->g2.affine = !lean;
+  P->pre.lean = P->h.lean = P->g2.lean = lean;
   msm_plan_finalize(P->pre);
   msm_plan_finalize(P->h);
   msm_plan_finalize(P->g2);
@@ -1018,7 +1018,7 @@ static size_t aux_bytes(const GShape& sh) {
   return std::max<size_t>(1, sh.n_aux) * e;
 }
 
-// lean: MSM runs without affine rounds, for a workspace too small for them
+// lean: MSM runs in their smaller form, for a workspace too small for the other
 static size_t gen_carve(const zkvc_pk* pk, void* base, size_t cap, GenBufs* B, bool measuring, bool lean) {
   const GenericKey& G = *pk->gen;
   const GShape& sh = G.sh;

@@ -264,13 +264,14 @@ int msm_plan_finalize(MsmPlan& p) {
   // term indices, bucket offsets and chunk bounds are 32-bit: 2^31 slots leave every sum
   // of an index and a chunk length below 2^32
   ZK_CHECK(slot <= (1ull << 31), ZKVC_EINVAL, "msm: %llu digit slots (at most 2^31)", (unsigned long long)slot);
-  p.rounds = p.affine ? tree_rounds(slot, key, base_end) : 0;
+  p.rounds = p.lean ? 0 : tree_rounds(slot, key, base_end);
   p.pad_slots = p.rounds ? key * ((1u << p.rounds) - 1u) : 0u;
   // default chunk: about two chunks per bucket, but at least ~40 k chunks so that the
   // accumulation fills the GPU, and 16 at the least (8 after affine rounds, where level 0
   // is a small part; 8 or 4 for runs of up to a few thousand chunks, where a
   // chunk's serial additions are the run's latency: a proof of [4,16] x [16,8] 467 us with
-  // 16, 362 with 8, 326 with 4); and at least the chunk that puts every point into one wave of
+  // 16, 362 with 8, 326 with 4; every chunk is a partial sum more, so the lean form keeps
+  // 16); and at least the chunk that puts every point into one wave of
   // resident accumulation threads (the chunks are balanced, so a second, partial wave
   // would only add a tail).  Counted in the points that the affine rounds leave.
   const uint64_t pts0 = (slot + p.pad_slots) >> p.rounds;
@@ -284,7 +285,8 @@ int msm_plan_finalize(MsmPlan& p) {
     // (7/8 of the resident threads: the prover's other streams hold some SM slots)
     const uint64_t resident = accum_resident_threads(p.tune.accum_threads) * 7 / 8;
     const uint64_t one_wave = resident ? (pts0 + resident - 1) / resident : 0;
-    const uint64_t least = p.rounds                     ? 8
+    const uint64_t least = p.lean                       ? 16
+                           : p.rounds                   ? 8
                            : slot < MSM_SMALL_TERMS / 8 ? p.tune.floor
                            : slot < MSM_SMALL_TERMS     ? 8
                                                         : p.tune.least;

@@ -53,9 +53,10 @@ struct MsmTune {
 
 struct MsmPlan {
   MsmTune tune;
-  bool affine = true;          // affine rounds where the run is large enough; without them it
-                               // needs about a quarter of the workspace (the prover and the
-                               // MSM entries fall back to that when the scratch is short)
+  bool lean = false;           // the smaller workspace: no affine rounds (large runs: about a
+                               // quarter) and default chunks of 16 terms at the least, so
+                               // fewer partial sums (small runs: down to two thirds); the
+                               // prover and the MSM entries fall back to it
   std::vector<MsmSeg> segs;
   std::vector<MsmOut> outs;
   uint64_t slots = 0;
@@ -118,7 +119,7 @@ template <class F>
 int msm_api(const uint8_t* d_points, const uint8_t* d_scalars, size_t n, void* d_ws, size_t ws_bytes,
             uint8_t* out, cudaStream_t st);
 template <class F>
-size_t msm_api_ws(size_t n, bool affine = true);
+size_t msm_api_ws(size_t n, bool lean = false);
 
 // Exclusive scan of n uint32 values into out[0..n] (out[n] = total); temp from the arena;
 // copy (if non-null) receives out[0..n) as well.

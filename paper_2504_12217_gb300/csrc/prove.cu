@@ -311,7 +311,7 @@ static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* 
       seg_of(g2[R2_BETA], 0, 1, 0, SK_ONE, nullptr),
       seg_of(g2[R2_DELTA], 0, 1, 0, SK_FR_CANON, rs + 1),
   };
-  P->small.affine = P->rest.affine = P->h.affine = P->g2.affine = !lean;
+  P->small.lean = P->rest.lean = P->h.lean = P->g2.lean = lean;
   P->small.tune.chunk = pk->prove_tune[0];
   P->rest.tune.chunk = pk->prove_tune[1];
   P->h.tune.chunk = pk->prove_tune[2];
@@ -330,7 +330,7 @@ static void plans(const zkvc_pk* pk, int mode, const int8_t* dX, const int32_t* 
   msm_plan_finalize(P->g2);
 }
 
-// lean: MSM runs without affine rounds, for a workspace too small for them
+// lean: MSM runs in their smaller form, for a workspace too small for the other
 static size_t carve(const zkvc_pk* pk, int mode, void* base, size_t cap, ProveBufs* B, bool measuring, bool lean) {
   const Shape& sh = pk->shape;
   const bool chain = mode == ZKVC_PROVE_CHAIN;
