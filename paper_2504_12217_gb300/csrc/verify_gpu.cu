@@ -398,7 +398,13 @@ int verify_batch_impl(const zkvc_vk* const* vks, const int8_t* const* X, const i
     ZK_TRY(msm_plan_finalize(plan));
     size_t wsb = msm_workspace_bytes<Fp>(plan);
     uint8_t* ws = nullptr;
-    ZK_TRY(buf.get(&ws, wsb));
+    if (buf.get(&ws, wsb) != ZKVC_OK) {  // once more with the run's smaller form
+      plan.lean = true;
+      ZK_TRY(msm_plan_finalize(plan));
+      wsb = msm_workspace_bytes<Fp>(plan);
+      ZK_TRY(buf.get(&ws, wsb));
+      set_error("%s", "");
+    }
     ZK_TRY(buf.part(&d_msm, plan.outs.size()));
     ZK_TRY(msm_run<Fp>(plan, nullptr, ws, wsb, d_msm, st));
   }
