@@ -10,6 +10,11 @@
 // preallocated arena managed by a first-fit allocator, so serving allocates no device
 // memory per request.  Every device wait is bounded (ZKVC_ETIMEOUT).
 //
+// The footprint counts the MSM runs' smaller workspaces, and a request always fits into it.
+// A request or batch takes their larger form (pairwise affine rounds) only where the rest of
+// the budget still holds a request of the largest key for every idle worker, so a budget of
+// k footprints has k requests in flight.
+//
 // Mode policy: a request admitted onto an otherwise idle GPU uses the fold prover
 // (lowest latency); one admitted beside others uses the chain prover (about 2.5x less
 // MSM work), which raises throughput when proofs share the GPU.  Both give the same bytes.
@@ -93,6 +98,13 @@ class ArenaAlloc {
     return m;
   }
   size_t cap() const { return cap_; }
+  // whether n blocks of these bytes fit at once
+  bool holds(size_t bytes, int n) const {
+    bytes = std::max<size_t>((bytes + 255) & ~size_t(255), 256);
+    size_t k = 0;
+    for (const auto& kv : free_) k += kv.second / bytes;
+    return k >= size_t(n);
+  }
 
  private:
   std::map<size_t, size_t> free_;
@@ -133,6 +145,7 @@ struct zkvc_server {
   std::unordered_map<uint64_t, std::unique_ptr<Request>> reqs;
   uint64_t next_id = 1;
   int in_flight = 0;
+  int slots = 0, busy = 0;  // workers, and those with a request or a batch
   uint64_t completed = 0, chain_count = 0, merged_count = 0, batch_count = 0;
   int merge_max = 64;
   std::vector<size_t> fp_batch;  // device bytes of a one-request batch per key (merge policy)
@@ -141,17 +154,29 @@ struct zkvc_server {
   std::string fatal;  // set if a worker could not start
   std::vector<size_t> fp_fold, fp_chain;  // least request footprint per key and mode
   std::vector<size_t> fp_fold_full, fp_chain_full;
+  size_t fp_most = 0;  // largest least footprint of a request beside others
   ~zkvc_server();
 };
 
 namespace zkvc {
 
-// Device bytes of one request: the least it runs in (lean: admission counts on this), or
-// with room for the affine rounds of large MSM runs, taken when it is free.
+// Device bytes of one request: the least it runs in (lean: admission counts on this; with
+// chunks of a few terms the form with rounds is the smaller one), or the MSM runs' full form.
 static size_t footprint(const zkvc_pk* pk, int mode, bool lean) {
   const Shape& sh = pk->shape;
-  return prove_workspace_bytes(pk, mode, lean) + round256(size_t(sh.a) * sh.n) + round256(size_t(sh.n) * sh.b) +
-         round256(size_t(sh.a) * sh.b * 4);
+  size_t ws = prove_workspace_bytes(pk, mode, false);
+  if (lean) ws = std::min(ws, prove_workspace_bytes(pk, mode, true));
+  return ws + round256(size_t(sh.a) * sh.n) + round256(size_t(sh.n) * sh.b) + round256(size_t(sh.a) * sh.b * 4);
+}
+
+// Room for an idle worker's request or batch (S->mu held): `full` bytes where what is left
+// then holds a request for each of the other idle workers, else `least`; 0: neither is free.
+static size_t place(zkvc_server* S, size_t full, size_t least, size_t* off) {
+  if (S->alloc.alloc(full, off)) {
+    if (full <= least || S->alloc.holds(S->fp_most, S->slots - S->busy - 1)) return full;
+    S->alloc.release(*off, full);
+  }
+  return S->alloc.alloc(least, off) ? least : 0;
 }
 
 struct WorkerRes {
@@ -196,6 +221,7 @@ static void run_merged(zkvc_server* S, zkvc_batch* MB, std::vector<Request*>& gr
     std::lock_guard<std::mutex> lk(S->mu);
     if (rc != ZKVC_ETIMEOUT) S->alloc.release(off, bytes);
     S->in_flight -= m;
+    S->busy--;
     S->completed += m;
     const auto t_done = Clock::now();
     for (int i = 0; i < m; i++) {
@@ -271,16 +297,11 @@ static void worker_main(zkvc_server* S) {
             est += f;
             kp.push_back(S->pks[h->key]);
           }
-          fp = 0;
-          while (kp.size() >= 2 && fp == 0) {
-            for (const bool lean : {false, true}) {
-              const size_t exact = batch_serve_bytes(kp.data(), (int)kp.size(), lean);
-              if (S->alloc.alloc(exact, &off)) {
-                fp = exact;
-                break;
-              }
-            }
-            if (fp == 0) kp.pop_back();
+          while (kp.size() >= 2) {
+            const int m = (int)kp.size();
+            fp = place(S, batch_serve_bytes(kp.data(), m, false), batch_serve_bytes(kp.data(), m, true), &off);
+            if (fp) break;
+            kp.pop_back();
           }
           if (kp.size() >= 2) {
             for (size_t i = 0; i < kp.size(); i++) {
@@ -288,6 +309,7 @@ static void worker_main(zkvc_server* S) {
               S->queue.pop_front();
             }
             S->in_flight += (int)grp.size();
+            S->busy++;
             S->merged_count += grp.size();
             S->batch_count++;
             S->peak_used = std::max(S->peak_used, S->alloc.used());
@@ -314,14 +336,12 @@ static void worker_main(zkvc_server* S) {
             S->cv_done.notify_all();
             continue;
           }
-          const size_t full = mode == ZKVC_PROVE_CHAIN ? S->fp_chain_full[h->key] : S->fp_fold_full[h->key];
-          bool placed = S->alloc.alloc(full, &off);
-          if (placed) fp = full;
-          else placed = S->alloc.alloc(fp, &off);
-          if (placed) {
+          fp = place(S, mode == ZKVC_PROVE_CHAIN ? S->fp_chain_full[h->key] : S->fp_fold_full[h->key], fp, &off);
+          if (fp) {
             S->queue.pop_front();
             q = h;
             S->in_flight++;
+            S->busy++;
             S->peak_used = std::max(S->peak_used, S->alloc.used());
             if (mode == ZKVC_PROVE_CHAIN) S->chain_count++;
             break;
@@ -376,6 +396,7 @@ static void worker_main(zkvc_server* S) {
       // else returns its slot at once
       if (wrc != ZKVC_ETIMEOUT) S->alloc.release(off, fp);
       S->in_flight--;
+      S->busy--;
       S->completed++;
       q->status = rc;
       q->done = true;
@@ -432,6 +453,7 @@ int zkvc_server_create(const zkvc_pk* const* pks, int npk, int slots, size_t mem
   S->device = dev;
   S->pks.assign(pks, pks + npk);
   S->policy = policy;
+  S->slots = slots;
   if (cudaMalloc(&S->arena, mem_budget) != cudaSuccess) {
     cudaGetLastError();
     S->arena = nullptr;
@@ -444,6 +466,7 @@ int zkvc_server_create(const zkvc_pk* const* pks, int npk, int slots, size_t mem
     S->fp_chain.push_back(footprint(pk, ZKVC_PROVE_CHAIN, true));
     S->fp_fold_full.push_back(footprint(pk, ZKVC_PROVE_FOLD, false));
     S->fp_chain_full.push_back(footprint(pk, ZKVC_PROVE_CHAIN, false));
+    S->fp_most = std::max(S->fp_most, policy == ZKVC_SERVER_FOLD ? S->fp_fold.back() : S->fp_chain.back());
     if (policy == ZKVC_SERVER_MERGE) S->fp_batch.push_back(batch_serve_bytes(&pk, 1, true));
   }
   for (int i = 0; i < slots; i++) S->workers.emplace_back(worker_main, S.get());
