@@ -32,7 +32,6 @@
 #include <cstring>
 #include <map>
 #include <memory>
-#include <mutex>
 #include <vector>
 
 #include "groth16.h"
@@ -78,11 +77,9 @@ __global__ void __launch_bounds__(MM_THREADS) k_b_matmul(const BInst* __restrict
   matmul_tc_tile(in.X, in.W, in.Y, a, in.n, b, blockIdx.x * MM_M, blockIdx.y * MM_N, 0, in.n, false, sm, in.flags);
 }
 
-static std::once_flag g_bmm_once;
-static void b_matmul_init() {
-  std::call_once(g_bmm_once, [] {
-    cudaFuncSetAttribute(k_b_matmul, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MatmulSmem));
-  });
+static int b_matmul_init() {
+  static OncePerDevice once;
+  return smem_limits(once, {{(const void*)k_b_matmul, sizeof(MatmulSmem)}});
 }
 
 __global__ void __launch_bounds__(256) k_b_crpc_ab(const BInst* __restrict__ I) {
@@ -424,7 +421,7 @@ static int enqueue(zkvc_batch* B) {
   k_b_randomness<<<(n + 63) / 64, 64, 0, st>>>(B->dinst, n); ZK_COUNT_LAUNCH();
   ZK_CUDA(cudaGetLastError());
   // witness
-  b_matmul_init();
+  ZK_TRY(b_matmul_init());
   k_b_matmul<<<dim3((maxb + MM_M - 1) / MM_M, (maxa + MM_N - 1) / MM_N, n), MM_THREADS, sizeof(MatmulSmem), st>>>(
       B->dinst);
   ZK_COUNT_LAUNCH();
@@ -624,7 +621,7 @@ static int decode_flags(const int* flags, int n, int* status, int* first_flag) {
 
 static int batch_create(const zkvc_pk* const* pks, int count, int flags, zkvc_batch** out) {
   ZK_CHECK(pks && out, ZKVC_EINVAL, "batch: null argument");
-  b_matmul_init();  // before any capture
+  ZK_TRY(b_matmul_init());  // before any capture
   ZK_CHECK(count >= 1 && count <= 4096, ZKVC_EINVAL, "batch: %d instances outside [1, 4096]", count);
   ZK_CHECK((flags & ~(ZKVC_BATCH_AUTOTUNE | ZKVC_BATCH_EAGER)) == 0, ZKVC_EINVAL, "batch: unknown flags 0x%x", flags);
   int dev = 0;
@@ -730,7 +727,7 @@ static int batch_prove(zkvc_batch* B, const int8_t* const* dX, const int8_t* con
 int batch_serve_open(int cap, zkvc_batch** out) {
   ZK_CHECK(out && cap >= 1 && cap <= 4096, ZKVC_EINVAL, "server batch: capacity %d", cap);
   *out = nullptr;
-  b_matmul_init();
+  ZK_TRY(b_matmul_init());
   ZK_TRY(ntt_init());
   std::unique_ptr<zkvc_batch> B(new zkvc_batch());
   ZK_CUDA(cudaGetDevice(&B->device));

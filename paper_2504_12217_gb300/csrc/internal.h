@@ -6,8 +6,10 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <initializer_list>
 
 #include "../../include/zkvc.h"
+#include "once_per_device.h"
 
 namespace zkvc {
 
@@ -86,6 +88,21 @@ bool prof_enabled();
     int rc_ = (expr);            \
     if (rc_ != ZKVC_OK) return rc_; \
   } while (0)
+
+// Raises kernels' limits of dynamic shared memory on the current device.
+struct SmemLimit {
+  const void* kernel;
+  size_t bytes;
+};
+inline int smem_limits(OncePerDevice& once, std::initializer_list<SmemLimit> kernels) {
+  int dev = 0;
+  ZK_CUDA(cudaGetDevice(&dev));
+  return once(dev, [&]() -> int {
+    for (const SmemLimit& k : kernels)
+      ZK_CUDA(cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.bytes));
+    return ZKVC_OK;
+  });
+}
 
 // Bump allocator over a caller-provided device workspace (256-byte aligned slices).
 // bytes rounded up to a multiple of 256 (the alignment of every device buffer carved here)

@@ -1,7 +1,6 @@
 // One-instance launcher of the tensor-core witness matmul (matmul_tc.cuh).
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "internal.h"
 #include "matmul_tc.cuh"
@@ -18,17 +17,13 @@ __global__ void __launch_bounds__(MM_THREADS) k_matmul_tc(const int8_t* __restri
                  first_wait_ns);
 }
 
-static std::once_flag g_mm_once;
 static std::atomic<uint64_t> g_first_wait_ns{MATMUL_WAIT_NS};
 
 void set_matmul_first_wait_ns(uint64_t ns) { g_first_wait_ns.store(ns, std::memory_order_relaxed); }
 
 int matmul_init() {
-  std::call_once(g_mm_once, [] {
-    cudaFuncSetAttribute(k_matmul_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MatmulSmem));
-  });
-  ZK_CUDA(cudaGetLastError());
-  return ZKVC_OK;
+  static OncePerDevice once;
+  return smem_limits(once, {{(const void*)k_matmul_tc, sizeof(MatmulSmem)}});
 }
 
 // K is split over CTAs (exact int32 atomics into a zeroed Y) while the output grid is

@@ -29,7 +29,6 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 #include "coop.cuh"
@@ -949,11 +948,11 @@ static uint64_t tree_level_blocks(uint64_t len, uint32_t rounds) {
 
 // shared memory of k_tree_down: two stages of two points and a prefix product per thread
 template <class F>
-static size_t tree_down_smem() {
-  static std::once_flag once;
-  constexpr size_t bytes = 2 * (2 * sizeof(Affine<F>) + sizeof(F)) * TREE_BT;
-  std::call_once(once, [] { cudaFuncSetAttribute(k_tree_down<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
-  return bytes;
+constexpr size_t TREE_DOWN_SMEM = 2 * (2 * sizeof(Affine<F>) + sizeof(F)) * TREE_BT;
+template <class F>
+static int tree_init() {
+  static OncePerDevice once;
+  return smem_limits(once, {{(const void*)k_tree_down<F>, TREE_DOWN_SMEM<F>}});
 }
 
 // slabs of equal length (a multiple of 2^rounds) for `terms` terms
@@ -1740,6 +1739,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
   if (accum_stage >= 0) prof_mark(accum_stage, true, st);
   const auto* ob = reinterpret_cast<const Affine<F>* const*>(L.obases);
   if (R) {
+    ZK_TRY(tree_init<F>());
     Affine<F>* const pts = reinterpret_cast<Affine<F>*>(L.tree_out);
     TreeRound<F> a{L.sorted, L.offs, K, (uint32_t)p.outs.size(), bases, ob, p.key_shift, 0, 0, 0, L.tree_slab,
                    nullptr, nullptr, reinterpret_cast<F*>(L.tree_levels)};
@@ -1752,7 +1752,7 @@ int msm_launch(const MsmExec* ex, const Affine<F>* bases, XYZZ<F>* results, cuda
         const unsigned blocks = (unsigned)((pairs + TREE_BT * a.per - 1) / (TREE_BT * a.per));
         k_tree_up<F><<<blocks, TREE_BT, 0, st>>>(a); ZK_COUNT_LAUNCH();
         k_tree_inv<F><<<(blocks * TREE_W + 63) / 64, 64, 0, st>>>(a); ZK_COUNT_LAUNCH();
-        k_tree_down<F><<<blocks, TREE_BT, tree_down_smem<F>(), st>>>(a); ZK_COUNT_LAUNCH();
+        k_tree_down<F><<<blocks, TREE_BT, TREE_DOWN_SMEM<F>, st>>>(a); ZK_COUNT_LAUNCH();
       }
     }
     if (lanes == 4)

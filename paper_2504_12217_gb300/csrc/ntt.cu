@@ -532,27 +532,19 @@ __global__ void __launch_bounds__(R4 ? 768 : 512, R4 ? 1 : 2)
   pass_store<false>(ev + (size_t(3) * m + i) * N, gdif, gid0, sm, SC_NONE, false, tabs);
 }
 
-static std::once_flag g_smem_once;
-
-static void ntt_smem_attrs() {
-  std::call_once(g_smem_once, [] {
-    cudaFuncSetAttribute(k_ntt_pass<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_pass<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_turn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_turn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 << 10);
-    cudaFuncSetAttribute(k_ntt_quotient_turn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 << 10);
-    cudaFuncSetAttribute(k_ntt_quotient_turn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 << 10);
-  });
-}
-
 int ntt_init() {
-  ntt_smem_attrs();
-  ZK_CUDA(cudaGetLastError());
-  return ZKVC_OK;
+  static OncePerDevice once;
+  constexpr size_t one = 64 << 10, three = 192 << 10;
+  return smem_limits(once, {{(const void*)k_ntt_pass<true, false, false>, one},
+                            {(const void*)k_ntt_pass<true, true, false>, one},
+                            {(const void*)k_ntt_pass<false, false, false>, one},
+                            {(const void*)k_ntt_pass<false, true, false>, one},
+                            {(const void*)k_ntt_pass<false, false, true>, one},
+                            {(const void*)k_ntt_pass<false, true, true>, one},
+                            {(const void*)k_ntt_turn<false>, one},
+                            {(const void*)k_ntt_turn<true>, one},
+                            {(const void*)k_ntt_quotient_turn<false>, three},
+                            {(const void*)k_ntt_quotient_turn<true>, three}});
 }
 
 // Stage split of an N = 2^L transform into passes of at most min(elog, 10) stages, the
@@ -605,7 +597,7 @@ static int run_passes(bool dit, Fr* data, int batch, size_t bstride, const NttDo
                       int load_scale, int store_scale, bool raw, int elog, cudaStream_t st) {
   ZK_CHECK(elog >= 8 && elog <= 11, ZKVC_EINVAL, "ntt: 2^%d elements per block outside [2^8, 2^11]", elog);
   ZK_CHECK(batch >= 1 && batch <= 65535, ZKVC_EINVAL, "ntt: batch of %d arrays", batch);
-  ntt_smem_attrs();
+  ZK_TRY(ntt_init());
   const std::vector<uint32_t> ks = pass_split(d->logN, elog);
   const uint32_t P = (uint32_t)ks.size();
   uint32_t s0 = 0;
@@ -622,7 +614,7 @@ int ntt_quotient_chain(Fr* ev, int m, size_t N, const NttDomain* d, cudaStream_t
   ZK_CHECK(elog >= 8 && elog <= 11, ZKVC_EINVAL, "ntt: 2^%d elements per block outside [2^8, 2^11]", elog);
   ZK_CHECK(m >= 1 && 3 * m <= 65535, ZKVC_EINVAL, "ntt: %d instances", m);
   ZK_CHECK(N == d->N, ZKVC_EINVAL, "ntt: array stride %zu is not N", N);
-  ntt_smem_attrs();
+  ZK_TRY(ntt_init());
   const uint32_t L = d->logN;
   const std::vector<uint32_t> ks = pass_split(L, elog);
   const uint32_t P = (uint32_t)ks.size();

@@ -29,8 +29,8 @@ enum ScaleMode : int {
   SC_N = 4,     // x N^-1
 };
 
-// Sets the pass kernels' shared-memory limit (64 KB blocks); call once before capturing
-// NTT launches in a graph (the first NTT call does it otherwise).
+// Sets the pass kernels' shared-memory limits on the current device; the NTT calls do it
+// themselves.
 int ntt_init();
 
 // Cached per (device, logN); built on first use (allocates; do not call under capture).
