@@ -110,8 +110,8 @@ int zkvc_fp2_mul(const uint8_t* d_a, const uint8_t* d_b, uint8_t* d_out, size_t 
 /* Elementwise inverses d_out[i] = d_a[i]^-1 mod r (fr) or mod p (fp), 0 -> 0, for n
  * canonical 32-byte little-endian elements in device memory; d_out may alias d_a.  The
  * inversion of the prover's affine conversions (the Groth16 proof encodes A, B and C in
- * affine coordinates, Sec. II): a binary GCD that takes 30 steps at a time on 62-bit
- * stand-ins of the operands (17 rounds).  Returns ZKVC_EINVAL on a null pointer with n > 0.
+ * affine coordinates, Sec. II): binary division, 30 halvings at a time on the operands' low
+ * words (at most 28 rounds).  Returns ZKVC_EINVAL on a null pointer with n > 0.
  */
 int zkvc_fr_inv(const uint8_t* d_a, uint8_t* d_out, size_t n, void* stream);
 int zkvc_fp_inv(const uint8_t* d_a, uint8_t* d_out, size_t n, void* stream);

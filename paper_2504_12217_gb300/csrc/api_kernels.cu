@@ -139,7 +139,7 @@ __global__ void k_field_mul(const Field<C>* a, const Field<C>* b, Field<C>* out,
   st_field(out + i, f_mul(f_to_mont(ld_field(a + i)), ld_field(b + i)));
 }
 
-// a^-1 (0 -> 0): Montgomery form in, inversion (binary GCD), canonical out
+// a^-1 (0 -> 0): Montgomery form in, inversion, canonical out
 template <class C>
 __global__ void k_field_inv(const Field<C>* a, Field<C>* out, size_t n) {
   size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;

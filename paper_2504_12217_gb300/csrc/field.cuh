@@ -74,6 +74,7 @@ struct FpCfg {
   static constexpr U256c MOD2 = cx_twice(MOD);
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
+  static constexpr U256c R3 = cx_pow2_mod(768, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
 };
 
@@ -83,6 +84,7 @@ struct FrCfg {
   static constexpr U256c MOD2 = cx_twice(MOD);
   static constexpr U256c R1 = cx_pow2_mod(256, MOD);
   static constexpr U256c R2 = cx_pow2_mod(512, MOD);
+  static constexpr U256c R3 = cx_pow2_mod(768, MOD);
   static constexpr uint32_t INV = cx_neg_inv32(MOD.w[0]);
 };
 
@@ -106,6 +108,8 @@ template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t r1_limb(int i) { ZKVC_LIMB_SWITCH(C::R1, i) }
 template <class C>
 __host__ __device__ __forceinline__ constexpr uint32_t r2_limb(int i) { ZKVC_LIMB_SWITCH(C::R2, i) }
+template <class C>
+__host__ __device__ __forceinline__ constexpr uint32_t r3_limb(int i) { ZKVC_LIMB_SWITCH(C::R3, i) }
 
 // ------------------------------------------------------------------ carry-chain rows
 // t[0..8] += a[0..7] * b : low halves into t[0..7] (carry into t[8]), then high halves
@@ -926,212 +930,159 @@ __device__ __forceinline__ Field<C> f_pow(const Field<C>& a, const uint32_t (&e)
 
 // Inverse of a Montgomery-form element (a R -> a^-1 R); 0 maps to 0.  Not constant-time.
 //
-// Divsteps (Bernstein and Yang, "Fast constant-time gcd computation and modular inversion",
-// 2019) on (f, g) = (N, a R): f odd, a step halves g, or g + f, or swaps the two first.  30
-// steps at a time run on the low 32 bits alone, since their decisions need no magnitudes,
-// and are recorded as a matrix of 31-bit integers with
-//   2^30 (f, g)' = [[u, v], [q, r]] (f, g);
-// the same matrix then updates (f, g) exactly and (d, e) modulo N, where d = f / (a R) and
-// e = g / (a R) up to the factor R^2 that e starts with, so that d ends as +-a^-1 R with
-// f = +-1 and no closing product.  The steps inside a batch run as many at once as the
-// trailing zeros and the step counter allow (up to six), so a batch is about eight rounds of
-// short dependent integer operations.  Numbers are signed 30-bit limbs: a division by 2^30
-// drops a limb, and no magnitude comparison or carry chain is left.  At most
-// (49 * 254 + 57) / 17 = 735 steps reach g = 0 for values below 2^254: 25 batches (18 on
-// average).
+// Binary division (Stehle and Zimmermann, "A binary recursive gcd algorithm", 2004) on
+// (f, g) = (N, a R), f odd: halve g until it is odd, counting the halvings j past those the
+// division before has brought for free; then (f, g) <- (g, f + q g) with the odd q of least
+// magnitude that makes the sum divisible by 2^(j + 1) (|q| < 2^j).  All of it is decided by
+// low bits, so 30 halvings at a time run on the low words alone and give a matrix
+//   2^30 (f, g)' = [[fa, fb], [ga, gb]] (f, g),  row sums of magnitudes at most 2^30
+// (as in the jumps of Bernstein and Yang, "Fast constant-time gcd computation and modular
+// inversion", 2019), which then updates the whole numbers.  f and g stay in [-N, N] and end
+// as +-1 and 0; d and e stay in [0, 3N/2] with d a R = f c and e a R = g c modulo N for one
+// c, which a batch divides by 4: the pair is multiplied by the matrix and divided by 2^32, a
+// limb, as one row of a Montgomery product does it, where f and g are divided by 2^30.
+// Remainders grow by (1 + sqrt 17) / 4 per division at the most, so 2 * 254 /
+// (2 - log2((1 + sqrt 17) / 2)) = 790 halvings reach |g| = 1 (about 540 on average) and one
+// more division 0: 28 batches, 18 on average.
 //
-// What bounds it: the latency of one thread, half in the rounds and half in the updates'
-// wide products.  Measured: one thread 31 k cycles, a warp of 32 inversions 40 k, against
-// 53 k for the binary GCD with magnitude stand-ins before.  (The rounds with selects in
-// place of the branches take 39 k and 54 k.)
-struct S30 {
-  int32_t v[9];
+// What bounds it: the latency of one thread, in equal parts in the divisions and in the
+// updates' wide products, and the first fetch of its code: a proof runs it a few times, each
+// in another kernel.  So the two rows' updates are a loop.  Measured: one thread 32.2 k cycles,
+// a warp of 32 inversions 42.0 k, 1.83 G inversions/s on the whole GPU, the chain-mode proof of
+// [49,320]x[320,512] 700 us; with the rows written out 30.0 k, 39.8 k, 1.99 G and 707 us
+// (divsteps on signed limbs, the form before: 30.5 k, 39.4 k, 1.70 G and 700 us).
+namespace inv {
+constexpr int BATCH = 30;         // halvings per matrix
+constexpr int QUOTIENT_BITS = 5;  // bits of a quotient found at once
+
+struct Rows {
+  int32_t fa, fb, ga, gb;
 };
 
-namespace inv30 {
-constexpr uint32_t M30 = 0x3fffffffu;
-
-// limb i of x in base 2^30
-__host__ __device__ constexpr int32_t limb30(const U256c& x, int i) {
-  const int bit = 30 * i, w = bit / 32, sh = bit % 32;
-  const uint64_t lo = x.w[w], hi = w + 1 < 8 ? x.w[w + 1] : 0u;
-  return (int32_t)(((lo | (hi << 32)) >> sh) & M30);
-}
-template <class C>
-__host__ __device__ constexpr int32_t mod30(int i) {
-  switch (i) {
-    case 0: return limb30(C::MOD, 0);
-    case 1: return limb30(C::MOD, 1);
-    case 2: return limb30(C::MOD, 2);
-    case 3: return limb30(C::MOD, 3);
-    case 4: return limb30(C::MOD, 4);
-    case 5: return limb30(C::MOD, 5);
-    case 6: return limb30(C::MOD, 6);
-    case 7: return limb30(C::MOD, 7);
-    default: return limb30(C::MOD, 8);
-  }
-}
-template <class C>
-__host__ __device__ constexpr int32_t rr30(int i) {
-  switch (i) {
-    case 0: return limb30(C::R2, 0);
-    case 1: return limb30(C::R2, 1);
-    case 2: return limb30(C::R2, 2);
-    case 3: return limb30(C::R2, 3);
-    case 4: return limb30(C::R2, 4);
-    case 5: return limb30(C::R2, 5);
-    case 6: return limb30(C::R2, 6);
-    case 7: return limb30(C::R2, 7);
-    default: return limb30(C::R2, 8);
-  }
-}
-
-struct Mat {
-  int32_t u, v, q, r;
-};
-
-// 30 divsteps from the low 32 bits of f (odd) and g; eta = -delta
-__device__ __forceinline__ int divsteps30(int eta, uint32_t f, uint32_t g, Mat* t) {
-  uint32_t u = 1, v = 0, q = 0, r = 1;
-  int i = 30;
+// A batch on the low words of f and g.  due: halvings since the last division less its j, so
+// the next division's j once positive; returned for the next batch.
+__device__ __forceinline__ int batch(int due, uint32_t f, uint32_t g, Rows& m) {
+  int32_t fa = 1, fb = 0, ga = 0, gb = 1;
+  uint32_t left = BATCH;
   for (;;) {
-    const int z = __clz((int)__brev(g | (0xffffffffu << i)));  // even steps: halvings
+    const uint32_t z = min((uint32_t)__ffs((int)g) - 1u, left);  // g = 0: what is left
     g >>= z;
-    u <<= z;
-    v <<= z;
-    eta -= z;
-    i -= z;
-    if (i == 0) break;
-    if (eta < 0) {  // g odd and delta > 0: (f, g) <- (g, -f)
-      eta = -eta;
-      uint32_t x = f;
+    fa <<= z;
+    fb <<= z;
+    left -= z;
+    due += (int)z;
+    if (left == 0) break;
+    if (due > 0) {  // g takes f's place
+      const uint32_t t = f;
       f = g;
-      g = 0u - x;
-      x = u;
-      u = q;
-      q = 0u - x;
-      x = v;
-      v = r;
-      r = 0u - x;
+      g = t;
+      const int32_t ta = fa, tb = fb;
+      fa = ga;
+      fb = gb;
+      ga = ta;
+      gb = tb;
+      due = -due;
     }
-    // the next min(eta + 1, i) steps keep f: add the multiple of f that clears as many of
-    // g's low bits (at most six: f (f^2 - 2) = -1 / f mod 2^6)
-    const uint32_t w = (f * g * (f * f - 2u)) & ~(0xffffffffu << min(min(eta + 1, i), 6));
-    g += f * w;
-    q += u * w;
-    r += v * w;
+    // g + w f clears bits of g: w = -g / f modulo 2^bits, of least magnitude where these
+    // complete the quotient ((3 f) xor 2 is 1 / f modulo 32)
+    const uint32_t want = (uint32_t)(1 - due), bits = min(min(want, left), (uint32_t)QUOTIENT_BITS);
+    const uint32_t w0 = (0u - g * ((3u * f) ^ 2u)) << (32u - bits);
+    const int32_t w = bits == want ? (int32_t)w0 >> (32u - bits) : (int32_t)(w0 >> (32u - bits));
+    g += f * (uint32_t)w;
+    ga += fa * w;
+    gb += fb * w;
   }
-  t->u = (int32_t)u;
-  t->v = (int32_t)v;
-  t->q = (int32_t)q;
-  t->r = (int32_t)r;
-  return eta;
+  // either row may change its sign, and with it that of f and d or of g and e
+  m = {abs(fa), fa < 0 ? -fb : fb, abs(ga), ga < 0 ? -gb : gb};
+  return due;
 }
 
-// (f, g) <- t (f, g) / 2^30, exact
-__device__ __forceinline__ void update_fg(S30& f, S30& g, const Mat& t) {
-  int64_t cf = (int64_t)t.u * f.v[0] + (int64_t)t.v * g.v[0];
-  int64_t cg = (int64_t)t.q * f.v[0] + (int64_t)t.r * g.v[0];
-  cf >>= 30;
-  cg >>= 30;
+// r = (a x + b y) / 2^30 (exact), x and y in two's complement, a >= 0: a and |b| times x and
+// y or its complement, and what the complement and the unsigned reading of a negative number
+// leave out: 1 for the one, 2^256 for the other
+__device__ __forceinline__ void combine(uint32_t (&r)[8], const uint32_t (&x)[8], uint32_t a, const uint32_t (&y)[8],
+                                        int32_t b) {
+  const uint32_t s = (uint32_t)(b >> 31), m = ((uint32_t)b ^ s) - s;
+  uint64_t e[4], o[4];
 #pragma unroll
-  for (int i = 1; i < 9; i++) {
-    const int32_t fi = f.v[i], gi = g.v[i];
-    cf += (int64_t)t.u * fi + (int64_t)t.v * gi;
-    cg += (int64_t)t.q * fi + (int64_t)t.r * gi;
-    f.v[i - 1] = (int32_t)((uint32_t)cf & M30);
-    g.v[i - 1] = (int32_t)((uint32_t)cg & M30);
-    cf >>= 30;
-    cg >>= 30;
+  for (int j = 0; j < 4; j++) {  // a + |b| <= 2^30: each below 2^62
+    e[j] = (uint64_t)x[2 * j] * a + (uint64_t)(y[2 * j] ^ s) * m;
+    o[j] = (uint64_t)x[2 * j + 1] * a + (uint64_t)(y[2 * j + 1] ^ s) * m;
   }
-  f.v[8] = (int32_t)cf;
-  g.v[8] = (int32_t)cg;
+  e[0] += m & s;
+  const uint32_t high = (a & (uint32_t)((int32_t)x[7] >> 31)) + (m & ((uint32_t)((int32_t)y[7] >> 31) ^ s));
+  uint32_t t[9];
+  t[0] = (uint32_t)e[0];
+  asm("add.cc.u32  %0, %8,  %15;\n\taddc.cc.u32 %1, %9,  %16;\n\taddc.cc.u32 %2, %10, %17;\n\t"
+      "addc.cc.u32 %3, %11, %18;\n\taddc.cc.u32 %4, %12, %19;\n\taddc.cc.u32 %5, %13, %20;\n\t"
+      "addc.cc.u32 %6, %14, %21;\n\taddc.u32 %7, %22, %23;"
+      : "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]), "=&r"(t[6]), "=&r"(t[7]), "=&r"(t[8])
+      : "r"((uint32_t)(e[0] >> 32)), "r"((uint32_t)e[1]), "r"((uint32_t)(e[1] >> 32)), "r"((uint32_t)e[2]),
+        "r"((uint32_t)(e[2] >> 32)), "r"((uint32_t)e[3]), "r"((uint32_t)(e[3] >> 32)), "r"((uint32_t)o[0]),
+        "r"((uint32_t)(o[0] >> 32)), "r"((uint32_t)o[1]), "r"((uint32_t)(o[1] >> 32)), "r"((uint32_t)o[2]),
+        "r"((uint32_t)(o[2] >> 32)), "r"((uint32_t)o[3]), "r"((uint32_t)(o[3] >> 32)), "r"(0u - high));
+#pragma unroll
+  for (int i = 0; i < 8; i++) r[i] = __funnelshift_r(t[i], t[i + 1], BATCH);
 }
 
-// (d, e) <- t (d, e) / 2^30 mod N; d and e stay in (-2N, N)
+// (a x + b y) / 2^32 modulo N, ny = 2N - y: for x and y up to 3N / 2 below 2N 2^30 / 2^32 + N
 template <class C>
-__device__ __forceinline__ void update_de(S30& d, S30& e, const Mat& t) {
-  constexpr uint32_t ninv = (0u - C::INV) & M30;  // N^-1 mod 2^30
-  const int32_t sd = d.v[8] >> 31, se = e.v[8] >> 31;
-  // multiples of N: one for each negative operand, then what makes the sum divisible
-  int32_t md = (t.u & sd) + (t.v & se), me = (t.q & sd) + (t.r & se);
-  int64_t cd = (int64_t)t.u * d.v[0] + (int64_t)t.v * e.v[0];
-  int64_t ce = (int64_t)t.q * d.v[0] + (int64_t)t.r * e.v[0];
-  md -= (int32_t)((ninv * (uint32_t)cd + (uint32_t)md) & M30);
-  me -= (int32_t)((ninv * (uint32_t)ce + (uint32_t)me) & M30);
-  cd += (int64_t)mod30<C>(0) * md;
-  ce += (int64_t)mod30<C>(0) * me;
-  cd >>= 30;
-  ce >>= 30;
+__device__ __forceinline__ Field<C> combine_mod(const Field<C>& x, uint32_t a, const Field<C>& y, const Field<C>& ny,
+                                                int32_t b) {
+  const uint32_t m = (uint32_t)abs(b);
+  uint32_t e[8], o[8];
 #pragma unroll
-  for (int i = 1; i < 9; i++) {
-    const int32_t di = d.v[i], ei = e.v[i];
-    cd += (int64_t)t.u * di + (int64_t)t.v * ei + (int64_t)mod30<C>(i) * md;
-    ce += (int64_t)t.q * di + (int64_t)t.r * ei + (int64_t)mod30<C>(i) * me;
-    d.v[i - 1] = (int32_t)((uint32_t)cd & M30);
-    e.v[i - 1] = (int32_t)((uint32_t)ce & M30);
-    cd >>= 30;
-    ce >>= 30;
+  for (int j = 0; j < 8; j++) {
+    const uint64_t p = (uint64_t)x.v[j] * a + (uint64_t)(b < 0 ? ny.v[j] : y.v[j]) * m;
+    (j & 1 ? o : e)[j & ~1] = (uint32_t)p;
+    (j & 1 ? o : e)[j | 1] = (uint32_t)(p >> 32);
   }
-  d.v[8] = (int32_t)cd;
-  e.v[8] = (int32_t)ce;
+  eo::red_row<C>(e, o);
+  Field<C> r;
+  asm("add.cc.u32  %0, %8,  %15;\n\taddc.cc.u32 %1, %9,  %16;\n\taddc.cc.u32 %2, %10, %17;\n\t"
+      "addc.cc.u32 %3, %11, %18;\n\taddc.cc.u32 %4, %12, %19;\n\taddc.cc.u32 %5, %13, %20;\n\t"
+      "addc.cc.u32 %6, %14, %21;\n\taddc.u32 %7, %22, 0;"
+      : "=&r"(r.v[0]), "=&r"(r.v[1]), "=&r"(r.v[2]), "=&r"(r.v[3]), "=&r"(r.v[4]), "=&r"(r.v[5]), "=&r"(r.v[6]),
+        "=&r"(r.v[7])
+      : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+        "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]));
+  return r;
 }
-
-// x in (-2N, N), negated if neg, brought to [0, N): limbs carry signed values until the end
-template <class C>
-__device__ __forceinline__ void normalize(S30& x, bool neg) {
-#pragma unroll
-  for (int k = 0; k < 2; k++) {
-    const int32_t add = x.v[8] >> 31;  // negative: add N (to (-N, N), then to [0, N))
-#pragma unroll
-    for (int i = 0; i < 9; i++) x.v[i] += mod30<C>(i) & add;
-    if (k == 0 && neg) {
-#pragma unroll
-      for (int i = 0; i < 9; i++) x.v[i] = -x.v[i];
-    }
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-      x.v[i + 1] += x.v[i] >> 30;
-      x.v[i] &= (int32_t)M30;
-    }
-  }
-}
-}  // namespace inv30
+}  // namespace inv
 
 template <class C>
 __device__ __noinline__ Field<C> f_inv(const Field<C>& a) {
   if (a.is_zero()) return Field<C>::zero();
-  S30 d, e, f, g;
+  Field<C> f = Field<C>::modulus(), g = a, d = Field<C>::zero(), e;
 #pragma unroll
-  for (int i = 0; i < 9; i++) {
-    const int bit = 30 * i, w = bit / 32, sh = bit % 32;
-    const uint32_t lo = a.v[w], hi = w + 1 < 8 ? a.v[w + 1] : 0u;
-    g.v[i] = (int32_t)(__funnelshift_r(lo, hi, sh) & inv30::M30);
-    f.v[i] = inv30::mod30<C>(i);
-    d.v[i] = 0;
-    e.v[i] = inv30::rr30<C>(i);
-  }
-  int eta = -1;
-  for (int batch = 0; batch < 25; batch++) {
-    inv30::Mat t;
-    // the low 32 bits: 30 of limb 0 and two of limb 1
-    eta = inv30::divsteps30(eta, (uint32_t)f.v[0] | ((uint32_t)f.v[1] << 30),
-                            (uint32_t)g.v[0] | ((uint32_t)g.v[1] << 30), &t);
-    inv30::update_de<C>(d, e, t);
-    inv30::update_fg(f, g, t);
-    int32_t z = 0;
+  for (int i = 0; i < 8; i++) e.v[i] = r3_limb<C>(i);
+  int due = 0, n = 1;
+  for (; n < 31; n++) {
+    inv::Rows m;
+    due = inv::batch(due, f.v[0], g.v[0], m);
+    Field<C> m2, ne;
 #pragma unroll
-    for (int i = 0; i < 9; i++) z |= g.v[i];
-    if (z == 0) break;
+    for (int i = 0; i < 8; i++) m2.v[i] = mod2_limb<C>(i);
+    sub8(ne.v, m2.v, e.v);
+    const Field<C> f0 = f, g0 = g, d0 = d, e0 = e;
+#pragma unroll 1
+    for (int row = 0; row < 2; row++) {  // f's row, then g's
+      f = g;
+      d = e;
+      inv::combine(g.v, f0.v, (uint32_t)m.fa, g0.v, m.fb);
+      e = inv::combine_mod(d0, (uint32_t)m.fa, e0, ne, m.fb);
+      m.fa = m.ga;
+      m.fb = m.gb;
+    }
+    if (g.is_zero()) break;
   }
-  inv30::normalize<C>(d, f.v[8] < 0);
-  Field<C> r;
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    const int bit = 32 * i, l = bit / 30, sh = bit % 30;  // bits [32 i, 32 i + 32) span limbs l, l + 1
-    r.v[i] = ((uint32_t)d.v[l] >> sh) | ((uint32_t)d.v[l + 1] << (30 - sh));
-  }
-  return r;
+  // d = +-(R^3 / 4^n) / (a R): times 4^n / R
+  const uint64_t c = uint64_t(1) << (2 * n);
+  Field<C> back = Field<C>::zero();
+  back.v[0] = (uint32_t)c;
+  back.v[1] = (uint32_t)(c >> 32);
+  const Field<C> r = f_mul(d, back);
+  return f.v[7] >> 31 ? f_neg(r) : r;
 }
 
 using Fp = Field<FpCfg>;
