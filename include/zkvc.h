@@ -347,8 +347,8 @@ int zkvc_prove(const zkvc_pk* pk, const int8_t* d_X, const int8_t* d_W, const ui
  *                     but 16 signed digits per witness entry instead of one.
  *   ZKVC_PROVE_CHAIN  computes A and B1 with small-scalar MSMs and then s A and r B1 as
  *                     two variable-base multiplications beside the H MSM (the scalars
- *                     split by the GLV endomorphism, four 127-bit halves on four lane
- *                     quads): about 2.5x less MSM work per proof, so more proofs per
+ *                     split by the GLV endomorphism, four 127-bit halves on two warps
+ *                     each): about 2.5x less MSM work per proof, so more proofs per
  *                     second when several proofs share the GPU.
  * Workspace sizes differ per mode.  zkvc_prove uses the key's mode (tuning value 6),
  * ZKVC_PROVE_FOLD unless zkvc_pk_autotune or zkvc_pk_set_tuning chose chain, and

@@ -130,14 +130,9 @@ static __device__ __noinline__ G2J p_add_affine_quad_g2(G2J p, G2A q) { return p
 __device__ __forceinline__ G1J p_add_affine_quad(const G1J& p, const G1A& q) { return p_add_affine_quad_g1(p, q); }
 __device__ __forceinline__ G2J p_add_affine_quad(const G2J& p, const G2A& q) { return p_add_affine_quad_g2(p, q); }
 
-static __device__ __noinline__ G1J p_dbl_quad_g1(G1J p) { return p_dbl_quad_body(p); }
-static __device__ __noinline__ G2J p_dbl_quad_g2(G2J p) { return p_dbl_quad_body(p); }
 static __device__ __noinline__ G1J p_add_quad_g1(G1J p, G1J q) { return p_add_quad_body(p, q); }
 static __device__ __noinline__ G2J p_add_quad_g2(G2J p, G2J q) { return p_add_quad_body(p, q); }
 
-__device__ __forceinline__ G1J p_dbl_quad(const G1J& p) { return p_dbl_quad_g1(p); }
-
-__device__ __forceinline__ G2J p_dbl_quad(const G2J& p) { return p_dbl_quad_g2(p); }
 __device__ __forceinline__ G1J p_add_quad(const G1J& p, const G1J& q) { return p_add_quad_g1(p, q); }
 __device__ __forceinline__ G2J p_add_quad(const G2J& p, const G2J& q) { return p_add_quad_g2(p, q); }
 

@@ -274,7 +274,9 @@ __device__ __forceinline__ Field<C> f_mul_cios(const Field<C>& a, const Field<C>
 // multiply-adds each (mad.lo.cc / madc.hi.cc on a register pair) with the carry handed on
 // inside the chain: one multiply-add instruction per term, against one multiply-add and one
 // carry addition in product scanning.  The row-by-row form follows Koc, Acar and Kaliski's
-// operand scanning (1996); the split by parity keeps its carries off the critical pairs.
+// operand scanning (1996); two accumulators for terms that are and are not aligned are known
+// from CUDA multiprecision work (Emmart, Luitjens, Weems and Woolley, "Optimizing modular
+// multiplication for NVIDIA's Maxwell GPUs", 2016).
 //
 // What bounds it: the multiplier's 32 wide multiply-adds per SM and clock; a product has
 // 128 of them and 8 low products, 132 clocks per warp and SM.  Measured on GB300 (2,070

@@ -204,9 +204,9 @@ static uint64_t accum_resident_threads(uint32_t at);
 // average per bucket.  r rounds pad every bucket to a multiple of 2^r terms, 2^(r-1) pads
 // on average, so r keeps them to about a sixteenth; what r rounds leave to the XYZZ
 // additions is 2^-r of the terms.  Measured (G1 MSM, eight windows of 16 bits): 2^18 points
-// = 4.2 M terms 1.54 ms with rounds, 1.59 without, 2^20 3.52 and 4.28, 3,000,001 8.53 and
-// 10.83; below 2^22 terms the rounds' launches and inversions cost what they save (2^17
-// points 1.26 and 1.25, 2^16 points 0.87 and 0.81).  G2 of 2^18 points 4.01 and 4.27.  At
+// = 4.2 M terms 1.50 ms with rounds, 1.56 without, 2^20 3.37 and 4.14, 3,000,001 8.08 and
+// 10.43; below 2^22 terms the rounds' launches and inversions cost what they save (2^17
+// points 1.26 and 1.25, 2^16 points 0.87 and 0.81).  G2 of 2^18 points 3.62 and 3.86.  At
 // 64 terms per bucket a fourth round loses (3.72 against 3.57 ms at 2^20 points).
 static uint32_t tree_rounds(uint64_t slots, uint32_t keys, uint64_t base_end) {
   if (slots < TREE_MIN_TERMS || base_end >= TREE_NONE_BASE) return 0;
@@ -675,9 +675,11 @@ __global__ void __launch_bounds__(256) k_tree_fill(const uint32_t* __restrict__ 
 // prefix product (kept in the sum's own place).
 //
 // What bounds it: k_tree_down by its products (G1: 27 clocks per pair and SM, 20 if the
-// multiplier never idled), k_tree_up of the first round by the gather of single 64-byte
-// points (4.2 TB/s of them).  A block that kept its pairs through all rounds, inverting once
-// per round itself, took 49 clocks per pair: warps idle at the barrier around the inversion.
+// multiplier never idled), k_tree_up of the first round by DRAM, at 6.1 TB/s, though two thirds
+// of what it reads is not used: of 3,000,001 points' first slab 0.94 GB of indices and x
+// coordinates at random places in 2.90 GB read.  A block that kept its pairs through all
+// rounds, inverting once per round itself, took 49 clocks per pair: warps idle at the barrier
+// around the inversion.
 // Measured for 15.4 M additions of a 2^20-point MSM: 1.9 ms against 2.6 for XYZZ.
 constexpr int TREE_BT = 128, TREE_W = 4, TREE_LEVELS = 2 * TREE_BT - TREE_W;
 constexpr uint32_t TREE_PER = 32;                 // pairs per thread at most
@@ -934,8 +936,8 @@ static uint32_t tree_per(uint64_t pairs) {
   return (uint32_t)std::min<uint64_t>(TREE_PER, std::max<uint64_t>(1, pairs / (4 * wave)));
 }
 
-// blocks whose products a slab of `len` terms needs room for: the first round's count bounds
-// the later rounds' as long as each thread takes at least one pair
+// blocks whose products a slab of `len` terms needs room for: the most of any round (a later
+// round has half the pairs, but may give each thread fewer)
 template <class F>
 static uint64_t tree_level_blocks(uint64_t len, uint32_t rounds) {
   uint64_t most = 0;

@@ -199,7 +199,6 @@ static __device__ __noinline__ void f12_pow_u(E12* r, const E12* a, E12* ac) {
 // f <- f^((p^12 - 1)/r) on threads 0 .. 95; s: scratch
 struct alignas(16) FinalScratch {
   E12 t, a, b, c, x, y, z;
-  Fp inv;
 };
 static __device__ __noinline__ void final_exp(E12* f, FinalScratch* s, const FrobTab* T) {
   // f^-1 = conj(f) g^(p^2) g^(p^4) / n, g = f conj(f) in Fp6 and n = g g^(p^2) g^(p^4) in Fp2
